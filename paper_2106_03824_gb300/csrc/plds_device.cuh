@@ -1140,49 +1140,69 @@ __device__ __forceinline__ void enqueue_ins(const GraphCtx &g, const RoundStage 
 // Step A4: insertion rounds (Algorithm 2).
 // ---------------------------------------------------------------------------
 
-// Sort the touched vertices by level (counting sort) into S; levlist gets the
-// distinct levels in increasing order.  Also resets the per-batch inc counters.
+// Sort the touched vertices that violate Invariant 1 by level (counting sort) into
+// S; levlist gets their distinct levels in increasing order.  Also resets the
+// per-batch inc counters.  Only violators are initial candidates: while a vertex
+// stays on its level its up-degree only grows, so one that violates now is tested
+// when its level is reached, and one that does not is marked by the arrival that
+// takes it past the cutoff.  (Listing every touched vertex made nearly every level
+// an initial-candidate level, which ended the runs of pure rounds there.)
 template <class Team>
-__device__ bool ins_sort_candidates(Team &T, const GraphCtx &g, int *sh) {
+__device__ bool ins_sort_candidates(Team &T, const GraphCtx &g, int *sh, const int32_t *sh_upmax) {
     const int32_t tc = g.ctl->tcount;
-    for (int i0 = T.wid() * 32; i0 < tc; i0 += T.nwarps() * 32) {
-        const int i = i0 + lane_id();
-        const int32_t x = i < tc ? g.touched[i] : 0;
-        const int32_t lx = i < tc ? g.level[x] : -1;
-        if (i < tc) g.inc[x] = 0;
+    const int64_t stride = (int64_t)T.nblocks() * blockDim.x;
+    int32_t *cand = g.R[0];
+    for (int64_t b0 = (int64_t)T.bid() * blockDim.x; b0 < tc; b0 += stride) {
+        const int64_t i = b0 + threadIdx.x;
+        bool viol = false;
+        int32_t x = 0, lx = -1;
+        if (i < tc) {
+            x = g.touched[i];
+            g.inc[x] = 0;
+            const int32_t lv = g.level[x];
+            viol = g.up[x] > sh_upmax[lv / g.Lg];
+            if (viol) lx = lv;
+        }
+        if (__syncthreads_or(viol) == 0) continue;
+        const int pos = block_reserve<int32_t>(&g.ctl->ncand, viol ? 1 : 0, sh);
+        if (viol) cand[pos] = x;
         const unsigned peers = __match_any_sync(kFull, lx);  // lanes with the same level add once
-        if (i < tc && lane_id() == __ffs(peers) - 1) atomicAdd(&g.bins[lx], __popc(peers));
+        if (viol && lane_id() == __ffs(peers) - 1) atomicAdd(&g.bins[lx], __popc(peers));
     }
     if (T.leader()) g.ctl->mcnt[0] = 0;
     if (!T.sync()) return false;
-    if (T.bid() == 0) {
-        int run = 0, runl = 0;
-        for (int b0 = 0; b0 < g.K; b0 += blockDim.x) {
-            int l = b0 + threadIdx.x;
-            int c = l < g.K ? g.bins[l] : 0;
-            int tot, totl;
-            int ex = block_exclusive(c, sh, &tot);
-            int exl = block_exclusive(c > 0 ? 1 : 0, sh, &totl);
-            if (l < g.K) {
-                g.bins[l] = run + ex;
-                if (c > 0) g.levlist[runl + exl] = l;
-            }
-            run += tot;
-            runl += totl;
+    const int32_t nc = g.ctl->ncand;
+    if (nc == 0) return true;  // nlev stays 0: no rounds
+    if (T.bid() == 0) {  // each thread scans its own run of levels
+        const int per = (g.K + blockDim.x - 1) / blockDim.x;
+        const int l0 = min(g.K, (int)threadIdx.x * per), l1 = min(g.K, l0 + per);
+        int sum = 0, nz = 0, tot, totl;
+        for (int l = l0; l < l1; ++l) {
+            const int c = g.bins[l];
+            sum += c;
+            nz += c > 0;
         }
-        if (threadIdx.x == 0) g.ctl->nlev = runl;
+        int run = block_exclusive(sum, sh, &tot);
+        int runl = block_exclusive(nz, sh, &totl);
+        for (int l = l0; l < l1; ++l) {
+            const int c = g.bins[l];
+            g.bins[l] = run;
+            run += c;
+            if (c > 0) g.levlist[runl++] = l;
+        }
+        if (threadIdx.x == 0) g.ctl->nlev = totl;
     }
     if (!T.sync()) return false;
-    for (int i0 = T.wid() * 32; i0 < tc; i0 += T.nwarps() * 32) {
+    for (int i0 = T.wid() * 32; i0 < nc; i0 += T.nwarps() * 32) {
         const int i = i0 + lane_id();
-        const int32_t x = i < tc ? g.touched[i] : 0;
-        const int32_t lx = i < tc ? g.level[x] : -1;
+        const int32_t x = i < nc ? cand[i] : 0;
+        const int32_t lx = i < nc ? g.level[x] : -1;
         const unsigned peers = __match_any_sync(kFull, lx);
         const int leader = __ffs(peers) - 1;
         int pos = 0;
-        if (i < tc && lane_id() == leader) pos = atomicAdd(&g.bins[lx], __popc(peers));
+        if (i < nc && lane_id() == leader) pos = atomicAdd(&g.bins[lx], __popc(peers));
         pos = __shfl_sync(kFull, pos, leader) + __popc(peers & ((1u << lane_id()) - 1u));
-        if (i < tc) g.S[pos] = x;
+        if (i < nc) g.S[pos] = x;
     }
     // after the scatter bins[l] is the end of level l's range (= start of l+1)
     return T.sync();
@@ -1206,10 +1226,11 @@ __device__ bool ins_sort_candidates(Team &T, const GraphCtx &g, int *sh) {
 //   - a mover of level l violates again on l + 1 iff its up-degree minus its
 //     neighbours left on l exceeds the cutoff; the scan of its last table chunk
 //     (per-vertex chunk counter) decides, nobody else touching its up-degree.
-// Movers of level l carry the flag of l's parity in their level word from their
-// marking (during round l - 1, where they still read as level l) until the end of
-// round l, whose readers see "mover of l" for a word with that flag and level l or
-// l + 1; the flag of the other parity is ignored.  A level with no movers jumps
+// The movers that phase k scans carry the flag of k's parity in their level word
+// from their marking (during phase k - 1, where they still read as level l) until
+// the end of phase k, whose readers see "mover of l" for a word with that flag and
+// level l or l + 1; the flag of the other parity is ignored (a vertex that stopped
+// keeps its last flag, but its level is below every later phase's).  A level with no movers jumps
 // to the next initial-candidate level, tested in a phase of its own.  Every flag
 // is cleared at the end.  The result is the same as rounds evaluated one level
 // after another (the same-sequence lemma): the marks depend only on final counts.
@@ -1225,10 +1246,10 @@ __device__ bool ins_sort_candidates(Team &T, const GraphCtx &g, int *sh) {
 // rounds at once: the level jumps by j, and rounds, moves and visits are counted
 // as the j rounds would have counted them.  The members' level words still read
 // x+1 (with their flag) until their next scan rewrites them; readers of that scan
-// take a flagged word anywhere from x+1 up as a mover (lmo = x+1), and j is even so
-// that the flag's parity is the one of the new level.
+// take a flagged word anywhere from x+1 up as a mover (lmo = x+1); the flag goes by
+// the phase, not the level, so j may be odd.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int32_t level_flag(int32_t l) { return (l & 1) ? kFlagOdd : kFlagEven; }
+__device__ __forceinline__ int32_t phase_flag(int k) { return (k & 1) ? kFlagOdd : kFlagEven; }
 
 // Effects of a mover of level l on 16 neighbours ws (level words lv), in two
 // passes so that the counter atomics of all 16 are in flight together: first every
@@ -1359,7 +1380,7 @@ __device__ __forceinline__ void marks_add(const GraphCtx &g, const RoundStage &s
 template <class Team>
 __device__ void ins_test_initial(Team &T, const GraphCtx &g, const RoundStage &st, int32_t s_lo, int32_t s_hi,
                                  int32_t L, int32_t cut, int32_t *wsm, int rot, int k1) {
-    const int32_t fl = level_flag(L);
+    const int32_t fl = phase_flag(k1);
     const int rank = (T.srank() + rot) % T.nwarps();
     for (int i0 = s_lo + rank * 32; i0 < s_hi; i0 += T.nwarps() * 32) {
         const int i = i0 + lane_id();
@@ -1450,7 +1471,7 @@ __device__ bool ins_rounds(Team &T, const GraphCtx &g, const int32_t *sh_upmax, 
                 atomicAdd(&g.ctl->st[kStRounds], 1ull);
                 atomicAdd(&g.ctl->st[kStMoves], (unsigned long long)m);
             }
-            const int32_t fcur = level_flag(l), fnext = level_flag(l + 1);
+            const int32_t fcur = phase_flag(k), fnext = phase_flag(k + 1);
             const int32_t cut_next = sh_upmax[(l + 1) / g.Lg];
             if (has_init)  // initial candidates on l + 1
                 ins_test_initial(T, g, st, s_lo, s_hi, l + 1, cut_next, wsm, T.nwarps() / 2, k + 1);
@@ -1700,9 +1721,8 @@ __device__ bool ins_rounds(Team &T, const GraphCtx &g, const int32_t *sh_upmax, 
                 // round l - 1 just ran; rounds l .. l + j - 1 are pure while no other
                 // neighbour sits on l .. l + j + 1, no initial candidate on l + 1 .. l + j
                 // and every member still violates on l + j
-                int64_t j = min(min(low_lvl - l - 2, init_lvl - l - 1), top - l);
-                j &= ~(int64_t)1;  // even: the movers' flag keeps its parity
-                if (j >= 2) {
+                const int64_t j = min(min(low_lvl - l - 2, init_lvl - l - 1), top - l);
+                if (j >= 1) {
                     skip = (int32_t)j;
                     if (T.leader()) {
                         const unsigned long long jm = (unsigned long long)j * (unsigned long long)m;
@@ -1744,6 +1764,7 @@ __device__ bool ins_rounds(Team &T, const GraphCtx &g, const int32_t *sh_upmax, 
         l = g.levlist[spos++];
         scan = false;
     }
+    if (nlev == 0) return true;  // nobody moved: no flag to clear
     // clear the movers' flags (every vertex: flags sit only on vertices that moved)
     for (int64_t v = T.tid(); v < g.n; v += T.nthreads()) {
         const int32_t raw = g.level[v];
@@ -2887,7 +2908,7 @@ __device__ void run_batch(Team &T, const GraphCtx &g, const BatchIn &in, int32_t
             if (!T.sync()) return;
             if (tr) tmark[nmark++] = global_ns();
         }
-        if (!g.jump && !ins_sort_candidates(T, g, sh_scan)) return;
+        if (!g.jump && !ins_sort_candidates(T, g, sh_scan, sh_upmax)) return;
         if (tr) {
             tmark[nmark++] = global_ns();
             trace_steps(g, tmark, nmark, -1);

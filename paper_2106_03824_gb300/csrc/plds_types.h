@@ -7,8 +7,8 @@ namespace pl {
 
 constexpr int32_t kEmpty = -1;          // hash slot never used since the last rebuild
 constexpr int32_t kTomb = -2;           // hash slot of a deleted neighbour
-// Insertion rounds mark the movers of level l in the level word with the flag of
-// l's parity; the level itself is the word & kLevelMask.  Flags never survive a batch.
+// Insertion rounds mark the movers of a phase in the level word with the flag of
+// the phase's parity; the level itself is the word & kLevelMask.  Flags never survive a batch.
 constexpr int32_t kFlagEven = 1 << 30;
 constexpr int32_t kFlagOdd = 1 << 29;
 constexpr int32_t kLevelMask = kFlagOdd - 1;
@@ -79,6 +79,7 @@ struct Ctl {
     int32_t tlcnt[2];     // thread-mode movers
     int32_t clcnt[2];     // chunk items
     int32_t nlev;         // number of distinct initial-candidate levels
+    int32_t ncand;        // initial candidates: touched vertices that violate Invariant 1
     int32_t pcnt[2];      // deletion pending list sizes
     int32_t rcnt[2];      // deletion recompute list sizes
     int32_t nextmin[2];   // deletion: smallest pending desire-level
