@@ -23,6 +23,7 @@
 
 #include "plds.h"
 #include "plds_device.cuh"
+#include "plds_kernels.h"
 #include "plds_tables.h"
 
 using namespace pl;
@@ -1615,47 +1616,6 @@ extern "C" int plds_batch_static(plds_t *h, const int32_t *edges, int64_t B, int
 // per-round launch sequence (descriptor upload, counter reset, kernel, control
 // word read-back) is captured once in a CUDA graph and replayed.
 // ---------------------------------------------------------------------------
-namespace {
-struct SetItem {
-    GraphCtx half[2];  // 0: insertion half, 1: deletion half
-};
-constexpr int kSetThreads = 256;
-constexpr int kSetStageShift = 3;
-}  // namespace
-
-__global__ void __launch_bounds__(kSetThreads, 2)
-    k_batch_set(const SetItem *__restrict__ items, int32_t count, int32_t *next) {
-    extern __shared__ int32_t sh[];
-    __shared__ GraphCtx gsh;
-    __shared__ int32_t idx;
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) idx = atomicAdd(next, 1);
-        __syncthreads();
-        const int i = idx;
-        if (i >= count) return;
-        for (int h = 0; h < 2; ++h) {
-            __syncthreads();
-            const int32_t *src = reinterpret_cast<const int32_t *>(&items[i].half[h]);
-            int32_t *dst = reinterpret_cast<int32_t *>(&gsh);
-            for (int k = threadIdx.x; k < (int)(sizeof(GraphCtx) / 4); k += blockDim.x) dst[k] = src[k];
-            __syncthreads();
-            // the host reads both halves' control blocks: clear them even for an empty half
-            int32_t *cw = reinterpret_cast<int32_t *>(gsh.ctl);
-            for (int k = threadIdx.x; k < (int)(sizeof(Ctl) / 4); k += blockDim.x) cw[k] = 0;
-            if (gsh.B == 0) continue;  // an empty half changes nothing
-            for (int64_t k = threadIdx.x; k < gsh.hcap; k += blockDim.x) gsh.hset[k] = kEmptyKey;
-            if (gsh.op == kOpInsert)
-                for (int k = threadIdx.x; k <= gsh.K; k += blockDim.x) gsh.bins[k] = 0;
-            __syncthreads();
-            BlockTeam T{gsh.ctl};
-            run_batch(T, gsh, BatchIn{gsh.edges, gsh.B, gsh.op, gsh.stamp_base}, sh, kSetStageShift);
-            __syncthreads();
-            if (ld_volatile(&gsh.ctl->err) != 0) break;  // the host resolves it and reruns this graph
-        }
-    }
-}
-
 struct plds_set {
     int32_t count = 0;
     std::vector<plds *> g;       // graph handles
@@ -2159,226 +2119,6 @@ extern "C" void plds_set_destroy(plds_set_t *s) {
 // The loop exits after an idle period or when the adjacency pool needs to grow
 // (the host grows it, gated by free HBM, and relaunches).
 // ---------------------------------------------------------------------------
-namespace {
-enum : int32_t { kSlotFree = 0, kSlotReady = 1, kSlotDone = 2 };
-enum : int32_t { kReqInsert = 0, kReqDelete = 1, kReqCoreness = 2 };
-enum : int32_t { kExitNone = 0, kExitIdle = 1, kExitNeedPool = 2, kExitError = 3 };
-constexpr int kMaxSeg = 64;  // requests merged into one batch at most
-
-struct alignas(64) ReqSlot {
-    int32_t state;  // kSlot*
-    int32_t op;     // kReq*
-    int64_t B;
-    const int32_t *edges;  // device-accessible
-    double *out;           // device-accessible (coreness queries)
-    int64_t ticket;
-    int64_t merge_cap;  // edges one merged batch may hold (0: never merge)
-    // written by the device
-    int32_t status;   // device error bits
-    int32_t batch_n;  // requests in the batch this one was applied in
-    int64_t batch_first;  // ticket of that batch's first request
-    uint64_t t_begin, t_end;  // device globaltimer
-    unsigned long long pool_top;  // adjacency slots handed out after the request
-    unsigned long long st[kStCount];
-    unsigned long long valid;
-};
-
-struct ServeCtl {  // device memory
-    int32_t exit_reason;
-    int32_t cmd;
-    int64_t head;        // next slot sequence number
-    int32_t stamp_next;  // stamps of the next request start here
-    int32_t nseg;        // requests in the current batch (0: a query or an unmerged request)
-    unsigned long long grow_total;
-    int64_t seg_total;   // edges gathered (after rejected requests are dropped)
-    ReqSlot cur;         // the head request (copied from the ring)
-    const int2 *seg_ptr[kMaxSeg];
-    int64_t seg_off[kMaxSeg + 1];
-    int32_t seg_bad[kMaxSeg];
-};
-
-struct ServeArgs {
-    ReqSlot *ring;  // device pointer of the pinned ring
-    int32_t slots;
-    int64_t idle_ns;
-    ServeCtl *sc;
-    const double *powtab;
-    int2 *ebuf;  // gathered edges of a merged batch [max_batch]
-};
-}  // namespace
-
-// Word-by-word copy that reads through volatile loads (the source may be host memory
-// the host is writing, or device memory written by another block).
-__device__ __forceinline__ void copy_slot(ReqSlot *dst, const ReqSlot *src) {
-    const volatile int32_t *sv = reinterpret_cast<const volatile int32_t *>(src);
-    int32_t *dv = reinterpret_cast<int32_t *>(dst);
-    for (int k = 0; k < (int)(sizeof(ReqSlot) / 4); ++k) dv[k] = sv[k];
-}
-
-// Leader: extend the batch that starts with the head request by the waiting
-// requests that follow it (same kind, total edges within the cap).
-__device__ void serve_select(const ServeArgs &a, ServeCtl *sc) {
-    const ReqSlot &c = sc->cur;
-    sc->nseg = 0;
-    if (c.op == kReqCoreness || c.merge_cap <= 0 || c.B > c.merge_cap) return;
-    int64_t total = c.B;
-    sc->seg_ptr[0] = reinterpret_cast<const int2 *>(c.edges);
-    sc->seg_off[0] = 0;
-    sc->seg_bad[0] = 0;
-    int ns = 1;
-    for (int j = 1; j < a.slots && ns < kMaxSeg; ++j) {
-        const ReqSlot *r = a.ring + ((sc->head + j) % a.slots);
-        if (*(volatile const int32_t *)&r->state != kSlotReady) break;
-        __threadfence_system();
-        const int32_t op = *(volatile const int32_t *)&r->op;
-        const int64_t B = *(volatile const int64_t *)&r->B;
-        if (op != c.op || total + B > c.merge_cap) break;
-        sc->seg_ptr[ns] = reinterpret_cast<const int2 *>(*(const int32_t *volatile *)&r->edges);
-        sc->seg_off[ns] = total;
-        sc->seg_bad[ns] = 0;
-        total += B;
-        ++ns;
-    }
-    sc->seg_off[ns] = total;
-    sc->seg_total = total;
-    sc->nseg = ns > 1 ? ns : 0;  // a request alone is read in place
-}
-
-// Grid: copy the batch's requests into one contiguous edge array; with `check`,
-// flag each request holding an id outside [0, n).  Segment offsets are in shared
-// memory (s_off[0..ns]).
-__device__ void serve_gather(GridTeam &T, const ServeCtl *sc, int ns, const int64_t *s_off, int2 *ebuf, int32_t n,
-                             bool check, int32_t *bad) {
-    const int64_t total = s_off[ns];
-    for (int64_t i = T.tid(); i < total; i += T.nthreads()) {
-        int lo = 0, hi = ns - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (s_off[mid] <= i) lo = mid;
-            else hi = mid - 1;
-        }
-        const int2 uv = sc->seg_ptr[lo][i - s_off[lo]];
-        if (check && (uv.x < 0 || uv.x >= n || uv.y < 0 || uv.y >= n)) *(volatile int32_t *)&bad[lo] = 1;
-        ebuf[i] = uv;
-    }
-}
-
-__global__ void __launch_bounds__(512) k_serve(const __grid_constant__ GraphCtx base, const ServeArgs a) {
-    extern __shared__ int32_t sh[];
-    __shared__ int64_t s_off[kMaxSeg + 1];
-    GridTeam T{base.ctl, base.wait_limit_ns, base.barrier_sleep_ns};
-    ServeCtl *sc = a.sc;
-    for (;;) {
-        // the leader waits for the next slot (bounded by the idle limit)
-        if (T.leader()) {
-            ReqSlot *r = a.ring + (sc->head % a.slots);
-            const uint64_t t0 = global_ns();
-            int32_t st;
-            while ((st = *(volatile int32_t *)&r->state) != kSlotReady && global_ns() - t0 < (uint64_t)a.idle_ns)
-                __nanosleep(256);
-            if (st == kSlotReady) {
-                __threadfence_system();
-                copy_slot(&sc->cur, r);
-                serve_select(a, sc);
-                sc->cmd = 1;
-            } else {
-                sc->cmd = 0;
-                sc->exit_reason = kExitIdle;
-            }
-            __threadfence();
-        }
-        if (!T.sync()) return;
-        if (ld_volatile(&sc->cmd) == 0) return;
-        // a fresh control block and key set for this request (the barrier words stay)
-        {
-            int32_t *cw = reinterpret_cast<int32_t *>(base.ctl);
-            const int first = (int)(offsetof(Ctl, err) / 4);
-            for (int k = T.tid() + first; k < (int)(sizeof(Ctl) / 4); k += T.nthreads()) cw[k] = 0;
-            for (int64_t k = T.tid(); k < base.hcap; k += T.nthreads()) base.hset[k] = kEmptyKey;
-            for (int k = T.tid(); k <= base.K; k += T.nthreads()) base.bins[k] = 0;
-            if (sc->stamp_next + 2 * base.K + 8 >= 0x7fffffff) {  // stamps wrap: clear them
-                for (int k = T.tid(); k < base.n; k += T.nthreads()) base.stamp[k] = 0;
-            }
-        }
-        ReqSlot req;
-        copy_slot(&req, &sc->cur);
-        const int ns = ld_volatile(&sc->nseg);
-        if (ns > 0) {  // gather the batch's requests, rejecting those with a bad id
-            for (int k = threadIdx.x; k <= ns; k += blockDim.x) s_off[k] = sc->seg_off[k];
-            __syncthreads();
-            serve_gather(T, sc, ns, s_off, a.ebuf, base.n, true, sc->seg_bad);
-            if (!T.sync()) return;
-            bool anybad = false;
-            for (int k = 0; k < ns; ++k) anybad |= ld_volatile(&sc->seg_bad[k]) != 0;
-            if (anybad) {  // gather again without the rejected requests (they keep length 0)
-                __syncthreads();
-                if (threadIdx.x == 0) {
-                    int64_t t = 0;
-                    for (int k = 0; k < ns; ++k) {
-                        s_off[k] = t;
-                        if (!ld_volatile(&sc->seg_bad[k])) t += sc->seg_off[k + 1] - sc->seg_off[k];
-                    }
-                    s_off[ns] = t;
-                }
-                __syncthreads();
-                if (T.leader()) sc->seg_total = s_off[ns];
-                // a zero-length segment is never selected by the search below (offsets
-                // equal), so the remaining requests' edges land contiguously
-                serve_gather(T, sc, ns, s_off, a.ebuf, base.n, false, sc->seg_bad);
-            }
-        }
-        if (!T.sync()) return;
-        int32_t sbase = sc->stamp_next;
-        if (sbase + 2 * base.K + 8 >= 0x7fffffff) sbase = 1;
-        const uint64_t t_begin = global_ns();
-        if (req.op == kReqCoreness) {
-            for (int64_t v = T.tid(); v < base.n; v += T.nthreads()) {
-                int32_t g = -1;
-                if (base.deg[v] > 0) g = max((base.level[v] + 1) / base.Lg - 1, 0);
-                req.out[v] = g < 0 ? 0.0 : a.powtab[g];
-            }
-        } else {
-            const BatchIn in{ns > 0 ? reinterpret_cast<const int32_t *>(a.ebuf) : req.edges,
-                             ns > 0 ? *(volatile const int64_t *)&sc->seg_total : req.B,
-                             req.op == kReqInsert ? kOpInsert : kOpDelete, sbase};
-            run_batch(T, base, in, sh, 0);
-        }
-        const bool ok = T.sync();
-        if (T.leader()) {
-            const int32_t err = ld_volatile(&base.ctl->err);
-            if (err == kErrNeedPool) {  // leave the slots ready; the host grows the pool and relaunches
-                sc->exit_reason = kExitNeedPool;
-                sc->grow_total = base.ctl->grow_total;
-                sc->stamp_next = sbase + base.K + 2;
-            } else {
-                const int nr = ns > 0 ? ns : 1;
-                const uint64_t t_end = global_ns();
-                const unsigned long long top = *(volatile unsigned long long *)base.pool_top;
-                for (int j = 0; j < nr; ++j) {
-                    ReqSlot *r = a.ring + ((sc->head + j) % a.slots);
-                    r->status = (ns > 0 && ld_volatile(&sc->seg_bad[j])) ? kErrInvalidId : err;
-                    r->batch_n = nr;
-                    r->batch_first = req.ticket;
-                    r->t_begin = t_begin;
-                    r->t_end = t_end;
-                    r->pool_top = top;
-                    for (int k = 0; k < kStCount; ++k) r->st[k] = base.ctl->st[k];
-                    r->valid = base.ctl->vcount;
-                }
-                __threadfence_system();
-                for (int j = 0; j < nr; ++j)
-                    *(volatile int32_t *)&a.ring[(sc->head + j) % a.slots].state = kSlotDone;
-                sc->head += nr;
-                sc->stamp_next = sbase + base.K + 2;
-                if (err) sc->exit_reason = kExitError;
-            }
-            __threadfence();
-        }
-        if (!ok) return;
-        if (!T.sync()) return;
-    }
-}
-
 struct plds_server {
     plds *h = nullptr;
     int32_t slots = 0;

@@ -150,6 +150,12 @@ __device__ __forceinline__ unsigned long long warp_sum64(unsigned long long x) {
     return x;
 }
 
+// The same for one 32-bit value per lane: two 16-bit halves, a hardware reduction each.
+__device__ __forceinline__ unsigned long long warp_total(unsigned x) {
+    const unsigned lo = __reduce_add_sync(kFull, x & 0xffffu), hi = __reduce_add_sync(kFull, x >> 16);
+    return (unsigned long long)lo + ((unsigned long long)hi << 16);
+}
+
 // Position in *counter for each lane with pred, -1 otherwise (one atomic per warp).
 __device__ __forceinline__ int warp_append(int32_t *counter, bool pred) {
     unsigned m = __ballot_sync(kFull, pred);
@@ -309,7 +315,7 @@ __device__ __forceinline__ bool item_ok(const GraphCtx &g, const int4 &it, int l
 // ---------------------------------------------------------------------------
 // Block-level exclusive scan used by the candidate sort (block 0 of the team).
 // ---------------------------------------------------------------------------
-__device__ int block_exclusive(int x, int *sh32, int *total) {
+inline __device__ int block_exclusive(int x, int *sh32, int *total) {
     int lane = lane_id(), w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     int tot;
     int ex = warp_exclusive(x, &tot);
@@ -944,6 +950,7 @@ struct RoundStage {
     int32_t *phs;
     int32_t *ff;             // block's climbing movers: {count, smallest new up-degree, lowest other level}
     unsigned long long *ff64;  // their {degree sum, new up-degree sum}
+    unsigned long long *ltop;  // insertion: int4 units handed out of each up-list buffer [3]
 };
 
 // Shared ints of a staging area whose capacities are the defaults >> shift
@@ -1102,7 +1109,7 @@ __device__ __forceinline__ void enqueue_ins(const GraphCtx &g, const RoundStage 
     int tot4;
     const int ex4 = warp_exclusive(want ? (rsize + 3) >> 2 : 0, &tot4);
     unsigned long long lbase = 0;
-    if (lane == 0 && tot4 > 0) lbase = atomicAdd(&g.ctl->ltop[abuf], (unsigned long long)tot4);
+    if (lane == 0 && tot4 > 0) lbase = atomicAdd(&st.ltop[abuf], (unsigned long long)tot4);
     lbase = __shfl_sync(kFull, lbase, 0);
     if (chunked) {
         const bool fits = want && lbase + (unsigned long long)tot4 <= (unsigned long long)(g.lcap >> 2);
@@ -1110,14 +1117,24 @@ __device__ __forceinline__ void enqueue_ins(const GraphCtx &g, const RoundStage 
         g.lfill[k1 & 1][v] = 0;  // the next phase's counters: last used two phases ago
     }
     const int nch = chunked ? (list ? max(1, (ilen + kChunk - 1) / kChunk) : (c + kChunk - 1) / kChunk) : 0;
-    int tot;
-    const int ex = warp_exclusive(nch, &tot);
+    const unsigned one = __ballot_sync(kFull, nch == 1);
+    int tot, ex;
+    if (!__any_sync(kFull, nch > 1)) {  // at most one item a lane: no need to spread them
+        tot = __popc(one);
+        ex = __popc(one & ((1u << lane) - 1u));
+    } else {
+        ex = warp_exclusive(nch, &tot);
+    }
     if (tot == 0) return;
     int pos = 0;
     bool sh = false;
     if (lane == 0) pos = stage_reserve(st.cl, tot, sh);
     pos = __shfl_sync(kFull, pos, 0);
     sh = __shfl_sync(kFull, sh, 0);
+    if (tot == __popc(one)) {
+        if (nch) stage_put(st.cl, sh, pos + ex, make_int4(v, lg, goff, list ? ilen : 0));
+        return;
+    }
     wsm[lane] = ex;
     wsm[32 + lane] = v;
     wsm[64 + lane] = lg;
@@ -1251,8 +1268,8 @@ __device__ bool ins_sort_candidates(Team &T, const GraphCtx &g, int *sh, const i
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int32_t phase_flag(int k) { return (k & 1) ? kFlagOdd : kFlagEven; }
 
-// Effects of a mover of level l on 16 neighbours ws (level words lv), in two
-// passes so that the counter atomics of all 16 are in flight together: first every
+// Effects of a mover of level l on N neighbours ws (level words lv), in two passes
+// so that the counter atomics of all N are in flight together: first every
 // neighbour is classified and its counter updated -- a neighbour on l + 1 gains an
 // up-neighbour (returning add: the one add that sees the old value equal to the
 // cutoff marks it), one on l + 2 an up*-neighbour -- then the marks are set.
@@ -1262,14 +1279,15 @@ __device__ __forceinline__ int32_t phase_flag(int k) { return (k & 1) ? kFlagOdd
 // changed; cnt4[q / 4] counts the neighbours left on l; low gets the lowest level
 // above l of a neighbour that is no mover.  Movers of l read as flagged words on
 // levels lmo .. l + 1 (lmo = l unless pure rounds were just skipped).
-__device__ __forceinline__ void ins_effects16(const GraphCtx &g, const int32_t (&ws)[16], const int32_t (&lv)[16],
-                                              int32_t l, int32_t lmo, int32_t fcur, int32_t fnext, int32_t cut_next,
-                                              int (&cnt4)[4], int32_t &low, unsigned &push, unsigned &keep,
-                                              unsigned &aff) {
-    int32_t old[16];
+template <int N>
+__device__ __forceinline__ void ins_effects(const GraphCtx &g, const int32_t (&ws)[N], const int32_t (&lv)[N],
+                                            int32_t l, int32_t lmo, int32_t fcur, int32_t fnext, int32_t cut_next,
+                                            int (&cnt4)[N / 4], int32_t &low, unsigned &push, unsigned &keep,
+                                            unsigned &aff) {
+    int32_t old[N];
     unsigned a1m = 0;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
+    for (int q = 0; q < N; ++q) {
         const int32_t w = ws[q], raw = lv[q], f = raw & kLevelMask;
         const bool ok = valid_id(g, w);  // not an empty slot or a tombstone
         const bool mov = ok && (raw & fcur) && f >= lmo && f <= l + 1;  // a mover of level l as well
@@ -1285,8 +1303,9 @@ __device__ __forceinline__ void ins_effects16(const GraphCtx &g, const int32_t (
         keep |= (mov || above) ? 1u << q : 0u;
         aff += (a1 || a2) ? 1u : 0u;
     }
+    if (a1m == 0) return;
 #pragma unroll
-    for (int q = 0; q < 16; ++q)
+    for (int q = 0; q < N; ++q)
         if (((a1m >> q) & 1u) && old[q] == cut_next && !(atomicOr(&g.level[ws[q]], fnext) & fnext)) push |= 1u << q;
 }
 
@@ -1312,8 +1331,8 @@ __device__ __forceinline__ void ff_note(const RoundStage &st, bool again, int32_
     const unsigned m = __ballot_sync(kFull, again);
     if (m == 0) return;
     const int32_t mn = (int32_t)__reduce_min_sync(kFull, again ? (unsigned)nu : (unsigned)kInf);
-    const unsigned long long sd = warp_sum64(again ? (unsigned long long)deg : 0ull);
-    const unsigned long long su = warp_sum64(again ? (unsigned long long)nu : 0ull);
+    const unsigned long long sd = warp_total(again ? (unsigned)deg : 0u);
+    const unsigned long long su = warp_total(again ? (unsigned)nu : 0u);
     if (lane_id() == __ffs(m) - 1) {
         atomicAdd(&st.ff[0], __popc(m));
         atomicMin(&st.ff[1], mn);
@@ -1353,15 +1372,16 @@ __device__ __forceinline__ void marks_flush(const GraphCtx &g, const RoundStage 
 }
 
 // Append the lanes' marked neighbours (bits of push over ws); mc is warp-uniform.
+template <int N>
 __device__ __forceinline__ void marks_add(const GraphCtx &g, const RoundStage &st, unsigned push,
-                                          const int32_t (&ws)[16], int32_t *mbuf, int &mc, int k1, int32_t *wsm) {
+                                          const int32_t (&ws)[N], int32_t *mbuf, int &mc, int k1, int32_t *wsm) {
+    if (!__any_sync(kFull, push != 0)) return;
     int tot;
     const int ex = warp_exclusive(__popc(push), &tot);
-    if (tot == 0) return;
     if (mc + tot > kMarkCap) marks_flush(g, st, mbuf, mc, k1, wsm);
     if (tot > kMarkCap) {  // more than the buffer holds: queue them one slot position at a time
 #pragma unroll
-        for (int q = 0; q < 16; ++q) {
+        for (int q = 0; q < N; ++q) {
             const bool mk = (push >> q) & 1u;
             if (__any_sync(kFull, mk)) enqueue_marked(g, st, mk, ws[q], k1, wsm);
         }
@@ -1369,7 +1389,7 @@ __device__ __forceinline__ void marks_add(const GraphCtx &g, const RoundStage &s
     }
     int pos = mc + ex;
 #pragma unroll
-    for (int q = 0; q < 16; ++q)
+    for (int q = 0; q < N; ++q)
         if ((push >> q) & 1u) mbuf[pos++] = ws[q];
     __syncwarp();
     mc += tot;
@@ -1396,388 +1416,601 @@ __device__ void ins_test_initial(Team &T, const GraphCtx &g, const RoundStage &s
     }
 }
 
-template <class Team>
-__device__ bool ins_rounds(Team &T, const GraphCtx &g, const int32_t *sh_upmax, int32_t *wsm, RoundStage st) {
+// Where the insertion rounds stand (the same in every thread of the team).
+struct InsState {
+    int32_t k = 0;          // phase index
+    int32_t l = 0, lmo = 0;  // level of phase k; its movers read as flagged words on lmo .. l + 1
+    int32_t spos = 0;       // next entry of levlist
+    int32_t ninit = kInf;   // its level, kInf when there is none
+    int32_t m = 0, tlc = 0, clc = 0;  // phase k's movers, thread-mode items and chunk items
+    bool scan = false;      // phase k scans the movers of l (else it tests the initial candidates on l)
+    bool done = false;
+};
+
+// One thread's share of the batch's statistics.
+struct InsCount {
     unsigned long long visits = 0, scanned = 0, upv = 0;
     unsigned aff = 0;  // neighbours whose counters a move changed
+};
+
+// After a phase whose movers all climb on to level l and nobody else does: how many
+// pure rounds lie ahead (lowc: kInf minus the lowest level of a neighbour that is
+// no mover, 0 for none; minup: the movers' smallest up-degree; init: the next
+// initial-candidate level).  Round l - 1 just ran; rounds l .. l + j - 1 are pure while
+// no other neighbour sits on l .. l + j + 1, no initial candidate on l + 1 .. l + j and
+// every member still violates on l + j.
+__device__ __forceinline__ int32_t ins_pure_rounds(const GraphCtx &g, const int32_t *sh_upmax, int32_t l,
+                                                   int32_t low, int32_t minup, int32_t init) {
+    int gg = l / g.Lg;  // highest group whose cutoff stays below the smallest up-degree
+    while (gg + 1 < g.G && sh_upmax[gg + 1] < minup) ++gg;
+    const int64_t top = (int64_t)(gg + 1) * g.Lg - 1;
+    const int64_t j = min(min((int64_t)low - l - 2, (int64_t)init - l - 1), top - l);
+    return j > 0 ? (int32_t)j : 0;
+}
+
+// The chunk items cl[0..clc) of a phase, U per warp step, all loads of a step issued
+// together; taken from the last warp down, so that in a small round the warps
+// scanning thread-mode items and those scanning chunks are different ones.  ph4: a
+// grid's prefetched first item of each warp (the other teams read the list).
+template <int U, class Team>
+__device__ __forceinline__ void ins_scan_chunks(Team &T, const GraphCtx &g, const RoundStage &st, int32_t *wsm,
+                                                int32_t *mbuf, int &mc, const InsState &s, int32_t cut_next,
+                                                const int4 *cl, int32_t &low, InsCount &a) {
     const int lane = lane_id();
+    const int32_t l = s.l, k = s.k, clc = s.clc;
+    const int32_t fcur = phase_flag(k), fnext = phase_flag(k + 1);
+    // up-lists: read from the buffer written in phase k - 1, written to this phase's
+    // buffer (its room was handed out in phase k - 1)
+    const int4 *lin4 = reinterpret_cast<const int4 *>(g.lbuf[(k + 2) % 3]);
+    int32_t *lwr = g.lbuf[k % 3];
+    int32_t *fill_cur = g.lfill[k & 1];  // reset when this phase's movers were queued
     const int4 *pool4 = reinterpret_cast<const int4 *>(g.slots);
-    const int32_t nlev = g.ctl->nlev;
+    const int crank = T.nwarps() - 1 - T.srank();
+    for (int c0 = crank; c0 < clc; c0 += U * T.nwarps()) {
+        int4 it[U];
+        bool ok[U], in[U];
+        int32_t ws[4 * U], lv[4 * U];
+        int32_t upl = 0, lol = -1, dgl = 0;  // lane u < U: item u's vertex: up-degree, output up-list, degree
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int cu = c0 + u * T.nwarps();
+            it[u] = cu < clc ? ((Team::kGrid && cu == crank) ? st.ph4[threadIdx.x >> 5] : cl[cu]) : make_int4(0, 0, 0, 0);
+            const bool lst = (it[u].y & 31) == 31;
+            ok[u] = cu < clc && (lst ? (it[u].x >= 0 && it[u].x < g.n && it[u].w >= 0 && it[u].z >= 0 &&
+                                        (int64_t)it[u].z * 4 + it[u].w <= g.lcap)
+                                     : item_ok(g, it[u], it[u].y & 31));
+            if (lane == u && ok[u]) {
+                upl = g.up[it[u].x];
+                lol = g.lout[it[u].x];
+                dgl = g.deg[it[u].x];
+            }
+            const int ng = lst ? (it[u].w + 3) >> 2 : (1 << (it[u].y & 31)) >> 2;
+            const int j = (it[u].y >> 5) * (kChunk / 4) + lane;
+            in[u] = ok[u] && j < ng;
+            const int4 s4 = in[u] ? (lst ? lin4[it[u].z + j] : pool4[it[u].z + j]) : empty4();
+            ws[4 * u] = s4.x; ws[4 * u + 1] = s4.y; ws[4 * u + 2] = s4.z; ws[4 * u + 3] = s4.w;
+        }
+#pragma unroll
+        for (int q = 0; q < 4 * U; ++q) lv[q] = valid_id(g, ws[q]) ? g.level[ws[q]] : 0;
+        int cl4[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) cl4[u] = 0;
+        unsigned push = 0, keep = 0;
+        ins_effects(g, ws, lv, l, s.lmo, fcur, fnext, cut_next, cl4, low, push, keep, a.aff);
+#pragma unroll
+        for (int u = 0; u < U; ++u) a.scanned += in[u] ? 4 : 0;
+        marks_add(g, st, push, ws, mbuf, mc, k + 1, wsm);
+        // per item u: neighbours left on l (cnt), entries kept for the up-list
+        // (kept, with this lane's offset kex[u]); lane u < U then issues item u's
+        // two atomics together: room in the up-list, and the chunk count
+        int kex[U];
+        int myc = 0, mykt = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int c = (int)__reduce_add_sync(kFull, (unsigned)cl4[u]);
+            int kt;
+            kex[u] = warp_exclusive(__popc((keep >> (4 * u)) & 0xFu), &kt);
+            if (lane == u) {
+                myc = c;
+                mykt = kt;
+            }
+        }
+        int4 mine = it[0];
+        bool mok = ok[0];
+#pragma unroll
+        for (int u = 1; u < U; ++u)
+            if (lane == u) {
+                mine = it[u];
+                mok = ok[u];
+            }
+        const bool mlst = (mine.y & 31) == 31;
+        int fbase = 0;
+        bool last = false;
+        int32_t total = 0;
+        if (lane < U && mok) {
+            const int nch = mlst ? max(1, (mine.w + kChunk - 1) / kChunk) : max(1, (1 << (mine.y & 31)) / kChunk);
+            last = true;
+            total = myc;
+            if (nch > 1) {  // (a mover of one chunk has its up-list and its count to itself)
+                if (lol >= 0 && mykt > 0) fbase = atomicAdd(&fill_cur[mine.x], mykt);
+                const unsigned long long o =
+                    atomicAdd(&g.acc[mine.x], (1ull << 32) | (unsigned long long)(uint32_t)myc);
+                last = (int)(o >> 32) + 1 == nch;
+                total = (int32_t)(uint32_t)(o & 0xffffffffull) + myc;
+                if (last) g.acc[mine.x] = 0ull;
+            }
+        }
+        // the kept neighbours go to their mover's up-list
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int32_t lo = __shfl_sync(kFull, lol, u);
+            const int kb0 = __shfl_sync(kFull, fbase, u);
+            if (lo < 0) continue;  // warp-uniform
+            const unsigned kb = (keep >> (4 * u)) & 0xFu;
+            int32_t *dst = lwr + (int64_t)lo * 4 + kb0 + kex[u];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if ((kb >> q) & 1u) *dst++ = ws[4 * u + q];
+        }
+        // the last chunk of a mover to finish completes it (lane u: item u)
+        int32_t nul = 0;  // lane u < U: item u's new up-degree
+        bool cont = false;
+        if (last) {
+            a.visits += dgl;  // a move examines the mover's neighbours: its degree
+            a.upv += upl;
+            nul = upl - total;
+            cont = ins_finish_mover(g, mine.x, upl, total, l, fcur, fnext, cut_next);
+            for (int p = nul; cont && lol >= 0 && (p & 3); ++p) lwr[(int64_t)lol * 4 + p] = kEmpty;
+        }
+        ff_note(st, cont, nul, dgl);
+        // a mover that keeps climbing is scanned next from its up-list, or from
+        // its table again when its list did not fit
+        int32_t mc_cap = 0;
+        int64_t moff = 0;
+        if (cont && lol < 0) {
+            if (mlst) {
+                mc_cap = g.cap[mine.x];
+                moff = g.off[mine.x];
+            } else {
+                mc_cap = 1 << (mine.y & 31);
+                moff = (int64_t)mine.z * 4;
+            }
+        }
+        enqueue_ins(g, st, cont, mine.x, mc_cap, moff, (cont && lol >= 0) ? nul : -1, lol, nul, k + 1, wsm);
+    }
+}
+
+// The work of phase k: the initial candidates S[s_lo, s_hi) (on l in a test phase,
+// on l + 1 in a scan phase), and in a scan phase the effects of the movers of l,
+// items tl[0..s.tlc) and cl[0..s.clc).
+template <class Team>
+__device__ __forceinline__ void ins_phase_work(Team &T, const GraphCtx &g, const RoundStage &st,
+                                               const int32_t *sh_upmax, int32_t *wsm, const InsState &s, int32_t s_lo,
+                                               int32_t s_hi, const int4 *tl, const int4 *cl, InsCount &a) {
+    const int lane = lane_id();
+    const int32_t l = s.l, k = s.k, tlc = s.tlc;
+    if (!s.scan) {
+        ins_test_initial(T, g, st, s_lo, s_hi, l, sh_upmax[l / g.Lg], wsm, 0, k + 1);
+        return;
+    }
+    const int4 *pool4 = reinterpret_cast<const int4 *>(g.slots);
     int32_t *mbuf = wsm + 160;
     int mc = 0;
-    int spos = 0;
-    int32_t l = nlev > 0 ? g.levlist[spos++] : 0;
-    int32_t lmo = l;     // movers of l read as flagged words on levels lmo .. l + 1
-    bool ffed = false;   // pure rounds were skipped just before this phase
-    bool scan = false;  // this phase scans the movers of l (else it tests the initial candidates on l)
-    for (int k = 0; nlev > 0; ++k) {
-        if ((scan && l >= g.K - 1) || k > 2 * g.K + 4) {  // the top group is never violated
-            if (T.leader()) report(g, kErrInternal, 5, l, k, 0);
+    int32_t low = kInf;  // lowest level above l of a neighbour of a mover that is no mover
+    const int32_t fcur = phase_flag(k), fnext = phase_flag(k + 1);
+    const int32_t cut_next = sh_upmax[(l + 1) / g.Lg];
+    if (s_lo < s_hi)  // initial candidates on l + 1
+        ins_test_initial(T, g, st, s_lo, s_hi, l + 1, cut_next, wsm, T.nwarps() / 2, k + 1);
+    // thread-mode movers: up to 4 groups (16 slots) per pass, loads issued together
+    for (int i0 = T.srank() * 32; i0 < tlc; i0 += T.nwarps() * 32) {
+        const int i = i0 + lane;
+        const int4 it = i < tlc ? tl[i] : make_int4(0, 0, 0, 0);
+        const bool have = i < tlc && item_ok(g, it, it.y);
+        const int ng = have ? (1 << it.y) >> 2 : 0;
+        const int32_t up_v = have ? g.up[it.x] : 0;  // issued with the slot loads
+        const int maxg = (int)__reduce_max_sync(kFull, (unsigned)ng);
+        int cnt_l = 0, ideg = 0;
+        for (int j0 = 0; j0 < maxg; j0 += 4) {
+            int32_t ws[16], lv[16];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int4 s4 = j0 + j < ng ? pool4[it.z + j0 + j] : empty4();
+                ws[4 * j] = s4.x; ws[4 * j + 1] = s4.y; ws[4 * j + 2] = s4.z; ws[4 * j + 3] = s4.w;
+            }
+#pragma unroll
+            for (int q = 0; q < 16; ++q) lv[q] = valid_id(g, ws[q]) ? g.level[ws[q]] : 0;
+            unsigned push = 0, keep = 0;
+            int c4[4] = {0, 0, 0, 0};
+#pragma unroll
+            for (int q = 0; q < 16; ++q) ideg += ws[q] >= 0;
+            ins_effects(g, ws, lv, l, s.lmo, fcur, fnext, cut_next, c4, low, push, keep, a.aff);
+            cnt_l += c4[0] + c4[1] + c4[2] + c4[3];
+            a.scanned += 4 * (unsigned long long)max(0, min(4, ng - j0));
+            marks_add(g, st, push, ws, mbuf, mc, k + 1, wsm);
+        }
+        a.visits += ideg;
+        a.upv += up_v;
+        const bool again = have && ins_finish_mover(g, it.x, up_v, cnt_l, l, fcur, fnext, cut_next);
+        ff_note(st, again, up_v - cnt_l, ideg);
+        enqueue_ins(g, st, again, it.x, have ? 1 << it.y : 0, (int64_t)it.z * 4, -1, 0, 0, k + 1, wsm);
+    }
+    if (!Team::kGrid && s.clc <= T.nwarps()) ins_scan_chunks<1>(T, g, st, wsm, mbuf, mc, s, cut_next, cl, low, a);
+    else ins_scan_chunks<4>(T, g, st, wsm, mbuf, mc, s, cut_next, cl, low, a);
+    marks_flush(g, st, mbuf, mc, k + 1, wsm);
+    low = (int32_t)__reduce_min_sync(kFull, (unsigned)low);
+    if (lane == 0 && low < kInf) atomicMin(&st.ff[2], low);
+}
+
+// The state after a phase that left nm movers for the next one, of which ncont
+// climb on (smallest up-degree minup, degree and up-degree sums sdeg and sup) and
+// whose movers' other neighbours start at level low; advances s to the next phase.
+__device__ __forceinline__ void ins_advance(const GraphCtx &g, const int32_t *sh_upmax, InsState &s, bool has_init,
+                                            int32_t ninit, int32_t nlev, int32_t nm, int32_t ncont, int32_t minup,
+                                            int32_t low, const unsigned long long *sdeg,
+                                            const unsigned long long *sup, bool leader) {
+    const int32_t m = s.m;
+    if (s.scan) {
+        if (has_init) ++s.spos;
+        ++s.l;
+        s.ninit = ninit;
+    }
+    s.lmo = s.l;
+    ++s.k;
+    s.m = nm;
+    if (s.scan && m > 0 && nm == m && ncont == m) {  // the same movers climb on: skip the pure rounds ahead
+        const int32_t j = ins_pure_rounds(g, sh_upmax, s.l, low, minup, s.ninit);
+        if (j > 0) {
+            if (leader) {
+                const unsigned long long jm = (unsigned long long)j * (unsigned long long)m;
+                const unsigned long long jv = (unsigned long long)j * *sdeg;
+                const unsigned long long ju = (unsigned long long)j * *sup;
+                atomicAdd(&g.ctl->st[kStRounds], (unsigned long long)j);
+                atomicAdd(&g.ctl->st[kStMoves], jm);
+                atomicAdd(&g.ctl->st[kStVisits], jv);
+                atomicAdd(&g.ctl->st[kStUpVisits], ju);
+                atomicAdd(&g.ctl->st[kStSkipRounds], (unsigned long long)j);
+                atomicAdd(&g.ctl->st[kStSkipMoves], jm);
+                atomicAdd(&g.ctl->st[kStSkipVisits], jv);
+                atomicAdd(&g.ctl->st[kStSkipUpVisits], ju);
+            }
+            s.l += j;
+        }
+    }
+    if (nm > 0) {
+        s.scan = true;
+    } else if (s.spos >= nlev) {
+        s.done = true;
+    } else {
+        s.l = s.lmo = s.ninit;
+        ++s.spos;
+        s.ninit = s.spos < nlev ? g.levlist[s.spos] : kInf;
+        s.scan = false;
+    }
+}
+
+// The initial candidates S[lo, hi) that the next phase tests: those on l (a test
+// phase), those on l + 1 (a scan phase) or none.
+__device__ __forceinline__ void ins_initial_range(const GraphCtx &g, const InsState &s, int32_t &lo, int32_t &hi) {
+    lo = hi = 0;
+    if (s.scan && s.ninit != s.l + 1) return;
+    const int32_t x = s.scan ? s.l + 1 : s.l;
+    lo = x == 0 ? 0 : g.bins[x - 1];
+    hi = g.bins[x];
+}
+
+__device__ __forceinline__ void ins_trace(const GraphCtx &g, const InsState &before, int32_t tlc, int32_t clc,
+                                          int32_t skip, uint64_t t0, uint64_t t1, int32_t last, int32_t first) {
+    if (g.ctl->trace_n >= g.trace_cap) return;
+    int32_t *rec = g.trace + 12 * g.ctl->trace_n++;
+    rec[0] = before.l; rec[1] = before.scan ? 1 : 0; rec[2] = before.m; rec[3] = tlc; rec[4] = clc;
+    rec[5] = (int32_t)(t1 - t0); rec[6] = (int32_t)(global_ns() - t1);
+    rec[7] = skip;
+    rec[8] = last;
+    rec[9] = first;
+    rec[10] = rec[11] = 0;
+}
+
+// Phases run by one block with its lists in shared memory: a block team's rounds, and
+// (kLimit) the small phases of a grid's rounds, which block 0 runs alone while the
+// other blocks wait at one grid barrier.  A phase boundary is one block barrier
+// (~0.1 us; a grid phase spends ~5 us from its last block's end of work to the next
+// phase's first loads: list room, publication, grid barrier, fetch), so a phase costs
+// its chain of dependent loads and atomics.  With kLimit the phases stop -- lists
+// published, s the next phase's state -- when the next lists are above kSoloCl chunk
+// or kSoloTl thread items, or when the stretch has taken a quarter of the wait limit.
+// The headers of a phase (three sets, phase index mod 3: a set is reset a phase
+// after its last readers passed the barrier) hold the list headers, the counts of the
+// lists' overflow to global memory, the movers, their totals and the error word.
+constexpr int kSoloCl = 96, kSoloTl = 512;  // largest lists of a phase that one block runs alone
+
+template <bool kLimit>
+__device__ bool ins_phases_local(const GraphCtx &g, const int32_t *sh_upmax, int32_t *wsm, RoundStage st,
+                                 InsState &s, int32_t s_lo, int32_t s_hi, const int4 *tl, const int4 *cl,
+                                 InsCount &a) {
+    BlockTeam T{g.ctl};
+    int32_t *sets = reinterpret_cast<int32_t *>(st.ph4);  // 3 sets of 16 ints
+    int4 *const tbuf[2] = {st.tl.buf, st.pk.buf};
+    int4 *const cbuf[2] = {st.cl.buf, st.cl.buf + (st.cl.cap >> 1)};
+    st.tl.cap = min(st.tl.cap, st.pk.cap);
+    st.cl.cap >>= 1;
+    st.ltop = reinterpret_cast<unsigned long long *>(st.phs + 16);
+    const int32_t nlev = g.ctl->nlev;
+    auto reset = [&](int set) {
+        int32_t *h = sets + 16 * set;
+        h[0] = 0; h[1] = st.tl.cap; h[2] = 0; h[3] = st.cl.cap;
+        h[4] = h[5] = h[6] = h[7] = 0;
+        h[8] = h[9] = kInf;
+        reinterpret_cast<unsigned long long *>(h + 10)[0] = 0;
+        reinterpret_cast<unsigned long long *>(h + 10)[1] = 0;
+        h[14] = 0;
+    };
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int i = 0; i < 3; ++i) {
+            reset(i);
+            st.ltop[i] = 0;
+        }
+    __syncthreads();
+    const uint64_t t_start = kLimit && threadIdx.x == 0 ? global_ns() : 0;
+    for (;;) {
+        if ((s.scan && s.l >= g.K - 1) || s.k > 2 * g.K + 4) {  // the top group is never violated
+            if (threadIdx.x == 0) report(g, kErrInternal, 5, s.l, s.k, 0);
             return false;
         }
-        const int cur = k % 3, nxt = (k + 1) % 3, old = (k + 2) % 3;
-        // up-lists: read from buffer old (written in phase k - 1), written to buffer
-        // cur (room handed out in phase k - 1), room handed out now from buffer nxt
-        const int32_t *lin = g.lbuf[old];
-        int32_t *lwr = g.lbuf[cur];
-        int32_t *fill_cur = g.lfill[k & 1];  // reset when this phase's movers were queued
-        const uint64_t t_phase = (g.trace && T.leader()) ? global_ns() : 0;
-        int32_t tlc = 0, clc = 0, m = 0;
-        bool has_init = false;
-        if (T.leader()) {  // the lists of phase k - 1 are done with; phase k + 1 fills them next
-            g.ctl->itl[old] = 0;
-            g.ctl->icl[old] = 0;
-            g.ctl->imcnt[old] = 0;
-            g.ctl->ltop[old] = 0;  // allocated from in phase k + 1 (its contents are read now)
-            g.ctl->icont[old] = 0;
-            g.ctl->iminup_c[old] = 0;
-            g.ctl->ilow_c[old] = 0;
-            g.ctl->isdeg[old] = 0;
-            g.ctl->isup[old] = 0;
-        }
-        int32_t low = kInf;  // lowest level above l of a neighbour of a mover that is no mover
-        st.tl.gcnt = &g.ctl->itl[nxt];
+        const int set = s.k % 3, nxt = (s.k + 1) % 3, b = s.k & 1;
+        int32_t *h = sets + 16 * set;
+        st.tl.buf = tbuf[b];
+        st.tl.hdr = h;
+        st.tl.gcnt = h + 4;
         st.tl.glist = g.TL[nxt];
         st.tl.gcap = g.n;
-        st.cl.gcnt = &g.ctl->icl[nxt];
+        st.cl.buf = cbuf[b];
+        st.cl.hdr = h + 2;
+        st.cl.gcnt = h + 5;
         st.cl.glist = g.CL[nxt];
         st.cl.gcap = g.clcap;
-        if (!scan) {
-            const int32_t s_lo = l == 0 ? 0 : g.bins[l - 1], s_hi = g.bins[l];
-            ins_test_initial(T, g, st, s_lo, s_hi, l, sh_upmax[l / g.Lg], wsm, 0, k + 1);
-        } else {
-            // counts, next initial-candidate level and its range (fetched at a grid barrier)
-            int32_t s_lo, s_hi;
-            if constexpr (Team::kGrid) {
-                m = st.phs[1];
-                tlc = st.phs[2];
-                clc = st.phs[3];
-                has_init = st.phs[4] == l + 1;
-                s_lo = st.phs[5];
-                s_hi = st.phs[6];
-                if (ffed && has_init) {  // fetched for the level before the skip
-                    s_lo = g.bins[l];
-                    s_hi = g.bins[l + 1];
-                }
-            } else {
-                m = g.ctl->imcnt[cur];
-                tlc = g.ctl->itl[cur];
-                clc = g.ctl->icl[cur];
-                has_init = spos < nlev && g.levlist[spos] == l + 1;
-                s_lo = has_init ? g.bins[l] : 0;
-                s_hi = has_init ? g.bins[l + 1] : 0;
-            }
-            if (T.leader()) {
-                atomicAdd(&g.ctl->st[kStRounds], 1ull);
-                atomicAdd(&g.ctl->st[kStMoves], (unsigned long long)m);
-            }
-            const int32_t fcur = phase_flag(k), fnext = phase_flag(k + 1);
-            const int32_t cut_next = sh_upmax[(l + 1) / g.Lg];
-            if (has_init)  // initial candidates on l + 1
-                ins_test_initial(T, g, st, s_lo, s_hi, l + 1, cut_next, wsm, T.nwarps() / 2, k + 1);
-            // thread-mode movers: up to 4 groups (16 slots) per pass, loads issued together
-            for (int i0 = T.srank() * 32; i0 < tlc; i0 += T.nwarps() * 32) {
-                const int i = i0 + lane;
-                const int4 it = i < tlc ? g.TL[cur][i] : make_int4(0, 0, 0, 0);
-                const bool have = i < tlc && item_ok(g, it, it.y);
-                const int ng = have ? (1 << it.y) >> 2 : 0;
-                const int32_t up_v = have ? g.up[it.x] : 0;  // issued with the slot loads
-                const int maxg = (int)__reduce_max_sync(kFull, (unsigned)ng);
-                int cnt_l = 0, ideg = 0;
-                for (int j0 = 0; j0 < maxg; j0 += 4) {
-                    int32_t ws[16], lv[16];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const int4 s4 = j0 + j < ng ? pool4[it.z + j0 + j] : empty4();
-                        ws[4 * j] = s4.x; ws[4 * j + 1] = s4.y; ws[4 * j + 2] = s4.z; ws[4 * j + 3] = s4.w;
-                    }
-#pragma unroll
-                    for (int q = 0; q < 16; ++q) lv[q] = valid_id(g, ws[q]) ? g.level[ws[q]] : 0;
-                    unsigned push = 0, keep = 0;
-                    int c4[4] = {0, 0, 0, 0};
-#pragma unroll
-                    for (int q = 0; q < 16; ++q) ideg += ws[q] >= 0;
-                    ins_effects16(g, ws, lv, l, lmo, fcur, fnext, cut_next, c4, low, push, keep, aff);
-                    cnt_l += c4[0] + c4[1] + c4[2] + c4[3];
-                    scanned += 4 * (unsigned long long)max(0, min(4, ng - j0));
-                    marks_add(g, st, push, ws, mbuf, mc, k + 1, wsm);
-                }
-                visits += ideg;
-                upv += up_v;
-                const bool again = have && ins_finish_mover(g, it.x, up_v, cnt_l, l, fcur, fnext, cut_next);
-                ff_note(st, again, up_v - cnt_l, ideg);
-                enqueue_ins(g, st, again, it.x, have ? 1 << it.y : 0, (int64_t)it.z * 4, -1, 0, 0, k + 1, wsm);
-            }
-            // chunk items: four per warp iteration, all loads of a step issued together;
-            // taken from the last warp down, so that in a small round the warps
-            // scanning thread-mode items and those scanning chunks are different ones
-            const int crank = T.nwarps() - 1 - T.srank();
-            const int4 *lin4 = reinterpret_cast<const int4 *>(lin);
-            for (int c0 = crank; c0 < clc; c0 += 4 * T.nwarps()) {
-                int4 it[4];
-                bool ok[4], in[4];
-                int32_t ws[16], lv[16];
-                int32_t upl = 0, lol = -1, dgl = 0;  // lane u < 4: item u's vertex: up-degree, output up-list, degree
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int cu = c0 + u * T.nwarps();
-                    it[u] = cu < clc ? ((Team::kGrid && cu == crank) ? st.ph4[threadIdx.x >> 5] : g.CL[cur][cu]) : make_int4(0, 0, 0, 0);
-                    const bool lst = (it[u].y & 31) == 31;
-                    ok[u] = cu < clc && (lst ? (it[u].x >= 0 && it[u].x < g.n && it[u].w >= 0 && it[u].z >= 0 &&
-                                                (int64_t)it[u].z * 4 + it[u].w <= g.lcap)
-                                             : item_ok(g, it[u], it[u].y & 31));
-                    if (lane == u && ok[u]) {
-                        upl = g.up[it[u].x];
-                        lol = g.lout[it[u].x];
-                        dgl = g.deg[it[u].x];
-                    }
-                    const int ng = lst ? (it[u].w + 3) >> 2 : (1 << (it[u].y & 31)) >> 2;
-                    const int j = (it[u].y >> 5) * (kChunk / 4) + lane;
-                    in[u] = ok[u] && j < ng;
-                    const int4 s4 = in[u] ? (lst ? lin4[it[u].z + j] : pool4[it[u].z + j]) : empty4();
-                    ws[4 * u] = s4.x; ws[4 * u + 1] = s4.y; ws[4 * u + 2] = s4.z; ws[4 * u + 3] = s4.w;
-                }
-#pragma unroll
-                for (int q = 0; q < 16; ++q) lv[q] = valid_id(g, ws[q]) ? g.level[ws[q]] : 0;
-                int cl4[4] = {0, 0, 0, 0};
-                unsigned push = 0, keep = 0;
-                ins_effects16(g, ws, lv, l, lmo, fcur, fnext, cut_next, cl4, low, push, keep, aff);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) scanned += in[u] ? 4 : 0;
-                marks_add(g, st, push, ws, mbuf, mc, k + 1, wsm);
-                // per item u: neighbours left on l (cnt), entries kept for the up-list
-                // (kept, with this lane's offset kex[u]); lane u < 4 then issues item u's
-                // two atomics together: room in the up-list, and the chunk count
-                int kex[4];
-                int myc = 0, mykt = 0;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int c = warp_sum(cl4[u]);
-                    int kt;
-                    kex[u] = warp_exclusive(__popc((keep >> (4 * u)) & 0xFu), &kt);
-                    if (lane == u) {
-                        myc = c;
-                        mykt = kt;
-                    }
-                }
-                int4 mine = it[0];
-                bool mok = ok[0];
-#pragma unroll
-                for (int u = 1; u < 4; ++u)
-                    if (lane == u) {
-                        mine = it[u];
-                        mok = ok[u];
-                    }
-                const bool mlst = (mine.y & 31) == 31;
-                int fbase = 0;
-                bool last = false;
-                int32_t total = 0;
-                if (lane < 4 && mok) {
-                    if (lol >= 0 && mykt > 0) fbase = atomicAdd(&fill_cur[mine.x], mykt);
-                    const int nch = mlst ? max(1, (mine.w + kChunk - 1) / kChunk) : max(1, (1 << (mine.y & 31)) / kChunk);
-                    last = true;
-                    total = myc;
-                    if (nch > 1) {
-                        const unsigned long long o =
-                            atomicAdd(&g.acc[mine.x], (1ull << 32) | (unsigned long long)(uint32_t)myc);
-                        last = (int)(o >> 32) + 1 == nch;
-                        total = (int32_t)(uint32_t)(o & 0xffffffffull) + myc;
-                        if (last) g.acc[mine.x] = 0ull;
-                    }
-                }
-                // the kept neighbours go to their mover's up-list
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int32_t lo = __shfl_sync(kFull, lol, u);
-                    const int kb0 = __shfl_sync(kFull, fbase, u);
-                    if (lo < 0) continue;  // warp-uniform
-                    const unsigned kb = (keep >> (4 * u)) & 0xFu;
-                    int32_t *dst = lwr + (int64_t)lo * 4 + kb0 + kex[u];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        if ((kb >> q) & 1u) *dst++ = ws[4 * u + q];
-                }
-                // the last chunk of a mover to finish completes it (lane u: item u)
-                int32_t nul = 0;  // lane u < 4: item u's new up-degree
-                bool cont = false;
-                if (last) {
-                    visits += dgl;  // a move examines the mover's neighbours: its degree
-                    upv += upl;
-                    nul = upl - total;
-                    cont = ins_finish_mover(g, mine.x, upl, total, l, fcur, fnext, cut_next);
-                    for (int p = nul; cont && lol >= 0 && (p & 3); ++p) lwr[(int64_t)lol * 4 + p] = kEmpty;
-                }
-                ff_note(st, cont, nul, dgl);
-                // a mover that keeps climbing is scanned next from its up-list, or from
-                // its table again when its list did not fit
-                int32_t mc_cap = 0;
-                int64_t moff = 0;
-                if (cont && lol < 0) {
-                    if (mlst) {
-                        mc_cap = g.cap[mine.x];
-                        moff = g.off[mine.x];
-                    } else {
-                        mc_cap = 1 << (mine.y & 31);
-                        moff = (int64_t)mine.z * 4;
-                    }
-                }
-                enqueue_ins(g, st, cont, mine.x, mc_cap, moff, (cont && lol >= 0) ? nul : -1, lol, nul, k + 1, wsm);
-            }
-            marks_flush(g, st, mbuf, mc, k + 1, wsm);
-            low = (int32_t)__reduce_min_sync(kFull, (unsigned)low);
-            if (lane == 0 && low < kInf) atomicMin(&st.ff[2], low);
-        }
-        const uint64_t t_work = (g.trace && T.leader()) ? global_ns() : 0;
-        if (g.trace) {  // every block: when it finished its share of the phase
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                const unsigned long long tb = global_ns();
-                atomicMax(&g.ctl->tw_max[k & 1], tb);
-                atomicMax(&g.ctl->tw_min_c[k & 1], ~tb);
-            }
-        }
-        stage_flush_round(g, st, 6u);
+        st.movers = h + 6;
+        st.ff = h + 7;
+        st.ff64 = reinterpret_cast<unsigned long long *>(h + 10);
+        int32_t err = 0;
+        uint64_t t_phase = 0;
         if (threadIdx.x == 0) {
-            if (*st.movers) {
-                atomicAdd(&g.ctl->imcnt[nxt], *st.movers);
-                *st.movers = 0;
-            }
-            if (st.ff[0]) {  // the block's climbing movers (complements: zero means none)
-                atomicAdd(&g.ctl->icont[nxt], st.ff[0]);
-                atomicMax(&g.ctl->iminup_c[nxt], kInf - st.ff[1]);
-                atomicAdd(&g.ctl->isdeg[nxt], st.ff64[0]);
-                atomicAdd(&g.ctl->isup[nxt], st.ff64[1]);
-                st.ff[0] = 0;
-                st.ff[1] = kInf;
-                st.ff64[0] = 0;
-                st.ff64[1] = 0;
-            }
-            if (st.ff[2] < kInf) {
-                atomicMax(&g.ctl->ilow_c[nxt], kInf - st.ff[2]);
-                st.ff[2] = kInf;
+            reset(nxt);  // last read after the barrier of phase k - 2
+            st.ltop[(s.k + 2) % 3] = 0;  // that buffer's room is handed out from phase k + 1 on
+            err = ld_volatile(&g.ctl->err);  // seen one phase late, off the critical chain
+            if (g.trace || kLimit) t_phase = global_ns();
+            if (s.scan) {
+                atomicAdd(&g.ctl->st[kStRounds], 1ull);
+                atomicAdd(&g.ctl->st[kStMoves], (unsigned long long)s.m);
             }
         }
-        // the level the next phase scans if it has movers, and its initial-candidate
-        // entry; warp 0 fetches them with the next phase's counts and each warp's
-        // first chunk item while it passes the barrier
-        int spos2 = spos;
-        int32_t l2 = l;
-        if (scan) {
-            if (has_init) ++spos2;
-            ++l2;
+        const bool has_init = s.scan && s.ninit == s.l + 1;
+        const int32_t ninit = has_init ? (s.spos + 1 < nlev ? g.levlist[s.spos + 1] : kInf) : s.ninit;
+        ins_phase_work(T, g, st, sh_upmax, wsm, s, s_lo, s_hi, tl, cl, a);
+        if (threadIdx.x == 0) {
+            h[14] = err;
+            if (kLimit) h[15] = t_phase - t_start > (uint64_t)(g.wait_limit_ns >> 2);
         }
-        bool passed;
-        if constexpr (Team::kGrid) {
-            const int4 *cl_next = g.CL[nxt];
-            passed = T.sync_fetch(
-                [&](int ln) {
-                    if (ln < (int)(blockDim.x >> 5)) {  // warp ln of the block: its first chunk item
-                        const int cr = T.nwarps() - 1 - (ln * T.nblocks() + T.bid());  // warp ln's srank
-                        st.ph4[ln] = cr < g.clcap ? cl_next[cr] : make_int4(0, 0, 0, 0);
-                    } else if (ln == 16) {
-                        st.phs[1] = g.ctl->imcnt[nxt];
-                    } else if (ln == 17) {
-                        st.phs[2] = g.ctl->itl[nxt];
-                    } else if (ln == 18) {
-                        st.phs[3] = g.ctl->icl[nxt];
-                    } else if (ln == 19) {
-                        st.phs[4] = spos2 < nlev ? g.levlist[spos2] : kInf;
-                    } else if (ln == 20) {
-                        st.phs[5] = l2 < g.K ? g.bins[l2] : 0;
-                    } else if (ln == 21) {
-                        st.phs[6] = l2 < g.K ? g.bins[l2 + 1] : 0;
-                    } else if (ln == 22) {
-                        st.phs[7] = g.ctl->icont[nxt];
-                    } else if (ln == 23) {
-                        st.phs[8] = g.ctl->ilow_c[nxt];
-                    } else if (ln == 24) {
-                        st.phs[9] = g.ctl->iminup_c[nxt];
-                    }
-                },
-                st.phs);
-        } else {
-            passed = T.sync();
+        __threadfence_block();
+        __syncthreads();
+        if (h[14] != 0) return false;
+        const InsState before = s;
+        const int nt = min(h[0], h[1]), nc = min(h[2], h[3]);  // entries in shared memory
+        const int32_t tot_t = nt + h[4], tot_c = nc + h[5];
+        ins_advance(g, sh_upmax, s, has_init, ninit, nlev, h[6], h[7], h[8], h[9], st.ff64, st.ff64 + 1,
+                    threadIdx.x == 0);
+        s.tlc = tot_t;
+        s.clc = tot_c;
+        if (g.trace && threadIdx.x == 0) {
+            const int32_t d = (int32_t)(global_ns() - t_phase);
+            ins_trace(g, before, before.tlc, before.clc, s.l - s.lmo, t_phase, t_phase + d, d, d);
         }
-        if (!passed) return false;
-        // the next phase: the movers of l + 1 (after a scan) or of l (after a test),
-        // else the initial candidates of the next level that has some
-        spos = spos2;
-        l = l2;
-        lmo = l;
-        ffed = false;
-        const int32_t nm = Team::kGrid ? st.phs[1] : g.ctl->imcnt[nxt];
-        int32_t skip = 0;
-        if (scan && m > 0 && nm == m) {
-            const int32_t ncont = Team::kGrid ? st.phs[7] : g.ctl->icont[nxt];
-            if (ncont == m) {  // the same movers climb on to l: skip the pure rounds ahead
-                const int32_t lowc = Team::kGrid ? st.phs[8] : g.ctl->ilow_c[nxt];
-                const int32_t mupc = Team::kGrid ? st.phs[9] : g.ctl->iminup_c[nxt];
-                const int64_t low_lvl = lowc ? (int64_t)(kInf - lowc) : (int64_t)kInf;
-                const int32_t minup = kInf - mupc;
-                const int64_t init_lvl = spos < nlev ? (int64_t)(Team::kGrid ? st.phs[4] : g.levlist[spos]) : (int64_t)kInf;
-                int gg = l / g.Lg;  // highest group whose cutoff stays below the smallest up-degree
-                while (gg + 1 < g.G && sh_upmax[gg + 1] < minup) ++gg;
-                const int64_t top = (int64_t)(gg + 1) * g.Lg - 1;
-                // round l - 1 just ran; rounds l .. l + j - 1 are pure while no other
-                // neighbour sits on l .. l + j + 1, no initial candidate on l + 1 .. l + j
-                // and every member still violates on l + j
-                const int64_t j = min(min(low_lvl - l - 2, init_lvl - l - 1), top - l);
-                if (j >= 1) {
-                    skip = (int32_t)j;
-                    if (T.leader()) {
-                        const unsigned long long jm = (unsigned long long)j * (unsigned long long)m;
-                        const unsigned long long jv = (unsigned long long)j * g.ctl->isdeg[nxt];
-                        const unsigned long long ju = (unsigned long long)j * g.ctl->isup[nxt];
-                        atomicAdd(&g.ctl->st[kStRounds], (unsigned long long)j);
-                        atomicAdd(&g.ctl->st[kStMoves], jm);
-                        atomicAdd(&g.ctl->st[kStVisits], jv);
-                        atomicAdd(&g.ctl->st[kStUpVisits], ju);
-                        atomicAdd(&g.ctl->st[kStSkipRounds], (unsigned long long)j);
-                        atomicAdd(&g.ctl->st[kStSkipMoves], jm);
-                        atomicAdd(&g.ctl->st[kStSkipVisits], jv);
-                        atomicAdd(&g.ctl->st[kStSkipUpVisits], ju);
-                    }
-                    lmo = l;
-                    l += skip;
-                    ffed = true;
-                }
-            }
-        }
-        if (g.trace && T.leader() && g.ctl->trace_n < g.trace_cap) {
-            int32_t *rec = g.trace + 12 * g.ctl->trace_n++;
-            const uint64_t t_end = global_ns();
-            rec[0] = scan ? l2 - 1 : l2; rec[1] = scan ? 1 : 0; rec[2] = m; rec[3] = tlc; rec[4] = clc;
-            rec[5] = (int32_t)(t_work - t_phase); rec[6] = (int32_t)(t_end - t_work);
-            rec[7] = skip;
-            // blocks' work ends after the phase start: the latest and the earliest
-            rec[8] = (int32_t)(g.ctl->tw_max[k & 1] - t_phase);
-            rec[9] = (int32_t)(~g.ctl->tw_min_c[k & 1] - t_phase);
-            rec[10] = rec[11] = 0;
-            g.ctl->tw_max[k & 1] = 0;
-            g.ctl->tw_min_c[k & 1] = 0;
-        }
-        if (nm > 0) {
-            scan = true;
+        if (s.done) return true;
+        ins_initial_range(g, s, s_lo, s_hi);
+        const bool leave = kLimit && (tot_t > kSoloTl || tot_c > kSoloCl || s_hi - s_lo > kSoloTl || h[15]);
+        if (h[4] == 0 && h[5] == 0 && !leave) {
+            tl = tbuf[b];
+            cl = cbuf[b];
             continue;
         }
-        if (spos >= nlev) break;
-        l = g.levlist[spos++];
-        scan = false;
+        // to the global lists: after the entries that overflowed there
+        if ((int64_t)tot_t > (int64_t)g.n || (int64_t)tot_c > g.clcap) {
+            if (threadIdx.x == 0) report(g, kErrListOverflow, 4, tot_t, tot_c, 0);
+            return false;
+        }
+        for (int i = threadIdx.x; i < nt; i += blockDim.x) g.TL[nxt][h[4] + i] = tbuf[b][i];
+        for (int i = threadIdx.x; i < nc; i += blockDim.x) g.CL[nxt][h[5] + i] = cbuf[b][i];
+        __threadfence_block();
+        __syncthreads();
+        tl = g.TL[nxt];
+        cl = g.CL[nxt];
+        if (leave) return true;
     }
-    if (nlev == 0) return true;  // nobody moved: no flag to clear
+}
+
+// One phase of a whole grid; advances s and the initial candidates' range to the
+// next phase.
+template <class Team>
+__device__ __forceinline__ bool ins_grid_phase(Team &T, const GraphCtx &g, const int32_t *sh_upmax, int32_t *wsm,
+                                               RoundStage &st, InsState &s, int32_t nlev, int32_t &s_lo,
+                                               int32_t &s_hi, InsCount &a) {
+    if ((s.scan && s.l >= g.K - 1) || s.k > 2 * g.K + 4) {  // the top group is never violated
+        if (T.leader()) report(g, kErrInternal, 5, s.l, s.k, 0);
+        return false;
+    }
+    const int k = s.k, cur = k % 3, nxt = (k + 1) % 3, old = (k + 2) % 3;
+    const uint64_t t_phase = (g.trace && T.leader()) ? global_ns() : 0;
+    if (T.leader()) {  // the lists of phase k - 1 are done with; phase k + 1 fills them next
+        g.ctl->itl[old] = 0;
+        g.ctl->icl[old] = 0;
+        g.ctl->imcnt[old] = 0;
+        g.ctl->ltop[old] = 0;  // allocated from in phase k + 1 (its contents are read now)
+        g.ctl->icont[old] = 0;
+        g.ctl->iminup_c[old] = 0;
+        g.ctl->ilow_c[old] = 0;
+        g.ctl->isdeg[old] = 0;
+        g.ctl->isup[old] = 0;
+        if (s.scan) {
+            atomicAdd(&g.ctl->st[kStRounds], 1ull);
+            atomicAdd(&g.ctl->st[kStMoves], (unsigned long long)s.m);
+        }
+    }
+    st.tl.gcnt = &g.ctl->itl[nxt];
+    st.tl.glist = g.TL[nxt];
+    st.tl.gcap = g.n;
+    st.cl.gcnt = &g.ctl->icl[nxt];
+    st.cl.glist = g.CL[nxt];
+    st.cl.gcap = g.clcap;
+    const bool has_init = s.scan && s.ninit == s.l + 1;
+    ins_phase_work(T, g, st, sh_upmax, wsm, s, s_lo, s_hi, g.TL[cur], g.CL[cur], a);
+    const uint64_t t_work = (g.trace && T.leader()) ? global_ns() : 0;
+    if (g.trace) {  // every block: when it finished its share of the phase
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const unsigned long long tb = global_ns();
+            atomicMax(&g.ctl->tw_max[k & 1], tb);
+            atomicMax(&g.ctl->tw_min_c[k & 1], ~tb);
+        }
+    }
+    stage_flush_round(g, st, 6u);
+    if (threadIdx.x == 0) {
+        if (*st.movers) {
+            atomicAdd(&g.ctl->imcnt[nxt], *st.movers);
+            *st.movers = 0;
+        }
+        if (st.ff[0]) {  // the block's climbing movers (complements: zero means none)
+            atomicAdd(&g.ctl->icont[nxt], st.ff[0]);
+            atomicMax(&g.ctl->iminup_c[nxt], kInf - st.ff[1]);
+            atomicAdd(&g.ctl->isdeg[nxt], st.ff64[0]);
+            atomicAdd(&g.ctl->isup[nxt], st.ff64[1]);
+            st.ff[0] = 0;
+            st.ff[1] = kInf;
+            st.ff64[0] = 0;
+            st.ff64[1] = 0;
+        }
+        if (st.ff[2] < kInf) {
+            atomicMax(&g.ctl->ilow_c[nxt], kInf - st.ff[2]);
+            st.ff[2] = kInf;
+        }
+    }
+    // the level the next phase scans if it has movers, and its initial-candidate
+    // entry; warp 0 fetches them with the next phase's counts and each warp's
+    // first chunk item while it passes the barrier
+    const int spos2 = has_init ? s.spos + 1 : s.spos;
+    const int32_t l2 = s.scan ? s.l + 1 : s.l;
+    const int4 *cl_next = g.CL[nxt];
+    const bool passed = T.sync_fetch(
+        [&](int ln) {
+            if (ln < (int)(blockDim.x >> 5)) {  // warp ln of the block: its first chunk item
+                const int cr = T.nwarps() - 1 - (ln * T.nblocks() + T.bid());  // warp ln's srank
+                st.ph4[ln] = cr < g.clcap ? cl_next[cr] : make_int4(0, 0, 0, 0);
+            } else if (ln == 16) {
+                st.phs[1] = g.ctl->imcnt[nxt];
+            } else if (ln == 17) {
+                st.phs[2] = g.ctl->itl[nxt];
+            } else if (ln == 18) {
+                st.phs[3] = g.ctl->icl[nxt];
+            } else if (ln == 19) {
+                st.phs[4] = spos2 < nlev ? g.levlist[spos2] : kInf;
+            } else if (ln == 20) {
+                st.phs[5] = l2 < g.K ? g.bins[l2] : 0;
+            } else if (ln == 21) {
+                st.phs[6] = l2 < g.K ? g.bins[l2 + 1] : 0;
+            } else if (ln == 22) {
+                st.phs[7] = g.ctl->icont[nxt];
+            } else if (ln == 23) {
+                st.phs[8] = g.ctl->ilow_c[nxt];
+            } else if (ln == 24) {
+                st.phs[9] = g.ctl->iminup_c[nxt];
+            }
+        },
+        st.phs);
+    if (!passed) return false;
+    const InsState before = s;
+    ins_advance(g, sh_upmax, s, has_init, st.phs[4], nlev, st.phs[1], st.phs[7], kInf - st.phs[9],
+                st.phs[8] ? kInf - st.phs[8] : kInf, &g.ctl->isdeg[nxt], &g.ctl->isup[nxt], T.leader());
+    s.tlc = st.phs[2];
+    s.clc = st.phs[3];
+    if (s.scan && s.l == l2 && s.ninit == s.l + 1) {
+        s_lo = st.phs[5];
+        s_hi = st.phs[6];
+    } else {
+        ins_initial_range(g, s, s_lo, s_hi);
+    }
+    if (g.trace && T.leader()) {
+        // blocks' work ends after the phase start: the latest and the earliest
+        ins_trace(g, before, before.tlc, before.clc, s.l - s.lmo, t_phase, t_work,
+                  (int32_t)(g.ctl->tw_max[k & 1] - t_phase), (int32_t)(~g.ctl->tw_min_c[k & 1] - t_phase));
+        g.ctl->tw_max[k & 1] = 0;
+        g.ctl->tw_min_c[k & 1] = 0;
+    }
+    return true;
+}
+
+template <class Team>
+__device__ bool ins_rounds(Team &T, const GraphCtx &g, const int32_t *sh_upmax, int32_t *wsm, RoundStage st) {
+    InsCount a;
+    const int32_t nlev = g.ctl->nlev;
+    if (nlev == 0) return true;  // nobody violates: nothing moves, no flag to clear
+    InsState s;
+    s.l = s.lmo = g.levlist[0];
+    s.spos = 1;
+    s.ninit = nlev > 1 ? g.levlist[1] : kInf;
+    int32_t s_lo, s_hi;
+    ins_initial_range(g, s, s_lo, s_hi);
+    if constexpr (!Team::kGrid) {
+        if (!ins_phases_local<false>(g, sh_upmax, wsm, st, s, s_lo, s_hi, nullptr, nullptr, a)) return false;
+    } else {
+        st.ltop = g.ctl->ltop;
+        while (!s.done) {
+            if (s.clc <= kSoloCl && s.tlc <= kSoloTl && s_hi - s_lo <= kSoloTl) {
+                // a small phase: block 0 goes on alone, the others wait for it
+                if (T.bid() == 0) {
+                    const int cur = s.k % 3;
+                    ins_phases_local<true>(g, sh_upmax, wsm, st, s, s_lo, s_hi, g.TL[cur], g.CL[cur], a);
+                    if (threadIdx.x == 0) {
+                        int32_t *o = g.ctl->solo;
+                        o[0] = s.k; o[1] = s.l; o[2] = s.lmo; o[3] = s.spos;
+                        o[4] = s.m; o[5] = s.tlc; o[6] = s.clc; o[7] = (s.done ? 1 : 0) | (s.scan ? 2 : 0);
+                        for (int i = 0; i < 3; ++i) {  // the grid's counters start clean
+                            g.ctl->itl[i] = g.ctl->icl[i] = g.ctl->imcnt[i] = g.ctl->icont[i] = 0;
+                            g.ctl->iminup_c[i] = g.ctl->ilow_c[i] = 0;
+                            g.ctl->isdeg[i] = g.ctl->isup[i] = 0;
+                            g.ctl->ltop[i] = 0;
+                        }
+                    }
+                }
+                if (!T.sync()) return false;
+                const int32_t *o = g.ctl->solo;
+                const int32_t fl = ld_volatile(o + 7);
+                s.k = ld_volatile(o); s.l = ld_volatile(o + 1); s.lmo = ld_volatile(o + 2); s.spos = ld_volatile(o + 3);
+                s.m = ld_volatile(o + 4); s.tlc = ld_volatile(o + 5); s.clc = ld_volatile(o + 6);
+                s.scan = (fl & 2) != 0;
+                if (fl & 1) break;
+                s.ninit = s.spos < nlev ? g.levlist[s.spos] : kInf;
+                ins_initial_range(g, s, s_lo, s_hi);
+                if (threadIdx.x < (blockDim.x >> 5)) {  // each warp's first chunk item
+                    const int cr = T.nwarps() - 1 - ((int)threadIdx.x * T.nblocks() + T.bid());
+                    st.ph4[threadIdx.x] = cr < s.clc ? g.CL[s.k % 3][cr] : make_int4(0, 0, 0, 0);
+                }
+                __syncthreads();
+            }
+            if (!ins_grid_phase(T, g, sh_upmax, wsm, st, s, nlev, s_lo, s_hi, a)) return false;
+        }
+    }
     // clear the movers' flags (every vertex: flags sit only on vertices that moved)
     for (int64_t v = T.tid(); v < g.n; v += T.nthreads()) {
         const int32_t raw = g.level[v];
         if (raw & ~kLevelMask) g.level[v] = raw & kLevelMask;
     }
-    visits = warp_sum64(visits);
-    scanned = warp_sum64(scanned);
-    upv = warp_sum64(upv);
-    const unsigned long long affs = warp_sum64(aff);
-    if (lane == 0) {
-        atomicAdd(&g.ctl->st[kStVisits], visits);
-        atomicAdd(&g.ctl->st[kStSlotsScanned], scanned);
-        atomicAdd(&g.ctl->st[kStUpVisits], upv);
+    a.visits = warp_sum64(a.visits);
+    a.scanned = warp_sum64(a.scanned);
+    a.upv = warp_sum64(a.upv);
+    const unsigned long long affs = warp_sum64(a.aff);
+    if (lane_id() == 0) {
+        atomicAdd(&g.ctl->st[kStVisits], a.visits);
+        atomicAdd(&g.ctl->st[kStSlotsScanned], a.scanned);
+        atomicAdd(&g.ctl->st[kStUpVisits], a.upv);
         if (affs) atomicAdd(&g.ctl->st[kStAffected], affs);
     }
     return T.sync();
@@ -1889,7 +2122,7 @@ __device__ __forceinline__ int warp_range_sum(const int32_t *h, int lo, int hi) 
 // answer d > 0, the neighbours on d - 1 or above minus dnmin[gn(d - 1)] (>= 0; kInf
 // for d = 0, 0 where it is not counted): while later moves do not take it below 0,
 // the answer stays d.
-__device__ int32_t warp_desire_level(const GraphCtx &g, int32_t w, int32_t lw, const int32_t *sh_dnmin,
+inline __device__ int32_t warp_desire_level(const GraphCtx &g, int32_t w, int32_t lw, const int32_t *sh_dnmin,
                                      int32_t *hist, int32_t *slack) {
     *slack = kInf;
     if (lw < 2) return 0;
@@ -1980,7 +2213,7 @@ __device__ int32_t warp_desire_level(const GraphCtx &g, int32_t w, int32_t lw, c
     }
 }
 
-__device__ int32_t block_desire_level(const GraphCtx &g, int32_t w, int32_t lw, const int32_t *sh_dnmin,
+inline __device__ int32_t block_desire_level(const GraphCtx &g, int32_t w, int32_t lw, const int32_t *sh_dnmin,
                                       int32_t *hist, int32_t *res, int32_t *slack) {
     *slack = kInf;  // as in warp_desire_level
     if (lw < 2) return 0;

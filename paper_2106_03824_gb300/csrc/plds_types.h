@@ -78,6 +78,7 @@ struct Ctl {
     int32_t mcnt[2];      // table growth / deletion movers
     int32_t tlcnt[2];     // thread-mode movers
     int32_t clcnt[2];     // chunk items
+    int32_t solo[8];      // insertion: where the rounds stand after phases run by block 0 alone
     int32_t nlev;         // number of distinct initial-candidate levels
     int32_t ncand;        // initial candidates: touched vertices that violate Invariant 1
     int32_t pcnt[2];      // deletion pending list sizes
