@@ -1609,26 +1609,29 @@ extern "C" int plds_batch_static(plds_t *h, const int32_t *edges, int64_t B, int
 //
 // A set owns `count` ordinary handles.  One round applies one mixed batch to
 // every graph (its insertion half, then its deletion half, as Algorithm 1
-// orders them).  The kernel is persistent: each block takes the next graph from
-// a work counter (graphs ordered by decreasing size) and runs that graph's whole
-// round with the same device routines as the single-graph kernel, the block
-// being the team (block barriers only, graphs progress independently).  The
-// per-round launch sequence (descriptor upload, counter reset, kernel, control
-// word read-back) is captured once in a CUDA graph and replayed.
+// orders them), with the same device routines as the single-graph kernel.  Two
+// persistent kernels take the graphs from two queues, side by side: a large graph is
+// run by a cluster of kSetCluster blocks (its steps and level phases spread over
+// them, cluster barriers between), any other by one block (block barriers only).
+// Graphs progress independently.  The per-round launch sequence (descriptor upload,
+// the two kernels, control word read-back) is captured once in a CUDA graph and
+// replayed.
 // ---------------------------------------------------------------------------
 struct plds_set {
     int32_t count = 0;
     std::vector<plds *> g;       // graph handles
-    std::vector<int32_t> order;  // graphs by decreasing n
+    std::vector<int32_t> order;  // graphs by decreasing n, the order of equal batches
     cudaStream_t stream = nullptr;   // the caller's stream (allocations, copies)
     cudaStream_t run = nullptr;      // private stream the captured round is replayed on
     bool graph_ok = true;
     plds *owner = nullptr;       // allocator and device of the set's own buffers
-    DevBuf items, ctls, next, edges;
+    DevBuf items, ctls, queue, edges;
     int64_t edges_cap = 0;
     SetItem *h_items = nullptr;  // pinned
     Ctl *h_ctls = nullptr;       // pinned
-    int grid = 0;
+    SetQueue *h_queue = nullptr;  // pinned
+    int grid = 0;                // blocks of the block kernel
+    int clusters = 0;            // clusters of the cluster kernel
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     int32_t captured_count = -1;
@@ -1648,8 +1651,25 @@ static int set_launch(plds_set *s, int32_t n_items, bool use_graph) {
     if (use_graph && s->exec && s->captured_count == n_items) return cudaGraphLaunch(s->exec, st) == cudaSuccess ? 0 : -1;
     auto enqueue = [&]() {
         cudaMemcpyAsync(s->items.p, s->h_items, sizeof(SetItem) * (size_t)n_items, cudaMemcpyHostToDevice, st);
-        cudaMemsetAsync(s->next.p, 0, sizeof(int32_t), st);
-        k_batch_set<<<s->grid, kSetThreads, smem, st>>>(P<SetItem>(s->items), n_items, P<int32_t>(s->next));
+        cudaMemcpyAsync(s->queue.p, s->h_queue, offsetof(SetQueue, slot), cudaMemcpyHostToDevice, st);
+        const SetItem *items = P<SetItem>(s->items);
+        SetQueue *q = P<SetQueue>(s->queue);
+        cudaLaunchAttribute at[1];
+        cudaLaunchConfig_t cfg{};
+        cfg.blockDim = dim3(kSetThreads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        cfg.gridDim = dim3(s->clusters * kSetCluster);
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = kSetCluster;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cudaLaunchKernelEx(&cfg, k_batch_set_cluster, items, q);
+        cfg.gridDim = dim3(s->grid);
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchKernelEx(&cfg, k_batch_set, items, q);
         cudaMemcpyAsync(s->h_ctls, s->ctls.p, sizeof(Ctl) * 2 * (size_t)n_items, cudaMemcpyDeviceToHost, st);
     };
     if (!use_graph) {
@@ -1725,9 +1745,10 @@ extern "C" plds_set_t *plds_set_create(int32_t count, const int32_t *n, double d
     for (int32_t i = 0; i < count; ++i) s->order[i] = i;
     std::stable_sort(s->order.begin(), s->order.end(), [&](int a, int b) { return s->g[a]->n > s->g[b]->n; });
     if (!dev_get(s->owner, s->items, sizeof(SetItem) * (size_t)count) ||
-        !dev_get(s->owner, s->ctls, sizeof(Ctl) * 2 * (size_t)count) || !dev_get(s->owner, s->next, 16) ||
+        !dev_get(s->owner, s->ctls, sizeof(Ctl) * 2 * (size_t)count) || !dev_get(s->owner, s->queue, sizeof(SetQueue)) ||
         cudaMallocHost(&s->h_items, sizeof(SetItem) * (size_t)count) != cudaSuccess ||
-        cudaMallocHost(&s->h_ctls, sizeof(Ctl) * 2 * (size_t)count) != cudaSuccess) {
+        cudaMallocHost(&s->h_ctls, sizeof(Ctl) * 2 * (size_t)count) != cudaSuccess ||
+        cudaMallocHost(&s->h_queue, sizeof(SetQueue)) != cudaSuccess) {
         cudaGetLastError();
         plds_set_destroy(s);
         set_status(PLDS_ENOMEM);
@@ -1738,6 +1759,9 @@ extern "C" plds_set_t *plds_set_create(int32_t count, const int32_t *n, double d
     int occ = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch_set, kSetThreads, smem);
     s->grid = std::max(1, occ) * s->owner->num_sms;
+    cudaFuncSetAttribute(k_batch_set_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_batch_set_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    s->clusters = std::min<int>((int)(sizeof(SetQueue::slot) / 4), std::max(1, s->grid / kSetCluster));
     set_status(PLDS_OK);
     return s;
 }
@@ -1774,10 +1798,22 @@ extern "C" int plds_set_update(plds_set_t *s, const int32_t *edges, const int64_
         dedges = P<int32_t>(s->edges);
     }
     // graphs still to run this round (all at first; then the ones that needed a bigger pool)
+    // in order of decreasing batch size
     std::vector<int32_t> todo(s->order);
+    auto batch_of = [&](int32_t gi) { return offsets[2 * gi + 2] - offsets[2 * gi]; };
+    std::stable_sort(todo.begin(), todo.end(), [&](int32_t a, int32_t b) { return batch_of(a) > batch_of(b); });
     Ctl *dctl = P<Ctl>(s->ctls);
     for (int attempt = 0; attempt < 4 && !todo.empty(); ++attempt) {
         const int32_t m = (int32_t)todo.size();
+        // a graph is large when one block would still be busy with it after all blocks
+        // together could have finished the round
+        int64_t sum = 0;
+        for (int32_t gi : todo) sum += batch_of(gi);
+        int32_t large = 0;
+        while (large < m && batch_of(todo[large]) * s->grid > sum) ++large;
+        s->h_queue->next[0] = s->h_queue->next[1] = 0;
+        s->h_queue->large = large;
+        s->h_queue->count = m;
         for (int32_t j = 0; j < m; ++j) {
             const int32_t gi = todo[j];
             plds *h = s->g[gi];
@@ -2082,12 +2118,13 @@ extern "C" void plds_set_destroy(plds_set_t *s) {
     if (s->owner) {
         dev_free(s->owner, s->items);
         dev_free(s->owner, s->ctls);
-        dev_free(s->owner, s->next);
+        dev_free(s->owner, s->queue);
         dev_free(s->owner, s->edges);
         cudaStreamSynchronize(s->stream);
     }
     if (s->h_items) cudaFreeHost(s->h_items);
     if (s->h_ctls) cudaFreeHost(s->h_ctls);
+    if (s->h_queue) cudaFreeHost(s->h_queue);
     for (plds *h : s->g) plds_destroy(h);
     cudaGetLastError();
     delete s;

@@ -34,6 +34,7 @@ __device__ __forceinline__ int ld_volatile(const int32_t *p) { return *(volatile
 // ---------------------------------------------------------------------------
 struct GridTeam {
     static constexpr bool kGrid = true;  // barriers cost a round trip to L2: fetch at the barrier
+    static constexpr bool kJump = true;  // may run the jump variant
     Ctl *ctl;
     int64_t limit_ns;
     int32_t sleep_ns;
@@ -103,8 +104,46 @@ struct GridTeam {
     }
 };
 
+// A thread-block cluster (hardware barrier; its blocks are always resident together).
+// The error word is read between two barriers, so that every block of the cluster
+// decides alike and no block is left waiting.
+struct ClusterTeam {
+    static constexpr bool kGrid = true;
+    static constexpr bool kJump = false;
+    Ctl *ctl;
+    int rank, size;
+    __device__ int tid() const { return rank * blockDim.x + threadIdx.x; }
+    __device__ int nthreads() const { return size * blockDim.x; }
+    __device__ int wid() const { return tid() >> 5; }
+    __device__ int nwarps() const { return nthreads() >> 5; }
+    __device__ int bid() const { return rank; }
+    __device__ int nblocks() const { return size; }
+    __device__ int srank() const { return (int)(threadIdx.x >> 5) * size + rank; }
+    __device__ bool leader() const { return rank == 0 && threadIdx.x == 0; }
+    static __device__ __forceinline__ void barrier() {
+        asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    }
+    __device__ bool sync() {
+        barrier();
+        const bool ok = ld_volatile(&ctl->err) == 0;
+        barrier();
+        return ok;
+    }
+    template <class F>
+    __device__ __forceinline__ bool sync_fetch(F fetch, int32_t *ok_slot) {
+        barrier();
+        if (threadIdx.x < 32) {
+            if (threadIdx.x == 0) *ok_slot = ld_volatile(&ctl->err);
+            fetch((int)threadIdx.x);
+        }
+        barrier();
+        return *ok_slot == 0;
+    }
+};
+
 struct BlockTeam {
     static constexpr bool kGrid = false;
+    static constexpr bool kJump = false;
     Ctl *ctl;
     __device__ int tid() const { return threadIdx.x; }
     __device__ int nthreads() const { return blockDim.x; }
@@ -3141,13 +3180,18 @@ __device__ void run_batch(Team &T, const GraphCtx &g, const BatchIn &in, int32_t
             if (!T.sync()) return;
             if (tr) tmark[nmark++] = global_ns();
         }
-        if (!g.jump && !ins_sort_candidates(T, g, sh_scan, sh_upmax)) return;
+        if (!(Team::kJump && g.jump) && !ins_sort_candidates(T, g, sh_scan, sh_upmax)) return;
         if (tr) {
             tmark[nmark++] = global_ns();
             trace_steps(g, tmark, nmark, -1);
         }
-        if (g.jump) ins_rounds_jump(T, g, sh_upmax, whist, sh_block);
-        else ins_rounds(T, g, sh_upmax, whist, stage_setup(sh_stage, stage_shift));
+        if constexpr (Team::kJump) {
+            if (g.jump) {
+                ins_rounds_jump(T, g, sh_upmax, whist, sh_block);
+                return;
+            }
+        }
+        ins_rounds(T, g, sh_upmax, whist, stage_setup(sh_stage, stage_shift));
     } else {
         if constexpr (!kRoundsOnly) {
             if (T.leader()) {

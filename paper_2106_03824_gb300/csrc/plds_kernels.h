@@ -14,9 +14,20 @@ struct SetItem {
     GraphCtx half[2];  // 0: insertion half, 1: deletion half
 };
 constexpr int kSetThreads = 256;
-constexpr int kSetStageShift = 3;
+constexpr int kSetStageShift = 1;
+constexpr int kSetCluster = 8;  // blocks per large graph
 
-__global__ void k_batch_set(const SetItem *items, int32_t count, int32_t *next);
+// A round's work: graphs items[0..large) for the clusters, items[large..count) for
+// single blocks; next[0] and next[1] are the two queues' heads, slot[c] the graph that
+// cluster c works on.
+struct SetQueue {
+    int32_t next[2];
+    int32_t large, count;
+    int32_t slot[1024];
+};
+
+__global__ void k_batch_set(const SetItem *items, SetQueue *q);
+__global__ void k_batch_set_cluster(const SetItem *items, SetQueue *q);
 
 // Serving form.
 enum : int32_t { kSlotFree = 0, kSlotReady = 1, kSlotDone = 2 };

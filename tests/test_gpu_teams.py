@@ -1,0 +1,75 @@
+"""The ways a batch's level phases are spread over the GPU, against the CPU oracle.
+
+A phase is run by one block alone (small lists), by the whole grid, or (batched form)
+by a block or a cluster of blocks; a batch passes from one to another as its lists
+grow and shrink.  Every quantity is an integer decided by exact arithmetic, so levels,
+counters and work counts must equal the oracle's after every batch.
+"""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2106_03824_gb300 import workloads as W
+from test_gpu_parity import P, assert_same, assert_stats  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+def _star_and_core(n, seed):
+    """Two hubs joined to half of the vertices each (tables of many chunks) over a random graph."""
+    rng = np.random.default_rng(seed)
+    leaves = rng.permutation(np.arange(2, n))[: n // 2]
+    hubs = np.stack([np.arange(leaves.size) % 2, leaves], 1)
+    e = np.concatenate([hubs, W.erdos_renyi(n, 4 * n, seed)]).astype(np.int32)
+    e = np.unique(np.sort(e, axis=1), axis=0)
+    return e[rng.permutation(e.shape[0])]
+
+
+GRAPHS = {
+    "power": lambda: (6_000, W.shuffled(W.chung_lu(6_000, 45_000, 2.2, seed=3), 4)),
+    "hubs": lambda: (5_000, _star_and_core(5_000, 5)),
+    "grid": lambda: (70 * 70, W.shuffled(W.grid2d(70, 0.1, seed=2), 6)),
+    "clique": lambda: (300, W.shuffled(W.erdos_renyi(300, 40_000, seed=8), 9)),
+}
+
+
+@pytest.mark.parametrize("name", sorted(GRAPHS))
+@pytest.mark.parametrize("sizes", [(1, 2, 31, 33, 257, 1000), (20_000, 1, 500, 7, 4_000), (513,)])
+def test_batches_of_uneven_size(P, name, sizes):  # noqa: F811
+    """Insertions from empty and deletions back, the batch sizes of `sizes` in turn
+    (at most 40 batches each way, the rest in one)."""
+    n, e = GRAPHS[name]()
+    g, o = P.PLDS(n), O.OraclePLDS(n)
+    for op in ("insert", "delete"):
+        rest = e if op == "insert" else W.shuffled(e, 17)
+        k = 0
+        while rest.shape[0]:
+            b = sizes[k % len(sizes)] if k < 40 else rest.shape[0]
+            part, rest = np.ascontiguousarray(rest[:b]), rest[b:]
+            getattr(g, op)(part)
+            assert getattr(o, op)(part) == 0
+            assert_same(g, o, f"{op} {k}")
+            assert_stats(g, o, f"{op} {k}")
+            k += 1
+    assert int(g.levels().max()) == 0
+    g.close()
+
+
+@pytest.mark.parametrize("ns", [(9_000,), (1, 2, 9_000, 40, 700), (4_000,) * 3 + (100,) * 60])
+def test_set_of_uneven_graphs(P, ns):  # noqa: F811
+    """A round's largest graphs go to clusters, the others to blocks: each equals the oracle."""
+    rng = np.random.default_rng(1)
+    edges = [W.shuffled(W.chung_lu(n, 9 * n, 2.3, seed=n), 1) if n > 2 else np.zeros((0, 2), np.int32) for n in ns]
+    S, orc = P.PLDSSet(list(ns)), [O.OraclePLDS(n) for n in ns]
+    for r in range(3):
+        halves = []
+        for e in edges:
+            m = e.shape[0]
+            ins = e[: int(m * (0.5, 0.8, 1.0)[r])]
+            dele = e[rng.permutation(m)[: m // 6]]
+            halves.append((ins, dele))
+        S.update(*S.pack(halves))
+        for g, o, (ins, dele) in zip(S.graphs, orc, halves):
+            assert o.insert(ins) == 0 and o.delete(dele) == 0
+            assert_same(g, o, f"round {r}, n={g.n}")
+    S.close()
