@@ -39,11 +39,13 @@ static int set_status(int s) {
 // Kernels
 // ---------------------------------------------------------------------------
 // The level rounds of one batch (after the step kernels below), one cooperative
-// launch: 152 blocks (one per SM) x 512 threads, grid barriers between rounds.
+// launch: 152 blocks (one per SM) x 512 threads, grid barriers between rounds.  One
+// kernel per kind of rounds (insertion, insertion by the jump variant, deletion).
+template <int kWhat>
 __global__ void __launch_bounds__(512) k_batch_grid(const __grid_constant__ GraphCtx g) {
     extern __shared__ int32_t sh[];
     GridTeam T{g.ctl, g.wait_limit_ns, g.barrier_sleep_ns};
-    run_batch<GridTeam, true>(T, g, BatchIn{g.edges, g.B, g.op, g.stamp_base}, sh, 0);
+    run_batch<GridTeam, true, kWhat>(T, g, BatchIn{g.edges, g.B, g.op, g.stamp_base}, sh, 0);
 }
 
 // The steps before the level rounds (preprocessing, table growth and shrinking,
@@ -114,10 +116,7 @@ __global__ void __launch_bounds__(kPreThreads) k_pre_apply_insert(const __grid_c
 __global__ void __launch_bounds__(kPreThreads) k_pre_apply_delete(const __grid_constant__ GraphCtx g) {
     if (ld_volatile(&g.ctl->err)) return;
     FreeTeam T;
-    if (T.leader()) {
-        g.ctl->nextmin[0] = kInf;
-        g.ctl->nextmin[1] = kInf;
-    }
+    if (T.leader()) del_reset(g.ctl);
     step_apply_delete(T, g);
 }
 
@@ -559,7 +558,7 @@ static void raise_smem_limit(K kernel, std::atomic<bool> (&done)[kAttrDevices], 
     if (device >= 0 && device < kAttrDevices) done[device].store(true, std::memory_order_release);
 }
 
-static std::atomic<bool> g_attr_batch[kAttrDevices];
+static std::atomic<bool> g_attr_batch[4][kAttrDevices];
 
 // The step kernels of one batch attempt, in stream order, then pre_done set so
 // that the cooperative kernel starts at the rounds.  Records ev0 before them and
@@ -609,15 +608,19 @@ static void undo_incoming(plds *h, const Ctl &c, const GraphCtx &g) {
 static int launch_batch(plds *h, const GraphCtx &g) {
     const int threads = block_threads(h);
     const size_t smem = smem_bytes(threads);
-    raise_smem_limit(k_batch_grid, g_attr_batch, h->device);
+    const int what = g.op == kOpDelete ? kDeleteRounds : g.jump ? kJumpRounds : kInsertRounds;
+    void (*kernel)(const GraphCtx) = what == kDeleteRounds ? k_batch_grid<kDeleteRounds>
+                                     : what == kJumpRounds ? k_batch_grid<kJumpRounds>
+                                                           : k_batch_grid<kInsertRounds>;
+    raise_smem_limit(kernel, g_attr_batch[what], h->device);
     int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch_grid, threads, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, smem);
     int per_sm = h->tune.blocks_per_sm > 0 ? std::min(h->tune.blocks_per_sm, occ) : 1;
     if (per_sm < 1) return PLDS_EDEVICE;
     dim3 grid(h->num_sms * per_sm), block(threads);
     void *args[] = {(void *)&g};
     if (!g.pre_done) cudaEventRecord(h->ev0, h->stream);
-    cudaError_t e = cudaLaunchCooperativeKernel((const void *)k_batch_grid, grid, block, args, smem, h->stream);
+    cudaError_t e = cudaLaunchCooperativeKernel((const void *)kernel, grid, block, args, smem, h->stream);
     cudaEventRecord(h->ev1, h->stream);
     h->launches++;
     if (e != cudaSuccess) {

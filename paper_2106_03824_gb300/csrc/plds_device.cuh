@@ -32,12 +32,37 @@ __device__ __forceinline__ int ld_volatile(const int32_t *p) { return *(volatile
 // ---------------------------------------------------------------------------
 // Teams
 // ---------------------------------------------------------------------------
+// Wait until the grid barrier has seen target arrivals (compared modulo 2^32), the
+// error word is set or limit_ns is over (then kErrTimeout is recorded).  A call of its
+// own: inlined it cost the rounds kernels registers around their scan loops.
+static __device__ __noinline__ void arrivals_wait(Ctl *ctl, uint32_t target, int64_t limit_ns, int32_t sleep_ns) {
+    volatile int32_t *errp = &ctl->err;
+    uint64_t t0 = 0;
+    unsigned spins = 0;
+    for (;;) {
+        unsigned long long v;
+        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(&ctl->bar_arrivals) : "memory");
+        if ((int32_t)((uint32_t)v - target) >= 0 || *errp != 0) break;
+        if ((++spins & 63u) == 0) {
+            const uint64_t now = global_ns();
+            if (t0 == 0) {
+                t0 = now;
+            } else if (now - t0 > (uint64_t)limit_ns) {
+                atomicOr(&ctl->err, kErrTimeout);
+                break;
+            }
+        }
+        if (sleep_ns) __nanosleep(sleep_ns);
+    }
+}
+
 struct GridTeam {
     static constexpr bool kGrid = true;  // barriers cost a round trip to L2: fetch at the barrier
     static constexpr bool kJump = true;  // may run the jump variant
     Ctl *ctl;
     int64_t limit_ns;
     int32_t sleep_ns;
+    uint32_t goal = 0;  // thread 0: arrivals that complete the last barrier (compared modulo 2^32)
     __device__ int tid() const { return blockIdx.x * blockDim.x + threadIdx.x; }
     __device__ int nthreads() const { return gridDim.x * blockDim.x; }
     __device__ int wid() const { return tid() >> 5; }
@@ -50,10 +75,10 @@ struct GridTeam {
     __device__ bool leader() const { return blockIdx.x == 0 && threadIdx.x == 0; }
     // Grid-wide barrier with a bounded wait: a block that waits longer than
     // limit_ns (or sees the error word set) records kErrTimeout and leaves.
-    // One 64-bit arrival counter, never reset: the k-th barrier is passed once
-    // the counter reaches (k+1) x blocks.  Thread 0 of each block arrives with a
-    // release add and polls with acquire loads; the block barriers around it
-    // carry the other threads' writes and reads.
+    // One 64-bit arrival counter, zero at launch and never reset: the k-th barrier
+    // is passed once the counter reaches (k+1) x blocks.  Thread 0 of each block
+    // arrives with a release add and polls with acquire loads; the block barriers
+    // around it carry the other threads' writes and reads.
     __device__ bool sync() {
         __syncthreads();
         if (threadIdx.x == 0) arrive_wait();
@@ -76,32 +101,27 @@ struct GridTeam {
         __syncthreads();
         return *ok_slot == 0;
     }
-    __device__ void arrive_wait() {
-        {
-            unsigned long long *cnt = &ctl->bar_arrivals;
-            unsigned long long a;
-            asm volatile("atom.add.release.gpu.global.u64 %0, [%1], 1;" : "=l"(a) : "l"(cnt) : "memory");
-            const unsigned long long target = (a / gridDim.x + 1) * (unsigned long long)gridDim.x;
-            volatile int32_t *errp = &ctl->err;
-            uint64_t t0 = 0;
-            unsigned spins = 0;
-            for (;;) {
-                unsigned long long v;
-                asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(cnt) : "memory");
-                if (v >= target || *errp != 0) break;
-                if ((++spins & 63u) == 0) {
-                    const uint64_t now = global_ns();
-                    if (t0 == 0) {
-                        t0 = now;
-                    } else if (now - t0 > (uint64_t)limit_ns) {
-                        atomicOr(&ctl->err, kErrTimeout);
-                        break;
-                    }
-                }
-                if (sleep_ns) __nanosleep(sleep_ns);
+    // One block went on alone while the others wait at the next barrier: once all of
+    // them have arrived there -- nobody still reads what the last barrier published --
+    // its thread 0 writes, then everybody passes the barrier.
+    template <class F>
+    __device__ __forceinline__ bool handoff(F write) {
+        if (blockIdx.x == 0) {
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                wait_for(goal + gridDim.x - 1);
+                write();
             }
         }
+        return sync();
     }
+    __device__ __forceinline__ void arrive_wait() {
+        goal += gridDim.x;
+        unsigned long long before;
+        asm volatile("atom.add.release.gpu.global.u64 %0, [%1], 1;" : "=l"(before) : "l"(&ctl->bar_arrivals) : "memory");
+        if (before != ~0ull) wait_for(goal);  // (polling only once the counter's old value is back)
+    }
+    __device__ __forceinline__ void wait_for(uint32_t target) { arrivals_wait(ctl, target, limit_ns, sleep_ns); }
 };
 
 // A thread-block cluster (hardware barrier; its blocks are always resident together).
@@ -128,6 +148,12 @@ struct ClusterTeam {
         const bool ok = ld_volatile(&ctl->err) == 0;
         barrier();
         return ok;
+    }
+    template <class F>
+    __device__ __forceinline__ bool handoff(F write) {  // as GridTeam's
+        barrier();
+        if (leader()) write();
+        return sync();
     }
     template <class F>
     __device__ __forceinline__ bool sync_fetch(F fetch, int32_t *ok_slot) {
@@ -377,7 +403,7 @@ inline __device__ int block_exclusive(int x, int *sh32, int *total) {
 // Steps A2+A3 (insert): put both directions into the tables and update deg, up
 // (other endpoint on a level >= own) and up* (other endpoint on a level >= own-1).
 template <class Team>
-__device__ void step_apply_insert(Team &T, const GraphCtx &g) {
+__device__ __forceinline__ void step_apply_insert(Team &T, const GraphCtx &g) {
     const int64_t V = (int64_t)g.ctl->vcount;
     for (int64_t i = T.tid(); i < V; i += T.nthreads()) {
         unsigned long long key = g.vkeys[i];
@@ -397,9 +423,14 @@ __device__ void step_apply_insert(Team &T, const GraphCtx &g) {
     }
 }
 
+// What a deletion batch's rounds start from (besides zeroed control words).
+__device__ __forceinline__ void del_reset(Ctl *c) {
+    c->nextmin[0] = c->nextmin[1] = c->qmin[0] = c->qmin[1] = kInf;
+}
+
 // Steps A2+A3 (delete): tombstone both directions, decrement the counters.
 template <class Team>
-__device__ void step_apply_delete(Team &T, const GraphCtx &g) {
+__device__ __forceinline__ void step_apply_delete(Team &T, const GraphCtx &g) {
     const int64_t V = (int64_t)g.ctl->vcount;
     for (int64_t i = T.tid(); i < V; i += T.nthreads()) {
         unsigned long long key = g.vkeys[i];
@@ -497,7 +528,7 @@ __device__ C block_reserve(C *cnt, C amount, C *sh) {
 // Step A1: canonicalise + validate.  Drops self-loops, keys each edge as
 // (min,max), keeps one copy of each key (batch hash set), flags ids outside [0,n).
 template <class Team>
-__device__ void pre_canon(Team &T, const GraphCtx &g, const BatchIn &in, unsigned long long *sh) {
+__device__ __forceinline__ void pre_canon(Team &T, const GraphCtx &g, const BatchIn &in, unsigned long long *sh) {
     const int2 *e = reinterpret_cast<const int2 *>(in.edges);
     unsigned long long loops = 0;
     const int64_t mask = g.hcap - 1, stride = (int64_t)T.nblocks() * blockDim.x;
@@ -534,7 +565,7 @@ __device__ void pre_canon(Team &T, const GraphCtx &g, const BatchIn &in, unsigne
 // collect the touched endpoints (deduplicated by stamp) and, for insertions, the
 // number of incoming edges per endpoint.
 template <class Team>
-__device__ void pre_filter(Team &T, const GraphCtx &g, const BatchIn &in, unsigned long long *sh) {
+__device__ __forceinline__ void pre_filter(Team &T, const GraphCtx &g, const BatchIn &in, unsigned long long *sh) {
     const int64_t U = (int64_t)g.ctl->ucount, stride = (int64_t)T.nblocks() * blockDim.x;
     const int32_t stouch = in.stamp_base;
     unsigned long long filtered = 0;
@@ -574,7 +605,7 @@ __device__ void pre_filter(Team &T, const GraphCtx &g, const BatchIn &in, unsign
 // stops the steps after this one; the incoming counts that valid keys left behind
 // are then cleared (k_undo_inc) before the call reports the error.
 template <class Team>
-__device__ void pre_canon_filter(Team &T, const GraphCtx &g, const BatchIn &in, unsigned long long *sh) {
+__device__ __forceinline__ void pre_canon_filter(Team &T, const GraphCtx &g, const BatchIn &in, unsigned long long *sh) {
     const int2 *e = reinterpret_cast<const int2 *>(in.edges);
     const int32_t stouch = in.stamp_base;
     unsigned long long loops = 0, filtered = 0;
@@ -633,7 +664,7 @@ __device__ void pre_canon_filter(Team &T, const GraphCtx &g, const BatchIn &in, 
 // list them (M[0] = {x, new size}) and total their sizes.  Run after pre_filter;
 // tcount is taken from its touched total.
 template <class Team>
-__device__ void pre_grow_request(Team &T, const GraphCtx &g, unsigned long long *sh) {
+__device__ __forceinline__ void pre_grow_request(Team &T, const GraphCtx &g, unsigned long long *sh) {
     const int32_t tc = (int32_t)g.ctl->ttotal;
     const int64_t stride = (int64_t)T.nblocks() * blockDim.x;
     if (T.leader()) g.ctl->tcount = tc;
@@ -660,7 +691,7 @@ __device__ void pre_grow_request(Team &T, const GraphCtx &g, unsigned long long 
 // take the growing tables, the batch's incoming counts are undone and the host
 // grows the pool and runs the batch again.
 template <class Team>
-__device__ void pre_pool_check(Team &T, const GraphCtx &g) {
+__device__ __forceinline__ void pre_pool_check(Team &T, const GraphCtx &g) {
     const unsigned long long top = *g.pool_top;
     if (top + g.ctl->grow_total <= (unsigned long long)g.pool_cap) {
         if (T.leader()) g.ctl->pool_old = top;  // the new tables will fill [top, top + grow_total)
@@ -678,7 +709,7 @@ constexpr int kGrowChunk = 512;  // shrinking: slots per chunk item
 constexpr int kMoveChunk = 128;  // growth: old slots per chunk item (one 16-byte group per lane)
 
 template <class Team>
-__device__ void pre_alloc(Team &T, const GraphCtx &g, unsigned long long *sh) {
+__device__ __forceinline__ void pre_alloc(Team &T, const GraphCtx &g, unsigned long long *sh) {
     const int64_t gc = (int64_t)g.ctl->gtotal, stride = (int64_t)T.nblocks() * blockDim.x;
     for (int64_t b0 = (int64_t)T.bid() * blockDim.x; b0 < gc; b0 += stride) {
         const int64_t i = b0 + threadIdx.x;
@@ -699,7 +730,7 @@ __device__ void pre_alloc(Team &T, const GraphCtx &g, unsigned long long *sh) {
 
 // Every new table starts empty: one fill of the contiguous rooms.
 template <class Team>
-__device__ void pre_clear(Team &T, const GraphCtx &g) {
+__device__ __forceinline__ void pre_clear(Team &T, const GraphCtx &g) {
     int4 *p = reinterpret_cast<int4 *>(g.slots + g.ctl->pool_old);
     const int64_t n4 = (int64_t)(g.ctl->grow_total >> 2);
     for (int64_t j = T.tid(); j < n4; j += T.nthreads()) p[j] = empty4();
@@ -709,7 +740,7 @@ __device__ void pre_clear(Team &T, const GraphCtx &g) {
 // hub's table is spread over many warps).  The vertices still point at their old
 // tables; pre_commit repoints them afterwards.
 template <class Team>
-__device__ void pre_grow(Team &T, const GraphCtx &g) {
+__device__ __forceinline__ void pre_grow(Team &T, const GraphCtx &g) {
     const int64_t nc_items = (int64_t)g.ctl->ctotal;
     for (int64_t c = T.wid(); c < nc_items; c += T.nwarps()) {
         const int4 ci = g.CL[0][c];
@@ -730,7 +761,7 @@ __device__ void pre_grow(Team &T, const GraphCtx &g) {
 
 // Every growing vertex points at its new table.
 template <class Team>
-__device__ void pre_commit(Team &T, const GraphCtx &g) {
+__device__ __forceinline__ void pre_commit(Team &T, const GraphCtx &g) {
     const int64_t gc = (int64_t)g.ctl->gtotal;
     for (int64_t i = T.tid(); i < gc; i += T.nthreads()) {
         const int4 it = g.M[0][i];
@@ -751,7 +782,7 @@ __device__ __forceinline__ void shrink_item(const GraphCtx &g, int list, unsigne
 // live keys}, whose rebuild is cut into chunks; speed only, skipped when the
 // arena is full.
 template <class Team>
-__device__ void pre_shrink_plan(Team &T, const GraphCtx &g, unsigned long long *sh) {
+__device__ __forceinline__ void pre_shrink_plan(Team &T, const GraphCtx &g, unsigned long long *sh) {
     const int32_t tc = (int32_t)g.ctl->ttotal;
     const int64_t stride = (int64_t)T.nblocks() * blockDim.x;
     if (T.leader()) g.ctl->tcount = tc;
@@ -797,7 +828,7 @@ __device__ void pre_shrink_plan(Team &T, const GraphCtx &g, unsigned long long *
 // Shrink, first pass: the small tables rebuilt whole, one warp each; the large
 // tables' live keys copied into their arena room, one warp per chunk of slots.
 template <class Team>
-__device__ void pre_shrink_a(Team &T, const GraphCtx &g) {
+__device__ __forceinline__ void pre_shrink_a(Team &T, const GraphCtx &g) {
     const int32_t sc = (int32_t)g.ctl->gtotal;
     for (int i = T.wid(); i < sc; i += T.nwarps()) {
         const int4 it = g.M[0][i];
@@ -838,7 +869,7 @@ __device__ void pre_shrink_a(Team &T, const GraphCtx &g) {
 // cleared (its first nc slots) and takes its new size; otherwise it is reported
 // and kept.
 template <class Team>
-__device__ void pre_shrink_b(Team &T, const GraphCtx &g) {
+__device__ __forceinline__ void pre_shrink_b(Team &T, const GraphCtx &g) {
     const int64_t n1 = (int64_t)g.ctl->c1total;
     for (int64_t c = T.wid(); c < n1; c += T.nwarps()) {
         const int4 ci = g.CL[1][c];
@@ -860,7 +891,7 @@ __device__ void pre_shrink_b(Team &T, const GraphCtx &g) {
 // Shrink, third pass: the copied keys go back into the cleared tables, one warp
 // per chunk of keys.
 template <class Team>
-__device__ void pre_shrink_c(Team &T, const GraphCtx &g) {
+__device__ __forceinline__ void pre_shrink_c(Team &T, const GraphCtx &g) {
     const int64_t n2 = (int64_t)g.ctl->c2total;
     for (int64_t c = T.wid(); c < n2; c += T.nwarps()) {
         const int4 ci = g.CL[2][c];
@@ -980,10 +1011,12 @@ constexpr int kStageF = 2048, kStageTL = 1024, kStageCL = 2048, kStagePK = 1024;
 // fetches for the next phase while it passes the team barrier (ph4: one item per
 // warp; phs: words).
 struct RoundStage {
-    Stage<int32_t> f;
+    Stage<int32_t> f, q;      // q shares tl's buffer (f's while tl fills)
     Stage<int4> tl, cl, pk;
     int32_t *movers;  // shared mover count of the block
-    int32_t *bmin;    // shared minimum pending level of the block
+    int32_t *bmin;    // shared minimum pending level of the block's near entries
+    int32_t *qmin;    // and of its far vertices
+    int32_t *rb;      // count of the listed vertices with large tables
     int32_t *tmp;
     int4 *ph4;
     int32_t *phs;
@@ -1013,13 +1046,17 @@ __device__ __forceinline__ RoundStage stage_setup(int32_t *base, int shift) {
     st.tl.hdr = hdr + 2;
     st.cl.hdr = hdr + 4;
     st.pk.hdr = hdr + 6;
+    st.q.buf = reinterpret_cast<int32_t *>(st.tl.buf);
+    st.q.hdr = hdr + 22;
+    st.q.cap = min(cf, 4 * ct);
+    st.qmin = hdr + 24;
     st.f.cap = cf;
     st.tl.cap = ct;
     st.cl.cap = cc;
     st.pk.cap = cp;
     st.movers = hdr + 8;
     st.bmin = hdr + 9;
-    st.tmp = hdr + 10;  // 4 ints
+    st.tmp = hdr + 10;  // 4 ints (a list's fifth: hdr[25])
     st.ff = hdr + 14;   // 3 ints
     st.ff64 = reinterpret_cast<unsigned long long *>(hdr + 18);  // 2 x 64 bit
     if (threadIdx.x == 0) {
@@ -1029,6 +1066,7 @@ __device__ __forceinline__ RoundStage stage_setup(int32_t *base, int shift) {
         hdr[6] = 0; hdr[7] = cp;
         hdr[8] = 0; hdr[9] = kInf;
         hdr[14] = 0; hdr[15] = kInf; hdr[16] = kInf;
+        hdr[22] = 0; hdr[23] = st.q.cap; hdr[24] = kInf;
         st.ff64[0] = 0;
         st.ff64[1] = 0;
     }
@@ -1042,8 +1080,8 @@ __device__ __forceinline__ void stage_init(int32_t *hdr, int cap) {
     hdr[1] = cap;
 }
 
-// Publish the selected lists of a phase (bit 0 f, 1 tl, 2 cl, 3 pk) together:
-// warp k reserves list k's global range, then the block copies all of them.
+// Publish the selected lists of a phase (bit 0 f, 1 tl, 2 cl, 3 pk, 4 q) together:
+// warp k (q: warp 0) reserves list k's global range, then the block copies all of them.
 // The headers are reset at the end; the next use comes after a team barrier.
 template <class V>
 __device__ __forceinline__ void stage_reserve_global(const GraphCtx &g, const Stage<V> &s, int32_t *base_out) {
@@ -1068,18 +1106,21 @@ __device__ __forceinline__ void stage_flush_round(const GraphCtx &g, const Round
         if (w == 1 && (which & 2u)) stage_reserve_global(g, st.tl, st.tmp + 1);
         if (w == 2 && (which & 4u)) stage_reserve_global(g, st.cl, st.tmp + 2);
         if (w == 3 && (which & 8u)) stage_reserve_global(g, st.pk, st.tmp + 3);
+        if (w == 0 && (which & 16u)) stage_reserve_global(g, st.q, st.tmp + 15);
     }
     __syncthreads();
     if (which & 1u) stage_copy_out(st.f, st.tmp[0]);
     if (which & 2u) stage_copy_out(st.tl, st.tmp[1]);
     if (which & 4u) stage_copy_out(st.cl, st.tmp[2]);
     if (which & 8u) stage_copy_out(st.pk, st.tmp[3]);
+    if (which & 16u) stage_copy_out(st.q, st.tmp[15]);
     __syncthreads();
     if (threadIdx.x == 0) {
         if (which & 1u) { st.f.hdr[0] = 0; st.f.hdr[1] = st.f.cap; }
         if (which & 2u) { st.tl.hdr[0] = 0; st.tl.hdr[1] = st.tl.cap; }
         if (which & 4u) { st.cl.hdr[0] = 0; st.cl.hdr[1] = st.cl.cap; }
         if (which & 8u) { st.pk.hdr[0] = 0; st.pk.hdr[1] = st.pk.cap; }
+        if (which & 16u) { st.q.hdr[0] = 0; st.q.hdr[1] = st.q.cap; }
     }
 }
 
@@ -1095,14 +1136,24 @@ __device__ __forceinline__ void enqueue_mover(const GraphCtx &g, const RoundStag
     const bool small = is_mover && c <= g.thread_max_cap;
     stage_push(st.tl, small, make_int4(v, lg, goff, aux));
     const int nch = (is_mover && !small) ? (c + kChunk - 1) / kChunk : 0;
-    int tot;
-    const int ex = warp_exclusive(nch, &tot);
+    const unsigned one = __ballot_sync(kFull, nch == 1);
+    int tot, ex;
+    if (!__any_sync(kFull, nch > 1)) {  // at most one item a lane: no need to spread them
+        tot = __popc(one);
+        ex = __popc(one & ((1u << lane) - 1u));
+    } else {
+        ex = warp_exclusive(nch, &tot);
+    }
     if (tot == 0) return;
     int pos = 0;
     bool sh = false;
     if (lane == 0) pos = stage_reserve(st.cl, tot, sh);
     pos = __shfl_sync(kFull, pos, 0);
     sh = __shfl_sync(kFull, sh, 0);
+    if (tot == __popc(one)) {
+        if (nch) stage_put(st.cl, sh, pos + ex, make_int4(v, lg, goff, aux));
+        return;
+    }
     // the warp writes all its chunk items together (a large table has many)
     wsm[lane] = ex;
     wsm[32 + lane] = v;
@@ -1204,7 +1255,7 @@ __device__ __forceinline__ void enqueue_ins(const GraphCtx &g, const RoundStage 
 // takes it past the cutoff.  (Listing every touched vertex made nearly every level
 // an initial-candidate level, which ended the runs of pure rounds there.)
 template <class Team>
-__device__ bool ins_sort_candidates(Team &T, const GraphCtx &g, int *sh, const int32_t *sh_upmax) {
+__device__ __forceinline__ bool ins_sort_candidates(Team &T, const GraphCtx &g, int *sh, const int32_t *sh_upmax) {
     const int32_t tc = g.ctl->tcount;
     const int64_t stride = (int64_t)T.nblocks() * blockDim.x;
     int32_t *cand = g.R[0];
@@ -1398,6 +1449,7 @@ __device__ __forceinline__ void enqueue_marked(const GraphCtx &g, const RoundSta
 // scratch, after the 160 ints enqueue_mover uses) and are queued 32 at a time, so
 // their table lookups are issued together.
 constexpr int kMarkCap = 256;
+constexpr int kTotalsAt = 160 + kMarkCap;  // a warp's totals: 6 x 64 bit of its kWarpHist ints
 
 __device__ __forceinline__ void marks_flush(const GraphCtx &g, const RoundStage &st, int32_t *mbuf, int &mc,
                                             int k1, int32_t *wsm) {
@@ -1437,7 +1489,7 @@ __device__ __forceinline__ void marks_add(const GraphCtx &g, const RoundStage &s
 // Test the initial candidates S[s_lo, s_hi) on level L against Invariant 1 (warp
 // ranks rotated by rot, so that a small test runs on other warps than a scan).
 template <class Team>
-__device__ void ins_test_initial(Team &T, const GraphCtx &g, const RoundStage &st, int32_t s_lo, int32_t s_hi,
+__device__ __forceinline__ void ins_test_initial(Team &T, const GraphCtx &g, const RoundStage &st, int32_t s_lo, int32_t s_hi,
                                  int32_t L, int32_t cut, int32_t *wsm, int rot, int k1) {
     const int32_t fl = phase_flag(k1);
     const int rank = (T.srank() + rot) % T.nwarps();
@@ -1466,11 +1518,55 @@ struct InsState {
     bool done = false;
 };
 
-// One thread's share of the batch's statistics.
-struct InsCount {
-    unsigned long long visits = 0, scanned = 0, upv = 0;
+// The statistics a thread gathers; when one comes near 32 bits, and at the end of the
+// batch, the warp's sums go to the warp's own totals in shared memory (after its
+// scratch and its buffer of marks).
+struct ScanCount {
+    unsigned visits = 0, scanned = 0, upv = 0;
     unsigned aff = 0;  // neighbours whose counters a move changed
+    unsigned evals = 0, evisits = 0;
 };
+
+__device__ __forceinline__ unsigned long long *warp_totals(int32_t *wsm) {
+    return reinterpret_cast<unsigned long long *>(wsm + kTotalsAt);
+}
+
+__device__ __forceinline__ void totals_clear(int32_t *wsm) {
+    if (lane_id() < 6) warp_totals(wsm)[lane_id()] = 0;
+    __syncwarp();
+}
+
+__device__ __forceinline__ void totals_add(int32_t *wsm, const ScanCount &a, bool ins) {
+    const unsigned long long v = warp_total(a.visits), c = warp_total(a.scanned), f = warp_total(a.aff);
+    const unsigned long long u = warp_total(ins ? a.upv : a.evals), e = ins ? 0ull : warp_total(a.evisits);
+    if (lane_id() == 0) {
+        unsigned long long *t = warp_totals(wsm);
+        t[0] += v;
+        t[1] += c;
+        t[2] += f;
+        t[3] += u;
+        t[4] += e;
+    }
+}
+
+// After each phase or round (all lanes of a warp call).
+__device__ __forceinline__ void totals_keep(int32_t *wsm, ScanCount &a, bool ins) {
+    if (__any_sync(kFull, (a.visits | a.scanned | a.upv | a.aff | a.evisits) >> 30)) {
+        totals_add(wsm, a, ins);
+        a = ScanCount{};
+    }
+}
+
+__device__ __forceinline__ void totals_flush(const GraphCtx &g, int32_t *wsm, const ScanCount &a, bool ins) {
+    totals_add(wsm, a, ins);
+    __syncwarp();
+    if (lane_id() < 5) {
+        const unsigned long long x = warp_totals(wsm)[lane_id()];
+        const int to = lane_id() == 0 ? kStVisits : lane_id() == 1 ? kStSlotsScanned : lane_id() == 2 ? kStAffected
+                       : lane_id() == 3 ? (ins ? kStUpVisits : kStDlEvals) : kStDlVisits;
+        if (x) atomicAdd(&g.ctl->st[to], x);
+    }
+}
 
 // After a phase whose movers all climb on to level l and nobody else does: how many
 // pure rounds lie ahead (lowc: kInf minus the lowest level of a neighbour that is
@@ -1494,7 +1590,7 @@ __device__ __forceinline__ int32_t ins_pure_rounds(const GraphCtx &g, const int3
 template <int U, class Team>
 __device__ __forceinline__ void ins_scan_chunks(Team &T, const GraphCtx &g, const RoundStage &st, int32_t *wsm,
                                                 int32_t *mbuf, int &mc, const InsState &s, int32_t cut_next,
-                                                const int4 *cl, int32_t &low, InsCount &a) {
+                                                const int4 *cl, int32_t &low, ScanCount &a) {
     const int lane = lane_id();
     const int32_t l = s.l, k = s.k, clc = s.clc;
     const int32_t fcur = phase_flag(k), fnext = phase_flag(k + 1);
@@ -1625,7 +1721,7 @@ __device__ __forceinline__ void ins_scan_chunks(Team &T, const GraphCtx &g, cons
 template <class Team>
 __device__ __forceinline__ void ins_phase_work(Team &T, const GraphCtx &g, const RoundStage &st,
                                                const int32_t *sh_upmax, int32_t *wsm, const InsState &s, int32_t s_lo,
-                                               int32_t s_hi, const int4 *tl, const int4 *cl, InsCount &a) {
+                                               int32_t s_hi, const int4 *tl, const int4 *cl, ScanCount &a) {
     const int lane = lane_id();
     const int32_t l = s.l, k = s.k, tlc = s.tlc;
     if (!s.scan) {
@@ -1664,7 +1760,7 @@ __device__ __forceinline__ void ins_phase_work(Team &T, const GraphCtx &g, const
             for (int q = 0; q < 16; ++q) ideg += ws[q] >= 0;
             ins_effects(g, ws, lv, l, s.lmo, fcur, fnext, cut_next, c4, low, push, keep, a.aff);
             cnt_l += c4[0] + c4[1] + c4[2] + c4[3];
-            a.scanned += 4 * (unsigned long long)max(0, min(4, ng - j0));
+            a.scanned += 4 * max(0, min(4, ng - j0));
             marks_add(g, st, push, ws, mbuf, mc, k + 1, wsm);
         }
         a.visits += ideg;
@@ -1678,6 +1774,7 @@ __device__ __forceinline__ void ins_phase_work(Team &T, const GraphCtx &g, const
     marks_flush(g, st, mbuf, mc, k + 1, wsm);
     low = (int32_t)__reduce_min_sync(kFull, (unsigned)low);
     if (lane == 0 && low < kInf) atomicMin(&st.ff[2], low);
+    totals_keep(wsm, a, true);
 }
 
 // The state after a phase that left nm movers for the next one, of which ncont
@@ -1763,9 +1860,9 @@ __device__ __forceinline__ void ins_trace(const GraphCtx &g, const InsState &bef
 constexpr int kSoloCl = 96, kSoloTl = 512;  // largest lists of a phase that one block runs alone
 
 template <bool kLimit>
-__device__ bool ins_phases_local(const GraphCtx &g, const int32_t *sh_upmax, int32_t *wsm, RoundStage st,
+__device__ __forceinline__ bool ins_phases_local(const GraphCtx &g, const int32_t *sh_upmax, int32_t *wsm, RoundStage st,
                                  InsState &s, int32_t s_lo, int32_t s_hi, const int4 *tl, const int4 *cl,
-                                 InsCount &a) {
+                                 ScanCount &a) {
     BlockTeam T{g.ctl};
     int32_t *sets = reinterpret_cast<int32_t *>(st.ph4);  // 3 sets of 16 ints
     int4 *const tbuf[2] = {st.tl.buf, st.pk.buf};
@@ -1872,7 +1969,7 @@ __device__ bool ins_phases_local(const GraphCtx &g, const int32_t *sh_upmax, int
 template <class Team>
 __device__ __forceinline__ bool ins_grid_phase(Team &T, const GraphCtx &g, const int32_t *sh_upmax, int32_t *wsm,
                                                RoundStage &st, InsState &s, int32_t nlev, int32_t &s_lo,
-                                               int32_t &s_hi, InsCount &a) {
+                                               int32_t &s_hi, ScanCount &a) {
     if ((s.scan && s.l >= g.K - 1) || s.k > 2 * g.K + 4) {  // the top group is never violated
         if (T.leader()) report(g, kErrInternal, 5, s.l, s.k, 0);
         return false;
@@ -1987,8 +2084,7 @@ __device__ __forceinline__ bool ins_grid_phase(Team &T, const GraphCtx &g, const
 }
 
 template <class Team>
-__device__ bool ins_rounds(Team &T, const GraphCtx &g, const int32_t *sh_upmax, int32_t *wsm, RoundStage st) {
-    InsCount a;
+__device__ __forceinline__ bool ins_rounds(Team &T, const GraphCtx &g, const int32_t *sh_upmax, int32_t *wsm, RoundStage st) {
     const int32_t nlev = g.ctl->nlev;
     if (nlev == 0) return true;  // nobody violates: nothing moves, no flag to clear
     InsState s;
@@ -1997,6 +2093,8 @@ __device__ bool ins_rounds(Team &T, const GraphCtx &g, const int32_t *sh_upmax, 
     s.ninit = nlev > 1 ? g.levlist[1] : kInf;
     int32_t s_lo, s_hi;
     ins_initial_range(g, s, s_lo, s_hi);
+    ScanCount a;
+    totals_clear(wsm);
     if constexpr (!Team::kGrid) {
         if (!ins_phases_local<false>(g, sh_upmax, wsm, st, s, s_lo, s_hi, nullptr, nullptr, a)) return false;
     } else {
@@ -2007,19 +2105,22 @@ __device__ bool ins_rounds(Team &T, const GraphCtx &g, const int32_t *sh_upmax, 
                 if (T.bid() == 0) {
                     const int cur = s.k % 3;
                     ins_phases_local<true>(g, sh_upmax, wsm, st, s, s_lo, s_hi, g.TL[cur], g.CL[cur], a);
-                    if (threadIdx.x == 0) {
+                    if (threadIdx.x == 0) {  // (read by the others only after the handoff)
                         int32_t *o = g.ctl->solo;
                         o[0] = s.k; o[1] = s.l; o[2] = s.lmo; o[3] = s.spos;
                         o[4] = s.m; o[5] = s.tlc; o[6] = s.clc; o[7] = (s.done ? 1 : 0) | (s.scan ? 2 : 0);
-                        for (int i = 0; i < 3; ++i) {  // the grid's counters start clean
-                            g.ctl->itl[i] = g.ctl->icl[i] = g.ctl->imcnt[i] = g.ctl->icont[i] = 0;
-                            g.ctl->iminup_c[i] = g.ctl->ilow_c[i] = 0;
-                            g.ctl->isdeg[i] = g.ctl->isup[i] = 0;
-                            g.ctl->ltop[i] = 0;
-                        }
                     }
                 }
-                if (!T.sync()) return false;
+                const bool fin = s.done;
+                const bool ok = T.handoff([&g, fin] {
+                    for (int i = 0; i < 3 && !fin; ++i) {  // the grid's counters start clean
+                        g.ctl->itl[i] = g.ctl->icl[i] = g.ctl->imcnt[i] = g.ctl->icont[i] = 0;
+                        g.ctl->iminup_c[i] = g.ctl->ilow_c[i] = 0;
+                        g.ctl->isdeg[i] = g.ctl->isup[i] = 0;
+                        g.ctl->ltop[i] = 0;
+                    }
+                });
+                if (!ok) return false;
                 const int32_t *o = g.ctl->solo;
                 const int32_t fl = ld_volatile(o + 7);
                 s.k = ld_volatile(o); s.l = ld_volatile(o + 1); s.lmo = ld_volatile(o + 2); s.spos = ld_volatile(o + 3);
@@ -2042,16 +2143,7 @@ __device__ bool ins_rounds(Team &T, const GraphCtx &g, const int32_t *sh_upmax, 
         const int32_t raw = g.level[v];
         if (raw & ~kLevelMask) g.level[v] = raw & kLevelMask;
     }
-    a.visits = warp_sum64(a.visits);
-    a.scanned = warp_sum64(a.scanned);
-    a.upv = warp_sum64(a.upv);
-    const unsigned long long affs = warp_sum64(a.aff);
-    if (lane_id() == 0) {
-        atomicAdd(&g.ctl->st[kStVisits], a.visits);
-        atomicAdd(&g.ctl->st[kStSlotsScanned], a.scanned);
-        atomicAdd(&g.ctl->st[kStUpVisits], a.upv);
-        if (affs) atomicAdd(&g.ctl->st[kStAffected], affs);
-    }
+    totals_flush(g, wsm, a, true);
     return T.sync();
 }
 
@@ -2371,89 +2463,6 @@ __device__ __forceinline__ int32_t thread_desire_level(const GraphCtx &g, int32_
     return lo + 1;
 }
 
-// A desire-level d computed for w (slack sl): recorded, and a pending entry in
-// P[q] unless it equals w's current pending level.
-__device__ __forceinline__ void dl_record(const GraphCtx &g, int32_t w, int32_t d, int32_t sl, int q, int32_t lmin,
-                                          int site) {
-    g.dslack[w] = sl;
-    if (d <= lmin) {
-        report(g, kErrInternal, site, w, d, lmin);
-    } else if (d != g.dlv[w]) {
-        g.dlv[w] = d;
-        const int pos = atomicAdd(&g.ctl->pcnt[q], 1);
-        g.P[q][pos] = make_int4(w, d, 0, 0);
-        atomicMin(&g.ctl->nextmin[q], d);
-    }
-}
-
-// Desire-levels for every vertex of src[0..count) that violates Invariant 2
-// (level > 0 and up* < dnmin[gn(level-1)]).  Two phases with a team barrier:
-// classify into a warp list (small tables, from the front of RL) and a block list
-// (large tables, from the back), then compute.  A result d becomes a pending
-// entry in P[q] unless it equals the vertex's current pending level; results at
-// or below lmin contradict the level lemma and are reported.  A pending vertex
-// whose slack has not gone below 0 since its last evaluation would get the same
-// answer again: that evaluation is counted (Algorithm 3 counts every evaluation)
-// without the scan.
-template <class Team>
-__device__ bool dl_batch(Team &T, const GraphCtx &g, const int32_t *src, int32_t count, int q, int32_t lmin,
-                         const int32_t *sh_dnmin, int32_t *whist, int32_t *bhist, unsigned long long &evals,
-                         unsigned long long &evisits) {
-    const int lane = lane_id();
-    int32_t *RL = g.R[1];
-    for (int i0 = T.srank() * 32; i0 < count; i0 += T.nwarps() * 32) {
-        const int i = i0 + lane;
-        bool viol = false, big = false;
-        int32_t w = 0;
-        if (i < count) {
-            w = src[i];
-            const int32_t lw = g.level[w], us = g.upstar[w], c = g.cap[w], dv = g.dlv[w];
-            viol = lw > 0 && us < sh_dnmin[(lw - 1) / g.Lg];
-            big = c > g.block_cap;
-            if (viol && dv >= 0 && g.dslack[w] >= 0) {  // same answer as last time: counted only
-                viol = false;
-                evals++;
-                evisits += g.deg[w];
-            }
-            if (viol && c <= kThreadDl) {  // a small table: this thread computes it
-                viol = false;
-                int32_t sl;
-                const int32_t d = thread_desire_level(g, w, lw, c, sh_dnmin, &sl);
-                evals++;
-                evisits += g.deg[w];
-                dl_record(g, w, d, sl, q, lmin, 10);
-            }
-        }
-        const int pw = warp_append(&g.ctl->rcnt[1], viol && !big);
-        if (viol && !big) RL[pw] = w;
-        const int pb = warp_append(&g.ctl->rbcnt, viol && big);
-        if (viol && big) RL[g.n - 1 - pb] = w;
-    }
-    if (!T.sync()) return false;
-    const int32_t nw = g.ctl->rcnt[1], nb = g.ctl->rbcnt;
-    for (int i = T.srank(); i < nw; i += T.nwarps()) {
-        const int32_t w = RL[i], lw = g.level[w];
-        int32_t sl;
-        const int32_t d = warp_desire_level(g, w, lw, sh_dnmin, whist, &sl);
-        if (lane == 0) {
-            evals++;
-            evisits += g.deg[w];
-            dl_record(g, w, d, sl, q, lmin, 8);
-        }
-    }
-    for (int i = T.bid(); i < nb; i += (T.nthreads() / blockDim.x)) {
-        const int32_t w = RL[g.n - 1 - i], lw = g.level[w];
-        int32_t sl;
-        const int32_t d = block_desire_level(g, w, lw, sh_dnmin, bhist, bhist + kWarpHist, &sl);
-        if (threadIdx.x == 0) {
-            evals++;
-            evisits += g.deg[w];
-            dl_record(g, w, d, sl, q, lmin, 9);
-        }
-    }
-    return true;
-}
-
 // ---------------------------------------------------------------------------
 // Step A6: deletion rounds (Algorithm 3).
 // ---------------------------------------------------------------------------
@@ -2484,220 +2493,736 @@ __device__ __forceinline__ void del_slack(const GraphCtx &g, int32_t w, int32_t 
     if (l < xs && xs <= pv) atomicSub(&g.dslack[w], 1);
 }
 
+// A desire-level d computed for w (slack sl, pending level dv so far) is recorded.
+// Returns where the vertex has to be listed: 1 among the near entries (d within the
+// current window), 2 among the far vertices, 3 nowhere new but its far level fell, 0
+// nowhere.  (While neighbours only move down a pending level never rises, so a vertex
+// becomes far from here at most once.)
+__device__ __forceinline__ int del_settle(const GraphCtx &g, int32_t w, int32_t d, int32_t sl, int32_t dv, int32_t l,
+                                          int32_t limit, int site) {
+    g.dslack[w] = sl;
+    if (d <= l) {
+        report(g, kErrInternal, site, w, d, l);
+        return 0;
+    }
+    if (d == dv) return 0;
+    g.dlv[w] = d;
+    return d <= limit ? 1 : dv > limit ? 3 : 2;
+}
+
+// Every lane of a warp: list the vertices settled above and keep the lists' minima.
+__device__ __forceinline__ void del_list(const RoundStage &st, int where, int32_t w, int32_t d) {
+    stage_push(st.pk, where == 1, make_int4(w, d, 0, 0));
+    stage_push(st.q, where == 2, w);
+    if (where == 1) atomicMin(st.bmin, d);
+    if (where >= 2) atomicMin(st.qmin, d);
+}
+
+// Where the deletion rounds stand (the same in every thread of the team).  Pending
+// vertices lie in two lists: near entries {v, level} with levels up to limit, one list
+// per round parity, scanned every round; and far vertices (their levels in dlv, above
+// limit), scanned only when the near list is used up and the window moves on.  The
+// window starts wide open; it narrows when rounds that one block could run follow one
+// another only because the near list is too long for it (a road-like graph: thousands of
+// pending vertices, a few on each level).
+struct DelState {
+    int32_t stage = 0;            // 0: take the movers, 1: apply them, 2: evaluate the affected
+    int32_t r = 0, l = -1;        // round, its level
+    int32_t limit = -1, delta = 1 << 20;  // near window and its width
+    int32_t calm = 0;             // small rounds in a row
+    int32_t pc = 0, nmin = kInf;  // near entries (list r & 1) and their lowest level
+    int32_t qp = 1, qc = 0, qmin = kInf;  // far list, its length, no level of its vertices below qmin
+    int32_t m = 0, tlc = 0, clc = 0, rc = 0;  // the round's movers, scan items, affected vertices
+    int32_t nbig = 0;             // large tables evaluated before the first round (diagnostics)
+    bool done = false;
+};
+
+// Desire-levels of the vertices of src[0..count) that violate Invariant 2 (level > 0
+// and up* < dnmin[gn(level-1)]): tables up to kThreadDl slots by a thread, others by
+// the warp that found them, one after another (a short list is spread one vertex per
+// warp), and tables above block_cap slots listed (st.rb, from the back of R[1]) for
+// del_eval_big.  Results at or below l contradict the level lemma and are reported.
+// A pending vertex whose slack has not gone below 0 since its last evaluation would
+// get the same answer again: that evaluation is counted (Algorithm 3 counts every
+// evaluation) without the scan.
 template <class Team>
-__device__ bool del_rounds(Team &T, const GraphCtx &g, const int32_t stamp_base, const int32_t *sh_dnmin, int32_t *whist, int32_t *bhist,
-                           int32_t *wsm, RoundStage st) {
-    unsigned long long visits = 0, scanned = 0, evals = 0, evisits = 0;
-    unsigned aff = 0;  // neighbours whose counters a move changed
+__device__ __forceinline__ void del_eval(Team &T, const GraphCtx &g, const RoundStage &st, const int32_t *src,
+                                         int32_t count, int32_t l, int32_t limit, const int32_t *sh_dnmin,
+                                         int32_t *whist, ScanCount &a) {
+    const int lane = lane_id();
+    const int per = min(32, (count + T.nwarps() - 1) / T.nwarps());
+    for (int i0 = T.srank() * per; i0 < count; i0 += T.nwarps() * per) {
+        const int i = i0 + lane;
+        bool small = false, mid = false, big = false;
+        int32_t w = 0, lw = 0, dv = -1, d = -1, sl = 0, dg = 0, where = 0;
+        if (lane < per && i < count) {
+            w = src[i];
+            const int32_t us = g.upstar[w], c = g.cap[w];
+            lw = g.level[w];
+            dv = g.dlv[w];
+            dg = g.deg[w];
+            bool viol = lw > 0 && us < sh_dnmin[(lw - 1) / g.Lg];
+            if (viol && dv >= 0 && g.dslack[w] >= 0) {  // same answer as last time: counted only
+                viol = false;
+                a.evals++;
+                a.evisits += dg;
+            }
+            small = viol && c <= kThreadDl;
+            big = viol && c > g.block_cap && !small;
+            mid = viol && !small && !big;
+            if (small) d = thread_desire_level(g, w, lw, c, sh_dnmin, &sl);
+        }
+        const unsigned mm = __ballot_sync(kFull, mid);
+        for (unsigned m = mm; m; m &= m - 1) {
+            const int j = __ffs(m) - 1;
+            int32_t s1;
+            const int32_t d1 = warp_desire_level(g, __shfl_sync(kFull, w, j), __shfl_sync(kFull, lw, j), sh_dnmin, whist, &s1);
+            if (lane == j) {
+                d = d1;
+                sl = s1;
+            }
+        }
+        if (small || mid) {
+            a.evals++;
+            a.evisits += dg;
+            where = del_settle(g, w, d, sl, dv, l, limit, 8);
+        }
+        del_list(st, where, w, d);
+        const int pb = warp_append(st.rb, big);
+        if (big) g.R[1][g.n - 1 - pb] = w;
+        if (g.trace && lane == 0 && mm) atomicAdd(&g.ctl->rcnt[1], __popc(mm));
+    }
+}
+
+// The nb listed vertices with large tables, a block each.
+template <class Team>
+__device__ __forceinline__ void del_eval_big(Team &T, const GraphCtx &g, const RoundStage &st, int32_t nb, int32_t l,
+                                             int32_t limit, const int32_t *sh_dnmin, int32_t *bhist, ScanCount &a) {
+    for (int i = T.bid(); i < nb; i += T.nblocks()) {
+        const int32_t w = g.R[1][g.n - 1 - i], lw = g.level[w];
+        int32_t sl;
+        const int32_t d = block_desire_level(g, w, lw, sh_dnmin, bhist, bhist + kWarpHist, &sl);
+        if (threadIdx.x < 32) {
+            int where = 0;
+            if (threadIdx.x == 0) {
+                a.evals++;
+                a.evisits += g.deg[w];
+                where = del_settle(g, w, d, sl, g.dlv[w], l, limit, 9);
+            }
+            del_list(st, where, w, d);
+        }
+    }
+}
+
+// Near entries of a round: those on level l move (their scans are queued), the others
+// that still hold stay pending.
+template <class Team>
+__device__ __forceinline__ void del_take(Team &T, const GraphCtx &g, const RoundStage &st, const int4 *near, int32_t pc,
+                                         int32_t l, int32_t limit, int32_t *wsm) {
+    const int lane = lane_id();
+    int32_t kmin = kInf, qmin = kInf;
+    for (int i0 = T.srank() * 32; i0 < pc; i0 += T.nwarps() * 32) {
+        const int i = i0 + lane;
+        bool mover = false, keep = false;
+        int32_t v = 0, d = 0, pv = 0, c = 0;
+        int64_t off = 0;
+        if (i < pc) {
+            const int4 e = near[i];
+            v = e.x;
+            d = e.y;
+            if (g.dlv[v] == d) {
+                if (d == l) {
+                    mover = true;
+                    pv = g.level[v];
+                    c = g.cap[v];
+                    off = g.off[v];
+                    g.level[v] = l;
+                    g.dlv[v] = -1;
+                    g.up[v] = 0;
+                    g.upstar[v] = 0;
+                } else {
+                    keep = true;
+                }
+            }
+        }
+        const bool far = keep && d > limit;  // (the window was narrowed)
+        keep = keep && !far;
+        stage_push(st.pk, keep, make_int4(v, d, 0, 0));
+        if (__any_sync(kFull, far)) stage_push(st.q, far, v);
+        if (keep) kmin = min(kmin, d);
+        if (far) qmin = min(qmin, d);
+        enqueue_mover(g, st, mover, v, pv, c, off, wsm);
+    }
+    kmin = (int32_t)__reduce_min_sync(kFull, (unsigned)kmin);
+    qmin = (int32_t)__reduce_min_sync(kFull, (unsigned)qmin);
+    if (lane == 0 && kmin != kInf) atomicMin(st.bmin, kmin);
+    if (lane == 0 && qmin != kInf) atomicMin(st.qmin, qmin);
+}
+
+// The window moves on: far vertices with levels up to limit become near entries, those
+// still pending beyond it go to the other far list.
+template <class Team>
+__device__ __forceinline__ void del_refill(Team &T, const GraphCtx &g, const RoundStage &st, const int32_t *far,
+                                           int32_t qc, int32_t limit) {
+    int32_t kmin = kInf, qmin = kInf;
+    for (int i0 = T.srank() * 32; i0 < qc; i0 += T.nwarps() * 32) {
+        const int i = i0 + lane_id();
+        const int32_t v = i < qc ? far[i] : 0;
+        const int32_t d = i < qc ? g.dlv[v] : -1;
+        const bool near = d >= 0 && d <= limit, stay = d > limit;
+        stage_push(st.pk, near, make_int4(v, d, 0, 0));
+        stage_push(st.q, stay, v);
+        if (near) kmin = min(kmin, d);
+        if (stay) qmin = min(qmin, d);
+    }
+    kmin = (int32_t)__reduce_min_sync(kFull, (unsigned)kmin);
+    qmin = (int32_t)__reduce_min_sync(kFull, (unsigned)qmin);
+    if (lane_id() == 0 && kmin != kInf) atomicMin(st.bmin, kmin);
+    if (lane_id() == 0 && qmin != kInf) atomicMin(st.qmin, qmin);
+}
+
+// The next window: from the lowest far level, wide enough for about a thousand entries
+// once it has been narrowed.
+__device__ __forceinline__ void del_window(const GraphCtx &g, DelState &s) {
+    s.limit = (int32_t)min((int64_t)s.qmin + s.delta - 1, (int64_t)g.K);
+}
+
+__device__ __forceinline__ void del_window_done(DelState &s) {
+    if (s.pc < 512) s.delta = min(4 * s.delta, 1 << 20);
+    else if (s.pc > 2048) s.delta = max(1, s.delta >> 2);
+}
+
+// Neighbours of the moves pv -> l of N slots ws: effects, and the affected neighbours
+// to evaluate again (queued once per round, stamp sid).
+template <int N>
+__device__ __forceinline__ void del_effects(const GraphCtx &g, const RoundStage &st, const int32_t (&ws)[N], int32_t l,
+                                            const int32_t (&pv)[N / 4], int32_t sid, int (&cu)[N / 4],
+                                            int (&cs)[N / 4], ScanCount &a) {
+    int32_t lv[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) lv[k] = valid_id(g, ws[k]) ? g.level[ws[k]] : 0;
+    unsigned push = 0, maybe = 0;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        a.visits += ws[k] >= 0;
+        const int e = del_effect(g, ws[k], lv[k], l, pv[k >> 2], cu[k >> 2], cs[k >> 2], a.aff);
+        if (e == 1) push |= 1u << k;
+        if (e == 2) maybe |= 1u << k;
+    }
+    if (push | maybe) {
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+            if ((push | maybe) >> k & 1u) {
+                const int32_t dv = g.dlv[ws[k]];
+                if (dv >= 0) {
+                    push |= 1u << k;  // pending: rechecked
+                    del_slack(g, ws[k], dv, l, pv[k >> 2]);
+                }
+            }
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+            if ((push >> k & 1u) && atomicExch(&g.stamp[ws[k]], sid) == sid) push &= ~(1u << k);
+    }
+    if (__any_sync(kFull, push != 0)) stage_push_masked(st.f, push, ws);
+}
+
+template <int U, class Team>
+__device__ __forceinline__ void del_apply_chunks(Team &T, const GraphCtx &g, const RoundStage &st, const int4 *cl,
+                                                 int32_t clc, int32_t l, int32_t sid, ScanCount &a) {
     const int lane = lane_id();
     const int4 *pool4 = reinterpret_cast<const int4 *>(g.slots);
-    for (int r = 0;; ++r) {
-        const int p = r & 1, q = p ^ 1;
-        const int32_t l = g.ctl->nextmin[p];
-        if (l == kInf) break;
-        if (r > g.K + 2) {
-            if (T.leader()) report(g, kErrInternal, 7, l, r, 0);
+    const int crank = T.nwarps() - 1 - T.srank();  // (thread-mode items start at the first warp)
+    for (int c0 = crank; c0 < clc; c0 += U * T.nwarps()) {
+        int4 it[U];
+        int32_t ws[4 * U], pv[U];
+        int cu[U], cs[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int ci = c0 + u * T.nwarps();
+            it[u] = ci < clc ? cl[ci] : make_int4(0, 0, 0, 0);
+            const int j = (it[u].y >> 5) * (kChunk / 4) + lane;
+            const bool in = ci < clc && item_ok(g, it[u], it[u].y & 31) && j < ((1 << (it[u].y & 31)) >> 2);
+            const int4 s4 = in ? pool4[it[u].z + j] : empty4();
+            ws[4 * u] = s4.x; ws[4 * u + 1] = s4.y; ws[4 * u + 2] = s4.z; ws[4 * u + 3] = s4.w;
+            a.scanned += in ? 4 : 0;
+            pv[u] = it[u].w;
+            cu[u] = cs[u] = 0;
+        }
+        del_effects(g, st, ws, l, pv, sid, cu, cs, a);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int x = (int)__reduce_add_sync(kFull, (unsigned)cu[u]), y = (int)__reduce_add_sync(kFull, (unsigned)cs[u]);
+            if (lane == 0) {
+                if (x) atomicAdd(&g.up[it[u].x], x);
+                if (y) atomicAdd(&g.upstar[it[u].x], y);
+            }
+        }
+    }
+}
+
+// Effects of the round's movers (scan items tl and cl) on their neighbours.
+template <class Team>
+__device__ __forceinline__ void del_apply(Team &T, const GraphCtx &g, const RoundStage &st, const DelState &s,
+                                          const int4 *tl, const int4 *cl, int32_t sid, ScanCount &a) {
+    const int lane = lane_id();
+    const int4 *pool4 = reinterpret_cast<const int4 *>(g.slots);
+    for (int i0 = T.srank() * 32; i0 < s.tlc; i0 += T.nwarps() * 32) {
+        const int i = i0 + lane;
+        const int4 it = i < s.tlc ? tl[i] : make_int4(0, 0, 0, 0);
+        const int ng = (i < s.tlc && item_ok(g, it, it.y)) ? (1 << it.y) >> 2 : 0;
+        const int maxg = (int)__reduce_max_sync(kFull, (unsigned)ng);
+        const int32_t pv[4] = {it.w, it.w, it.w, it.w};
+        int cu[4] = {0, 0, 0, 0}, cs[4] = {0, 0, 0, 0};
+        for (int j0 = 0; j0 < maxg; j0 += 4) {
+            int32_t ws[16];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int4 s4 = j0 + j < ng ? pool4[it.z + j0 + j] : empty4();
+                ws[4 * j] = s4.x; ws[4 * j + 1] = s4.y; ws[4 * j + 2] = s4.z; ws[4 * j + 3] = s4.w;
+            }
+            a.scanned += 4 * max(0, min(4, ng - j0));
+            del_effects(g, st, ws, s.l, pv, sid, cu, cs, a);
+        }
+        if (i < s.tlc) {
+            const int x = cu[0] + cu[1] + cu[2] + cu[3], y = cs[0] + cs[1] + cs[2] + cs[3];
+            if (x) atomicAdd(&g.up[it.x], x);
+            if (y) atomicAdd(&g.upstar[it.x], y);
+        }
+    }
+    if (!Team::kGrid && s.clc <= T.nwarps()) del_apply_chunks<1>(T, g, st, cl, s.clc, s.l, sid, a);
+    else del_apply_chunks<4>(T, g, st, cl, s.clc, s.l, sid, a);
+}
+
+// A grid's block publishes the near and far vertices it listed, and their minima.
+__device__ __forceinline__ void del_flush(const GraphCtx &g, const RoundStage &st, unsigned which, int32_t *nmin,
+                                          int32_t *qmin) {
+    stage_flush_round(g, st, which);
+    if (threadIdx.x == 0) {
+        if (*st.bmin != kInf) atomicMin(nmin, *st.bmin);
+        if (*st.qmin != kInf) atomicMin(qmin, *st.qmin);
+        *st.bmin = *st.qmin = kInf;
+    }
+}
+
+__device__ __forceinline__ void del_trace(const GraphCtx &g, const DelState &s, int32_t pc, int32_t nb, uint64_t t0,
+                                          uint64_t t1, uint64_t t2) {
+    if (g.ctl->trace_n >= g.trace_cap) return;
+    int32_t *rec = g.trace + 12 * g.ctl->trace_n++;
+    rec[0] = s.l; rec[1] = pc; rec[2] = s.m; rec[3] = s.tlc; rec[4] = s.clc;
+    rec[5] = (int32_t)(t1 - t0); rec[6] = (int32_t)(t2 - t1);
+    rec[7] = (int32_t)(global_ns() - t2);
+    rec[8] = g.ctl->rcnt[1];  // desire-levels computed by a warp
+    rec[9] = nb;              // and by a block
+    rec[10] = rec[11] = 0;
+    g.ctl->rcnt[1] = 0;
+}
+
+// The first evaluation: the batch's touched vertices, all of them far (no window yet).
+template <class Team>
+__device__ __forceinline__ bool del_initial(Team &T, const GraphCtx &g, RoundStage &st, const int32_t *sh_dnmin, int32_t *whist,
+                            int32_t *bhist, DelState &s, ScanCount &a) {
+    st.pk.gcnt = &g.ctl->pcnt[0];  // (never used: no level is within the window)
+    st.pk.glist = g.P[0];
+    st.pk.gcap = 2 * (int64_t)g.n;
+    st.q.gcnt = &g.ctl->qcnt[s.qp];
+    st.q.glist = g.lfill[s.qp];
+    st.q.gcap = g.n;
+    st.rb = &g.ctl->rbcnt;
+    del_eval(T, g, st, g.touched, g.ctl->tcount, -1, s.limit, sh_dnmin, whist, a);
+    del_flush(g, st, 16u, &g.ctl->nextmin[0], &g.ctl->qmin[s.qp]);
+    if (!T.sync()) return false;
+    const int32_t nb = s.nbig = g.ctl->rbcnt;
+    if (nb > 0) {
+        del_eval_big(T, g, st, nb, -1, s.limit, sh_dnmin, bhist, a);
+        del_flush(g, st, 16u, &g.ctl->nextmin[0], &g.ctl->qmin[s.qp]);
+        if (!T.sync()) return false;
+        if (T.leader()) g.ctl->rbcnt = 0;  // next used several barriers from here
+    }
+    s.qc = g.ctl->qcnt[s.qp];
+    s.qmin = g.ctl->qmin[s.qp];
+    return true;
+}
+
+// Rounds run by one block with its lists in shared memory: a block team's rounds, and
+// (kLimit) the small rounds of a grid, which block 0 runs alone while the other blocks
+// wait at one grid barrier (a grid's round takes three such barriers with lists
+// published before each; a block's three block barriers).  With kLimit the rounds stop, at
+// the stage that s names, when the next stage is above the kSolo bounds or the stretch
+// has taken a quarter of the wait limit; a stage's input lists are then in global memory.
+constexpr int kSoloNear = 4096, kSoloFar = 4096, kSoloEval = 256;
+
+template <bool kLimit>
+__device__ __forceinline__ bool del_rounds_local(const GraphCtx &g, int32_t stamp_base, const int32_t *sh_dnmin, int32_t *whist,
+                                 int32_t *bhist, int32_t *wsm, RoundStage st, DelState &s, ScanCount &a) {
+    BlockTeam T{g.ctl};
+    int4 *const nbuf[2] = {st.pk.buf, st.cl.buf + (st.cl.cap >> 1)};
+    st.cl.cap >>= 1;
+    const int32_t ncap = min(st.pk.cap, st.cl.cap);
+    int32_t *lc = reinterpret_cast<int32_t *>(st.ph4);  // entries beyond the shared lists: near, tl, cl, f, refilled far;
+                                                          // 5: flag; 6: end of the far list; 7: large tables
+    st.pk.cap = ncap;
+    st.pk.gcnt = lc;
+    st.pk.gcap = 2 * (int64_t)g.n;
+    st.tl.gcnt = lc + 1;
+    st.tl.glist = g.TL[0];
+    st.tl.gcap = g.n;
+    st.cl.gcnt = lc + 2;
+    st.cl.glist = g.CL[0];
+    st.cl.gcap = g.clcap;
+    st.f.gcnt = lc + 3;
+    st.f.glist = g.R[0];
+    st.f.gcap = g.n;
+    st.q.gcap = g.n;
+    st.rb = lc + 7;
+    const int4 *near = g.P[s.r & 1], *tl = st.tl.buf, *cl = st.cl.buf;
+    const int32_t *aff = st.f.buf;
+    auto reset = [&] {  // thread 0
+        lc[0] = lc[1] = lc[2] = lc[3] = lc[4] = lc[7] = 0;
+        lc[6] = s.qc;
+        st.pk.hdr[0] = 0; st.pk.hdr[1] = ncap;
+        st.tl.hdr[0] = 0; st.tl.hdr[1] = st.tl.cap;
+        st.cl.hdr[0] = 0; st.cl.hdr[1] = st.cl.cap;
+        st.f.hdr[0] = 0; st.f.hdr[1] = st.f.cap;
+        st.q.hdr[0] = 0; st.q.hdr[1] = st.q.cap;
+        *st.movers = 0;
+        *st.bmin = *st.qmin = kInf;
+    };
+    // a list's shared entries after those that went to its global list; its length
+    auto publish = [&](auto &x, int over) {
+        const int nsh = min(x.hdr[0], x.hdr[1]);
+        for (int i = threadIdx.x; i < nsh; i += blockDim.x)
+            if (over + i < x.gcap) x.glist[over + i] = x.buf[i];
+        if (threadIdx.x == 0 && (int64_t)over + nsh > x.gcap) report(g, kErrListOverflow, 4, over, nsh, (int32_t)x.gcap);
+    };
+    auto total = [&](auto &x, int over) { return min(x.hdr[0], x.hdr[1]) + over; };
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        reset();
+        lc[5] = 0;
+    }
+    __syncthreads();
+    const uint64_t t_start = kLimit && threadIdx.x == 0 ? global_ns() : 0;
+    uint64_t t0 = 0, t1 = 0, t2 = 0;
+    bool leave = false;
+    int32_t refills = 0;
+    for (;;) {
+        const int p = s.r & 1, q = p ^ 1;
+        if (s.nmin == kInf) {  // the near list is used up
+            s.pc = 0;
+            if (s.qc == 0) {
+                s.done = true;
+                return true;
+            }
+            if (kLimit && (s.qc > kSoloFar || leave)) return true;
+            if (++refills > g.K + 4) {  // every window takes at least one level
+                if (threadIdx.x == 0) report(g, kErrInternal, 26, s.qc, s.qmin, s.limit);
+                return false;
+            }
+            del_window(g, s);
+            st.pk.buf = nbuf[p];
+            st.pk.glist = g.P[p];
+            st.q.glist = g.lfill[s.qp ^ 1];
+            st.q.gcnt = lc + 4;
+            del_refill(T, g, st, g.lfill[s.qp], s.qc, s.limit);
+            __syncthreads();
+            const int over = lc[0], overq = lc[4];
+            s.pc = total(st.pk, over);
+            s.qc = total(st.q, overq);
+            s.nmin = *st.bmin;
+            s.qmin = *st.qmin;
+            near = nbuf[p];
+            const bool out = over > 0 || (kLimit && s.pc > kSoloNear);
+            if (out) {
+                publish(st.pk, over);
+                near = g.P[p];
+            }
+            publish(st.q, overq);
+            s.qp ^= 1;
+            del_window_done(s);
+            __syncthreads();
+            if (threadIdx.x == 0) reset();
+            __syncthreads();
+            if (kLimit && out) return true;
+            continue;
+        }
+        // take
+        const int32_t pc = s.pc;
+        s.l = s.nmin;
+        if (s.r > 2 * g.K + 4) {
+            if (threadIdx.x == 0) report(g, kErrInternal, 7, s.l, s.r, 0);
             return false;
         }
-        const int32_t sid = sid_of(stamp_base, l);
-        const uint64_t t_round = (g.trace && T.leader()) ? global_ns() : 0;
-        st.pk.gcnt = &g.ctl->pcnt[q];
+        int32_t err = 0;
+        if (threadIdx.x == 0) {
+            err = ld_volatile(&g.ctl->err);  // seen a round late, off the critical chain
+            if (g.trace || kLimit) t0 = global_ns();
+        }
+        st.pk.buf = nbuf[q];
         st.pk.glist = g.P[q];
+        st.q.glist = g.lfill[s.qp];
+        st.q.gcnt = lc + 6;  // new far vertices go behind those already listed
+        del_take(T, g, st, near, pc, s.l, s.limit, wsm);
+        if (threadIdx.x == 0 && (err || (kLimit && t0 - t_start > (uint64_t)(g.wait_limit_ns >> 2)))) lc[5] = err ? 2 : 1;
+        __syncthreads();
+        if (lc[5] == 2) return false;
+        s.m = *st.movers;
+        s.tlc = total(st.tl, lc[1]);
+        s.clc = total(st.cl, lc[2]);
+        if (threadIdx.x == 0) {
+            if (s.m > 0) atomicAdd(&g.ctl->st[kStRounds], 1ull);
+            atomicAdd(&g.ctl->st[kStMoves], (unsigned long long)s.m);
+            if (g.trace) t1 = global_ns();
+        }
+        leave = kLimit && lc[5] != 0;
+        const bool heavy = kLimit && (s.tlc > kSoloTl || s.clc > kSoloCl);
+        tl = st.tl.buf;
+        cl = st.cl.buf;
+        if (lc[1] > 0 || heavy) {
+            publish(st.tl, lc[1]);
+            tl = g.TL[0];
+        }
+        if (lc[2] > 0 || heavy) {
+            publish(st.cl, lc[2]);
+            cl = g.CL[0];
+        }
+        if (heavy) {  // the grid applies this round: the kept near entries with it
+            publish(st.pk, lc[0]);
+            s.pc = total(st.pk, lc[0]);
+            s.nmin = *st.bmin;
+            s.stage = 1;
+            __syncthreads();
+            if (threadIdx.x == 0) reset();
+            __syncthreads();
+            return true;
+        }
+        __threadfence_block();
+        __syncthreads();
+        // apply
+        del_apply(T, g, st, s, tl, cl, sid_of(stamp_base, s.l), a);
+        __threadfence_block();
+        __syncthreads();
+        if (g.trace && threadIdx.x == 0) t2 = global_ns();
+        s.rc = total(st.f, lc[3]);
+        aff = st.f.buf;
+        const bool wide = kLimit && s.rc > kSoloEval;
+        if (lc[3] > 0 || wide) {
+            publish(st.f, lc[3]);
+            aff = g.R[0];
+            __syncthreads();
+        }
+        if (wide) {  // the grid evaluates
+            publish(st.pk, lc[0]);
+            s.pc = total(st.pk, lc[0]);
+            s.nmin = *st.bmin;
+            s.stage = 2;
+            __syncthreads();
+            if (threadIdx.x == 0) reset();
+            __syncthreads();
+            return true;
+        }
+        // evaluate
+        del_eval(T, g, st, aff, s.rc, s.l, s.limit, sh_dnmin, whist, a);
+        __threadfence_block();
+        __syncthreads();
+        const int32_t nb = lc[7];
+        if (nb > 0) {
+            del_eval_big(T, g, st, nb, s.l, s.limit, sh_dnmin, bhist, a);
+            __threadfence_block();
+            __syncthreads();
+        }
+        const int32_t over = lc[0];
+        s.pc = total(st.pk, over);
+        s.nmin = *st.bmin;
+        s.qmin = min(s.qmin, *st.qmin);
+        const int32_t qc = total(st.q, lc[6]);
+        if (qc > s.qc) publish(st.q, lc[6]);
+        s.qc = qc;
+        near = nbuf[q];
+        leave = leave || (kLimit && s.pc > kSoloNear);
+        if (over > 0 || leave) {
+            publish(st.pk, over);
+            near = g.P[q];
+        }
+        ++s.r;
+        totals_keep(wsm, a, false);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            if (g.trace) del_trace(g, s, pc, nb, t0, t1, t2);
+            reset();
+        }
+        __syncthreads();
+        if (leave) return true;
+    }
+}
+
+template <class Team>
+__device__ __forceinline__ bool del_rounds(Team &T, const GraphCtx &g, const int32_t stamp_base, const int32_t *sh_dnmin,
+                           int32_t *whist, int32_t *bhist, int32_t *wsm, RoundStage st, DelState s, ScanCount a) {
+    totals_clear(wsm);
+    if constexpr (!Team::kGrid) {
+        if (!del_rounds_local<false>(g, stamp_base, sh_dnmin, whist, bhist, wsm, st, s, a)) return false;
+    } else {
+        Ctl *c = g.ctl;
         st.pk.gcap = 2 * (int64_t)g.n;
-        st.tl.gcnt = &g.ctl->tlcnt[0];
+        st.tl.gcnt = &c->tlcnt[0];
         st.tl.glist = g.TL[0];
         st.tl.gcap = g.n;
-        st.cl.gcnt = &g.ctl->clcnt[0];
+        st.cl.gcnt = &c->clcnt[0];
         st.cl.glist = g.CL[0];
         st.cl.gcap = g.clcap;
-        st.f.gcnt = &g.ctl->rcnt[0];
+        st.f.gcnt = &c->rcnt[0];
         st.f.glist = g.R[0];
         st.f.gcap = g.n;
-        int32_t kmin = kInf;
-        if (T.leader()) {
-            g.ctl->rcnt[0] = 0;
-            g.ctl->rcnt[1] = 0;
-            g.ctl->rbcnt = 0;
-        }
-        // Phase 1: pending entries with dl == l move; the rest stay pending.
-        const int32_t pc = g.ctl->pcnt[p];
-        for (int i0 = T.srank() * 32; i0 < pc; i0 += T.nwarps() * 32) {
-            const int i = i0 + lane;
-            bool mover = false, keep = false;
-            int32_t v = 0, d = 0, pv = 0, c = 0;
-            int64_t off = 0;
-            if (i < pc) {
-                const int4 e = g.P[p][i];
-                v = e.x;
-                d = e.y;
-                if (g.dlv[v] == d) {
-                    if (d == l) {
-                        mover = true;
-                        pv = g.level[v];
-                        c = g.cap[v];
-                        off = g.off[v];
-                        g.level[v] = l;
-                        g.dlv[v] = -1;
-                        g.up[v] = 0;
-                        g.upstar[v] = 0;
-                    } else {
-                        keep = true;
-                    }
+        st.q.gcap = g.n;
+        st.rb = &c->rbcnt;
+        s.done = s.qc == 0;  // nobody violates
+        while (!s.done) {
+            // (a round handed back by the block costs more than a grid's own: only after small rounds)
+            if (s.stage == 0 && s.tlc <= kSoloTl && s.clc <= kSoloCl && s.rc <= kSoloEval &&
+                (s.nmin != kInf ? s.pc <= kSoloNear : s.qc <= kSoloFar)) {
+                if (T.bid() == 0) {
+                    del_rounds_local<true>(g, stamp_base, sh_dnmin, whist, bhist, wsm, st, s, a);
+                }
+                const bool ok = T.handoff([&] {
+                    st.pk.hdr[1] = st.pk.cap;  // the grid's stages use the whole buffers
+                    st.cl.hdr[1] = st.cl.cap;
+                    const int p = s.r & 1, w = s.stage == 0 ? p : p ^ 1;  // where s's near entries are
+                    int32_t *o = c->solo;
+                    o[0] = s.stage | (s.done ? 4 : 0);
+                    o[1] = s.r; o[2] = s.l; o[3] = s.limit; o[4] = s.delta; o[5] = s.qp;
+                    o[6] = s.pc; o[7] = s.nmin; o[8] = s.qc; o[9] = s.qmin;
+                    o[10] = s.m; o[11] = s.tlc; o[12] = s.clc; o[13] = s.rc;
+                    c->pcnt[w] = s.pc;
+                    c->nextmin[w] = s.nmin;
+                    c->pcnt[w ^ 1] = 0;
+                    c->nextmin[w ^ 1] = kInf;
+                    c->qcnt[s.qp] = s.qc;
+                    c->qmin[s.qp] = s.qmin;
+                    c->qcnt[s.qp ^ 1] = 0;
+                    c->qmin[s.qp ^ 1] = kInf;
+                    c->mcnt[0] = c->tlcnt[0] = c->clcnt[0] = c->rcnt[0] = 0;
+                    c->rbcnt = 0;
+                });
+                if (!ok) return false;
+                const int32_t *o = c->solo;
+                const int32_t f = ld_volatile(o);
+                s.stage = f & 3;
+                s.done = (f & 4) != 0;
+                s.r = ld_volatile(o + 1); s.l = ld_volatile(o + 2); s.limit = ld_volatile(o + 3); s.delta = ld_volatile(o + 4);
+                s.qp = ld_volatile(o + 5); s.pc = ld_volatile(o + 6); s.nmin = ld_volatile(o + 7); s.qc = ld_volatile(o + 8);
+                s.qmin = ld_volatile(o + 9); s.m = ld_volatile(o + 10); s.tlc = ld_volatile(o + 11);
+                s.clc = ld_volatile(o + 12); s.rc = ld_volatile(o + 13);
+                if (s.done) break;
+            }
+            const int p = s.r & 1, q = p ^ 1;
+            const int32_t pc = s.pc;
+            const bool tr = g.trace && T.leader();
+            uint64_t t0 = tr ? global_ns() : 0, t1 = t0, t2 = t0;
+            if (s.stage == 0 && s.nmin == kInf) {  // the near list is used up: the window moves on
+                if (s.qc == 0) break;
+                if (s.r > 2 * g.K + 4) {
+                    if (T.leader()) report(g, kErrInternal, 26, s.qc, s.qmin, s.limit);
+                    return false;
+                }
+                del_window(g, s);
+                // (into the other parity's lists: slower blocks may still read this parity's
+                // counts, published by the last barrier)
+                const int qn = s.qp ^ 1;
+                st.pk.gcnt = &c->pcnt[q];
+                st.pk.glist = g.P[q];
+                st.q.gcnt = &c->qcnt[qn];
+                st.q.glist = g.lfill[qn];
+                del_refill(T, g, st, g.lfill[s.qp], s.qc, s.limit);
+                del_flush(g, st, 24u, &c->nextmin[q], &c->qmin[qn]);
+                if (!T.sync()) return false;
+                if (T.leader()) {  // the old far list, filled again by the next refill
+                    c->qcnt[s.qp] = 0;
+                    c->qmin[s.qp] = kInf;
+                }
+                ++s.r;
+                s.qp = qn;
+                s.pc = c->pcnt[q];
+                s.nmin = c->nextmin[q];
+                s.qc = c->qcnt[qn];
+                s.qmin = c->qmin[qn];
+                del_window_done(s);
+                if (s.nmin == kInf && !T.sync()) return false;  // (a refill straight after this one)
+                continue;
+            }
+            st.pk.gcnt = &c->pcnt[q];
+            st.pk.glist = g.P[q];
+            st.q.gcnt = &c->qcnt[s.qp];
+            st.q.glist = g.lfill[s.qp];
+            if (s.stage == 0) {
+                s.l = s.nmin;
+                if (s.r > 2 * g.K + 4) {
+                    if (T.leader()) report(g, kErrInternal, 7, s.l, s.r, 0);
+                    return false;
+                }
+                if (T.leader()) {
+                    c->rcnt[0] = 0;
+                    c->rbcnt = 0;
+                }
+                st.q.buf = st.f.buf;
+                del_take(T, g, st, g.P[p], s.pc, s.l, s.limit, wsm);
+                del_flush(g, st, 30u, &c->nextmin[q], &c->qmin[s.qp]);
+                st.q.buf = reinterpret_cast<int32_t *>(st.tl.buf);
+                if (threadIdx.x == 0) {
+                    if (*st.movers) atomicAdd(&c->mcnt[0], *st.movers);
+                    *st.movers = 0;
+                }
+                if (!T.sync()) return false;
+                s.m = c->mcnt[0];
+                s.tlc = c->tlcnt[0];
+                s.clc = c->clcnt[0];
+                if (T.leader()) {
+                    if (s.m > 0) atomicAdd(&c->st[kStRounds], 1ull);
+                    atomicAdd(&c->st[kStMoves], (unsigned long long)s.m);
+                    c->pcnt[p] = 0;
+                    c->nextmin[p] = kInf;
                 }
             }
-            stage_push(st.pk, keep, make_int4(v, d, 0, 0));
-            if (keep) kmin = min(kmin, d);
-            enqueue_mover(g, st, mover, v, pv, c, off, wsm);
-        }
-        kmin = (int32_t)__reduce_min_sync(kFull, (unsigned)kmin);
-        if (lane == 0 && kmin != kInf) atomicMin(st.bmin, kmin);
-        stage_flush_round(g, st, 14u);
-        if (threadIdx.x == 0) {
-            if (*st.movers) atomicAdd(&g.ctl->mcnt[0], *st.movers);
-            if (*st.bmin != kInf) atomicMin(&g.ctl->nextmin[q], *st.bmin);
-            *st.movers = 0;
-            *st.bmin = kInf;
-        }
-        if (!T.sync()) return false;
-        // Phase 2: movers' neighbours.
-        const uint64_t t_mid1 = (g.trace && T.leader()) ? global_ns() : 0;
-        if (T.leader()) {
-            const int32_t mc = g.ctl->mcnt[0];
-            if (mc > 0) g.ctl->st[kStRounds] += 1;
-            g.ctl->st[kStMoves] += (unsigned long long)mc;
-            g.ctl->pcnt[p] = 0;
-            g.ctl->nextmin[p] = kInf;
-        }
-        const int32_t tlc = g.ctl->tlcnt[0];
-        for (int i0 = T.srank() * 32; i0 < tlc; i0 += T.nwarps() * 32) {
-            const int i = i0 + lane;
-            const int4 it = i < tlc ? g.TL[0][i] : make_int4(0, 0, 0, 0);
-            const int ng = (i < tlc && item_ok(g, it, it.y)) ? (1 << it.y) >> 2 : 0;
-            const int maxg = (int)__reduce_max_sync(kFull, (unsigned)ng);
-            int cu = 0, cs = 0;
-            for (int j0 = 0; j0 < maxg; j0 += 4) {
-                int32_t ws[16], lv[16];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int4 s4 = j0 + j < ng ? pool4[it.z + j0 + j] : empty4();
-                    ws[4 * j] = s4.x; ws[4 * j + 1] = s4.y; ws[4 * j + 2] = s4.z; ws[4 * j + 3] = s4.w;
-                }
-#pragma unroll
-                for (int k = 0; k < 16; ++k) lv[k] = valid_id(g, ws[k]) ? g.level[ws[k]] : 0;
-                unsigned push = 0, maybe = 0;
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    visits += ws[k] >= 0;
-                    const int e = del_effect(g, ws[k], lv[k], l, it.w, cu, cs, aff);
-                    if (e == 1) push |= 1u << k;
-                    if (e == 2) maybe |= 1u << k;
-                }
-#pragma unroll
-                for (int k = 0; k < 16; ++k)
-                    if ((push | maybe) >> k & 1u) {
-                        const int32_t dv = g.dlv[ws[k]];
-                        if (dv >= 0) {
-                            push |= 1u << k;  // pending: rechecked
-                            del_slack(g, ws[k], dv, l, it.w);
-                        }
-                    }
-#pragma unroll
-                for (int k = 0; k < 16; ++k)
-                    if ((push >> k & 1u) && atomicExch(&g.stamp[ws[k]], sid) == sid) push &= ~(1u << k);
-                scanned += 4 * (unsigned long long)max(0, min(4, ng - j0));
-                stage_push_masked(st.f, push, ws);
+            if (s.stage <= 1) {
+                if (tr) t1 = global_ns();
+                del_apply(T, g, st, s, g.TL[0], g.CL[0], sid_of(stamp_base, s.l), a);
+                stage_flush_round(g, st, 1u);
+                if (!T.sync()) return false;
+                s.rc = c->rcnt[0];
             }
-            if (i < tlc) {
-                if (cu) atomicAdd(&g.up[it.x], cu);
-                if (cs) atomicAdd(&g.upstar[it.x], cs);
+            if (tr) t2 = global_ns();
+            if (T.leader()) {
+                c->mcnt[0] = 0;
+                c->tlcnt[0] = 0;
+                c->clcnt[0] = 0;
             }
-        }
-        const int32_t clc = g.ctl->clcnt[0];
-        for (int c0 = T.srank(); c0 < clc; c0 += 4 * T.nwarps()) {
-            int4 it[4];
-            bool in[4];
-            int32_t ws[16], lv[16];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int cu = c0 + u * T.nwarps();
-                it[u] = cu < clc ? g.CL[0][cu] : make_int4(0, 0, 0, 0);
-                const int j = (it[u].y >> 5) * (kChunk / 4) + lane;
-                in[u] = cu < clc && item_ok(g, it[u], it[u].y & 31) && j < ((1 << (it[u].y & 31)) >> 2);
-                const int4 s4 = in[u] ? pool4[it[u].z + j] : empty4();
-                ws[4 * u] = s4.x; ws[4 * u + 1] = s4.y; ws[4 * u + 2] = s4.z; ws[4 * u + 3] = s4.w;
+            del_eval(T, g, st, g.R[0], s.rc, s.l, s.limit, sh_dnmin, whist, a);
+            del_flush(g, st, 24u, &c->nextmin[q], &c->qmin[s.qp]);
+            if (!T.sync()) return false;
+            const int32_t nb = c->rbcnt;
+            if (nb > 0) {
+                del_eval_big(T, g, st, nb, s.l, s.limit, sh_dnmin, bhist, a);
+                del_flush(g, st, 24u, &c->nextmin[q], &c->qmin[s.qp]);
+                if (!T.sync()) return false;
             }
-#pragma unroll
-            for (int k = 0; k < 16; ++k) lv[k] = valid_id(g, ws[k]) ? g.level[ws[k]] : 0;
-            int cu4[4] = {0, 0, 0, 0}, cs4[4] = {0, 0, 0, 0};
-            unsigned push = 0, maybe = 0;
-#pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                visits += ws[k] >= 0;
-                const int e = del_effect(g, ws[k], lv[k], l, it[k >> 2].w, cu4[k >> 2], cs4[k >> 2], aff);
-                if (e == 1) push |= 1u << k;
-                if (e == 2) maybe |= 1u << k;
+            totals_keep(wsm, a, false);
+            s.pc = c->pcnt[q];
+            s.nmin = c->nextmin[q];
+            s.qc = c->qcnt[s.qp];
+            s.qmin = c->qmin[s.qp];
+            s.stage = 0;
+            ++s.r;
+            s.calm = s.tlc <= kSoloTl && s.clc <= kSoloCl && s.rc <= kSoloEval ? s.calm + 1 : 0;
+            // narrow the window: the next take sends the rest away.  Only from a wide open
+            // one, whose far list is empty: in another a vertex that came back near may still
+            // be listed (and its count, which faster blocks' takes change, decides nothing).
+            if (s.calm >= 2 && s.pc > kSoloNear && s.limit >= g.K) {
+                s.delta = 16;
+                s.limit = s.nmin + s.delta - 1;
             }
-#pragma unroll
-            for (int k = 0; k < 16; ++k)
-                if ((push | maybe) >> k & 1u) {
-                    const int32_t dv = g.dlv[ws[k]];
-                    if (dv >= 0) {
-                        push |= 1u << k;  // pending: rechecked
-                        del_slack(g, ws[k], dv, l, it[k >> 2].w);
-                    }
-                }
-#pragma unroll
-            for (int k = 0; k < 16; ++k)
-                if ((push >> k & 1u) && atomicExch(&g.stamp[ws[k]], sid) == sid) push &= ~(1u << k);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) scanned += in[u] ? 4 : 0;
-            stage_push_masked(st.f, push, ws);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int a = warp_sum(cu4[u]), b = warp_sum(cs4[u]);
-                if (lane == 0) {
-                    if (a) atomicAdd(&g.up[it[u].x], a);
-                    if (b) atomicAdd(&g.upstar[it[u].x], b);
-                }
-            }
-        }
-        stage_flush_round(g, st, 1u);
-        if (!T.sync()) return false;
-        // Phase 3: neighbours that now violate Invariant 2 get their desire-level
-        // recomputed (it always lands above l).
-        const uint64_t t_mid2 = (g.trace && T.leader()) ? global_ns() : 0;
-        int32_t tr_movers = 0;
-        if (g.trace && T.leader()) tr_movers = g.ctl->mcnt[0];
-        if (T.leader()) {
-            g.ctl->mcnt[0] = 0;
-            g.ctl->tlcnt[0] = 0;
-            g.ctl->clcnt[0] = 0;
-        }
-        if (!dl_batch(T, g, g.R[0], g.ctl->rcnt[0], q, l, sh_dnmin, whist, bhist, evals, evisits)) return false;
-        if (!T.sync()) return false;
-        if (g.trace && T.leader() && g.ctl->trace_n < g.trace_cap) {
-            int32_t *rec = g.trace + 12 * g.ctl->trace_n++;
-            const uint64_t t_end = global_ns();
-            rec[0] = l; rec[1] = pc; rec[2] = tr_movers; rec[3] = tlc; rec[4] = clc;
-            rec[5] = (int32_t)(t_mid1 - t_round); rec[6] = (int32_t)(t_mid2 - t_mid1);
-            rec[7] = (int32_t)(t_end - t_mid2);
-            rec[8] = g.ctl->rcnt[1];  // desire-levels computed by a warp after the classifying pass
-            rec[9] = g.ctl->rbcnt;    // and by a block
-            rec[10] = rec[11] = 0;
+            if (tr) del_trace(g, s, pc, nb, t0, t1, t2);
         }
     }
-    visits = warp_sum64(visits);
-    scanned = warp_sum64(scanned);
-    const unsigned long long affs = warp_sum64(aff);
-    if (lane == 0) {
-        atomicAdd(&g.ctl->st[kStVisits], visits);
-        atomicAdd(&g.ctl->st[kStSlotsScanned], scanned);
-        if (affs) atomicAdd(&g.ctl->st[kStAffected], affs);
-    }
-    if (evals) {
-        atomicAdd(&g.ctl->st[kStDlEvals], evals);
-        atomicAdd(&g.ctl->st[kStDlVisits], evisits);
-    }
+    totals_flush(g, wsm, a, false);
     return true;
 }
 
@@ -2898,7 +3423,7 @@ __device__ int32_t jump_apply(const GraphCtx &g, int32_t v, int32_t l, int32_t t
 }
 
 template <class Team>
-__device__ bool ins_rounds_jump(Team &T, const GraphCtx &g, const int32_t *sh_upmax, int32_t *whist,
+__device__ __forceinline__ bool ins_rounds_jump(Team &T, const GraphCtx &g, const int32_t *sh_upmax, int32_t *whist,
                                 int32_t *sh_block) {
     const int lane = lane_id();
     const int32_t tc = g.ctl->tcount;
@@ -3110,7 +3635,9 @@ __device__ bool ins_rounds_jump(Team &T, const GraphCtx &g, const int32_t *sh_up
 }
 
 // ---------------------------------------------------------------------------
-// One whole batch (Algorithm 1, one half): returns early when the team stopped
+// One whole batch (Algorithm 1, one half); inlined with all its steps, so that the
+// graph's context is read from kernel parameter space (called as a function it took
+// generic loads, and insertion batches twice as long): returns early when the team stopped
 // (error word set).  sh: shared memory with the group tables, a block-scan
 // scratch and one histogram per warp (the first also serves block-wide
 // desire-levels).
@@ -3123,16 +3650,20 @@ __device__ __forceinline__ void trace_steps(const GraphCtx &g, const uint64_t (&
 }
 
 // kRoundsOnly: the steps before the rounds already ran as separate kernels (the
-// single-graph calls); they are compiled out, leaving the rounds kernel leaner.
-template <class Team, bool kRoundsOnly = false>
-__device__ void run_batch(Team &T, const GraphCtx &g, const BatchIn &in, int32_t *sh, int stage_shift) {
+// single-graph calls); they are compiled out, and kWhat leaves one kind of rounds, so
+// that each rounds kernel gets its registers to itself.
+enum : int { kAnyRounds = 0, kInsertRounds = 1, kJumpRounds = 2, kDeleteRounds = 3 };
+
+template <class Team, bool kRoundsOnly = false, int kWhat = kAnyRounds>
+__device__ __forceinline__ void run_batch(Team &T, const GraphCtx &g, const BatchIn &in, int32_t *sh, int stage_shift) {
     int32_t *sh_upmax = sh;
     int32_t *sh_dnmin = sh + kMaxGroups;
     int *sh_scan = sh + 2 * kMaxGroups;  // 64 ints
     unsigned long long *sh_res = reinterpret_cast<unsigned long long *>(sh_scan);  // block_reserve: <= 17 slots
     int32_t *sh_block = sh + 2 * kMaxGroups + 64;  // kWarpHist + 32 ints, block-wide desire-levels
-    int32_t *whist = sh_block + kWarpHist + 32 + (threadIdx.x >> 5) * kWarpHist;
-    int32_t *sh_stage = sh_block + kWarpHist + 32 + (blockDim.x >> 5) * kWarpHist;
+    // (the staging area before the warps' histograms: its addresses are constants then)
+    int32_t *sh_stage = sh_block + kWarpHist + 32;
+    int32_t *whist = sh_stage + stage_ints(stage_shift) + (threadIdx.x >> 5) * kWarpHist;
     for (int i = threadIdx.x; i < g.G; i += blockDim.x) {
         sh_upmax[i] = g.upmax[i];
         sh_dnmin[i] = g.dnmin[i];
@@ -3160,7 +3691,8 @@ __device__ void run_batch(Team &T, const GraphCtx &g, const BatchIn &in, int32_t
         if (!T.sync()) return;
         if (tr) tmark[nmark++] = global_ns();
     }
-    if (in.op == kOpInsert) {
+    constexpr bool kMayJump = Team::kJump && (kWhat == kAnyRounds || kWhat == kJumpRounds);
+    if (kWhat == kAnyRounds ? in.op == kOpInsert : kWhat != kDeleteRounds) {
         if constexpr (!kRoundsOnly) {
             pre_grow_request(T, g, sh_res);
             if (!T.sync()) return;
@@ -3180,23 +3712,28 @@ __device__ void run_batch(Team &T, const GraphCtx &g, const BatchIn &in, int32_t
             if (!T.sync()) return;
             if (tr) tmark[nmark++] = global_ns();
         }
-        if (!(Team::kJump && g.jump) && !ins_sort_candidates(T, g, sh_scan, sh_upmax)) return;
-        if (tr) {
-            tmark[nmark++] = global_ns();
-            trace_steps(g, tmark, nmark, -1);
-        }
-        if constexpr (Team::kJump) {
-            if (g.jump) {
+        if constexpr (kMayJump) {
+            if (kWhat == kJumpRounds || g.jump) {
+                if (tr) {
+                    tmark[nmark++] = global_ns();
+                    trace_steps(g, tmark, nmark, -1);
+                }
                 ins_rounds_jump(T, g, sh_upmax, whist, sh_block);
                 return;
             }
         }
-        ins_rounds(T, g, sh_upmax, whist, stage_setup(sh_stage, stage_shift));
+        if constexpr (kWhat != kJumpRounds) {
+            if (!ins_sort_candidates(T, g, sh_scan, sh_upmax)) return;
+            if (tr) {
+                tmark[nmark++] = global_ns();
+                trace_steps(g, tmark, nmark, -1);
+            }
+            ins_rounds(T, g, sh_upmax, whist, stage_setup(sh_stage, stage_shift));
+        }
     } else {
         if constexpr (!kRoundsOnly) {
             if (T.leader()) {
-                g.ctl->nextmin[0] = kInf;
-                g.ctl->nextmin[1] = kInf;
+                del_reset(g.ctl);
             }
             step_apply_delete(T, g);
             if (!T.sync()) return;
@@ -3211,25 +3748,19 @@ __device__ void run_batch(Team &T, const GraphCtx &g, const BatchIn &in, int32_t
             if (!T.sync()) return;
             if (tr) tmark[nmark++] = global_ns();
         }
-        unsigned long long evals = 0, evisits = 0;
-        if (!dl_batch(T, g, g.touched, g.ctl->tcount, 0, -1, sh_dnmin, whist, sh_block, evals, evisits)) return;
-        if (evals) {
-            atomicAdd(&g.ctl->st[kStDlEvals], evals);
-            atomicAdd(&g.ctl->st[kStDlVisits], evisits);
-        }
-        if (!T.sync()) return;
+        RoundStage st = stage_setup(sh_stage, stage_shift);
+        DelState ds;
+        ScanCount dc;
+        if (!del_initial(T, g, st, sh_dnmin, whist, sh_block, ds, dc)) return;
         if (tr) {
             tmark[nmark++] = global_ns();
             trace_steps(g, tmark, nmark, -2);
             g.trace[8] = g.ctl->tcount;   // vertices the batch touched
             g.trace[9] = g.ctl->rcnt[1];  // of them violating, desire-level by a warp
-            g.trace[10] = g.ctl->rbcnt;   // by a block (tables above block_cap)
-        }
-        if (T.leader()) {
+            g.trace[10] = ds.nbig;        // by a block (tables above block_cap)
             g.ctl->rcnt[1] = 0;
-            g.ctl->rbcnt = 0;
         }
-        del_rounds(T, g, in.stamp_base, sh_dnmin, whist, sh_block, whist, stage_setup(sh_stage, stage_shift));
+        del_rounds(T, g, in.stamp_base, sh_dnmin, whist, sh_block, whist, st, ds, dc);
     }
 }
 

@@ -78,12 +78,14 @@ struct Ctl {
     int32_t mcnt[2];      // table growth / deletion movers
     int32_t tlcnt[2];     // thread-mode movers
     int32_t clcnt[2];     // chunk items
-    int32_t solo[8];      // insertion: where the rounds stand after phases run by block 0 alone
+    int32_t solo[16];     // where the rounds stand after a stretch run by block 0 alone
     int32_t nlev;         // number of distinct initial-candidate levels
     int32_t ncand;        // initial candidates: touched vertices that violate Invariant 1
     int32_t pcnt[2];      // deletion pending list sizes
     int32_t rcnt[2];      // deletion recompute list sizes
-    int32_t nextmin[2];   // deletion: smallest pending desire-level
+    int32_t nextmin[2];   // deletion: smallest level of a near list's entries
+    int32_t qcnt[2];      // deletion: far vertices (lists lfill[0..1])
+    int32_t qmin[2];      // no level of theirs lies below
     int32_t err_site;     // which check raised the first error (0 = none)
     int32_t err_info[3];  // values seen by that check (diagnostics)
     int32_t trace_n;      // per-round records written
@@ -127,7 +129,7 @@ struct GraphCtx {
     int32_t *tomb;         // [n] tombstones in the table
     int32_t *stamp;        // [n] dedupe stamps
     int32_t *dlv;          // [n] pending desire-level, -1 when none
-    int32_t *dslack;       // [n] deletion: slack of a pending vertex's desire-level (see dl_batch)
+    int32_t *dslack;       // [n] deletion: slack of a pending vertex's desire-level (see del_eval)
     int32_t *inc;          // [n] incoming insertions of the batch
     int32_t *slots;        // adjacency pool
     unsigned long long *pool_top;  // slots handed out
@@ -147,13 +149,14 @@ struct GraphCtx {
     int32_t *lbuf[3];      // insertion: up-list buffers (phase index mod 3), lcap entries each
     int64_t lcap;
     int32_t *lout;         // [n] insertion: a chunk-mode mover's output up-list (int4 units), -1 none
-    int32_t *lfill[2];     // [n] insertion: entries written to it so far (by phase parity)
+    int32_t *lfill[2];     // [n] insertion: entries written to it so far (by phase parity);
+                           // deletion: the far pending vertices
     int4 *M[2];            // movers {v, aux, cap, -} [n]
     int4 *TL[3];           // thread-mode scan items {v, log2 cap, offset/4, aux} [n]
     int4 *CL[3];           // chunk scan items {v, chunk<<5 | log2 cap, offset/4, aux} [clcap]
     int64_t clcap;
-    int4 *P[2];            // pending {v, dl, -, -} [2n]
-    int32_t *R[2];         // desire-level recompute candidates; R[1]: violators to evaluate [n]
+    int4 *P[2];            // near pending entries {v, dl, -, -} [2n]
+    int32_t *R[2];         // affected vertices to evaluate; R[1]: those with large tables [n]
     int32_t *arena;        // table-shrink scratch
     int64_t arena_cap;
     int32_t *trace;        // per-round diagnostics records (8 int32 each) or null
