@@ -16,7 +16,7 @@ CSRC = PKG / "csrc"
 INC = PKG.parent / "include"
 OUT_DIR = PKG / "_lib"
 LIB = OUT_DIR / "libplds_gb300.so"
-SOURCES = ["plds_api.cu", "plds_serve.cu", "plds_set.cu", "plds_set_cluster.cu", "plds_tables.cpp"]
+SOURCES = ["plds_api.cu", "plds_serve.cu", "plds_set.cu", "plds_set_cluster.cu", "plds_whole.cu", "plds_tables.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

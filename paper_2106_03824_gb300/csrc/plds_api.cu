@@ -558,15 +558,23 @@ static void raise_smem_limit(K kernel, std::atomic<bool> (&done)[kAttrDevices], 
     if (device >= 0 && device < kAttrDevices) done[device].store(true, std::memory_order_release);
 }
 
-static std::atomic<bool> g_attr_batch[4][kAttrDevices];
+static std::atomic<bool> g_attr_batch[8][kAttrDevices];
+
+// Batches of at most this many edges run as one cooperative launch (k_whole_*): their
+// steps are short, and seven launches with their gaps cost more than the grid barriers
+// between steps at one block per SM.
+constexpr int64_t kWholeB = 16384;
 
 // The step kernels of one batch attempt, in stream order, then pre_done set so
-// that the cooperative kernel starts at the rounds.  Records ev0 before them and
-// evm after them.
+// that the cooperative kernel starts at the rounds (a batch of at most kWholeB edges
+// has none: its cooperative kernel runs everything).  Records ev0 before them and evm
+// after them.
 static void launch_pre(plds *h, GraphCtx &g) {
-    const int blocks = std::max(1, h->num_sms * 8);
+    // a thread per edge or touched endpoint, eight blocks per SM at most
+    const int blocks = (int)std::min<int64_t>(h->num_sms * 8, std::max<int64_t>(h->num_sms, (2 * g.B + kPreThreads - 1) / kPreThreads));
     cudaStream_t s = h->stream;
     cudaEventRecord(h->ev0, s);
+    if (g.B <= kWholeB) return;  // launch_batch runs the whole batch
     int k = 0;
     if (g.B > 0) {
         k_pre_canon_filter<<<blocks, kPreThreads, 0, s>>>(g);
@@ -605,6 +613,11 @@ static void undo_incoming(plds *h, const Ctl &c, const GraphCtx &g) {
     cudaStreamSynchronize(h->stream);
 }
 
+// Device time of the steps of a batch run in one launch, from its own clock readings.
+static int64_t whole_pre_ns(const Ctl &c) {
+    return c.t_rounds > c.t_begin ? (int64_t)(c.t_rounds - c.t_begin) : 0;
+}
+
 static int launch_batch(plds *h, const GraphCtx &g) {
     const int threads = block_threads(h);
     const size_t smem = smem_bytes(threads);
@@ -612,14 +625,15 @@ static int launch_batch(plds *h, const GraphCtx &g) {
     void (*kernel)(const GraphCtx) = what == kDeleteRounds ? k_batch_grid<kDeleteRounds>
                                      : what == kJumpRounds ? k_batch_grid<kJumpRounds>
                                                            : k_batch_grid<kInsertRounds>;
-    raise_smem_limit(kernel, g_attr_batch[what], h->device);
+    if (!g.pre_done)
+        kernel = what == kDeleteRounds ? k_whole_delete : what == kJumpRounds ? k_whole_jump : k_whole_insert;
+    raise_smem_limit(kernel, g_attr_batch[what + (g.pre_done ? 0 : 4)], h->device);
     int occ = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, smem);
     int per_sm = h->tune.blocks_per_sm > 0 ? std::min(h->tune.blocks_per_sm, occ) : 1;
     if (per_sm < 1) return PLDS_EDEVICE;
     dim3 grid(h->num_sms * per_sm), block(threads);
     void *args[] = {(void *)&g};
-    if (!g.pre_done) cudaEventRecord(h->ev0, h->stream);
     cudaError_t e = cudaLaunchCooperativeKernel((const void *)kernel, grid, block, args, smem, h->stream);
     cudaEventRecord(h->ev1, h->stream);
     h->launches++;
@@ -662,9 +676,13 @@ static int run_op(plds *h, const int32_t *edges, int64_t B, int32_t op) {
             h->stamp_base = 1;
         }
         cudaMemsetAsync(h->ctl.p, 0, sizeof(Ctl), h->stream);
-        cudaMemsetAsync(h->hset.p, 0xff, 8 * (size_t)h->hcap, h->stream);
-        if (op == kOpInsert) cudaMemsetAsync(h->bins.p, 0, sizeof(int32_t) * ((size_t)h->T.K + 1), h->stream);
+        // the key set in the size this batch needs (the buffer's is that of the largest so far)
+        const int64_t hc = std::min<int64_t>(h->hcap, pow2_at_least(2 * std::max<int64_t>(B, 1024)));
+        cudaMemsetAsync(h->hset.p, 0xff, 8 * (size_t)hc, h->stream);
+        if (op == kOpInsert && B > kWholeB)
+            cudaMemsetAsync(h->bins.p, 0, sizeof(int32_t) * ((size_t)h->T.K + 1), h->stream);
         GraphCtx g = make_ctx(h, op, dedges, B);
+        g.hcap = hc;
         h->stamp_base += h->T.K + 2;
         launch_pre(h, g);
         int rc = launch_batch(h, g);
@@ -677,7 +695,8 @@ static int run_op(plds *h, const int32_t *edges, int64_t B, int32_t op) {
         }
         float ms = 0.f;
         if (cudaEventElapsedTime(&ms, h->ev0, h->ev1) == cudaSuccess) h->last.kernel_ns += (int64_t)(ms * 1e6);
-        if (cudaEventElapsedTime(&ms, h->ev0, h->evm) == cudaSuccess) h->last.pre_ns += (int64_t)(ms * 1e6);
+        if (!g.pre_done) h->last.pre_ns += whole_pre_ns(h->host_ctl);
+        else if (cudaEventElapsedTime(&ms, h->ev0, h->evm) == cudaSuccess) h->last.pre_ns += (int64_t)(ms * 1e6);
         cudaGetLastError();
         const Ctl &c = h->host_ctl;
         h->last.err_bits = c.err;
@@ -1543,7 +1562,8 @@ extern "C" int plds_batch_static(plds_t *h, const int32_t *edges, int64_t B, int
     const int64_t hc = std::min<int64_t>(kStaticHcap, pow2_at_least(2 * std::max<int64_t>(B, 1024)));
     cudaMemsetAsync(h->ctl.p, 0, sizeof(Ctl), h->stream);
     cudaMemsetAsync(base + kStOffHset, 0xff, 8 * (size_t)hc, h->stream);
-    if (op == kOpInsert) cudaMemsetAsync(h->bins.p, 0, sizeof(int32_t) * ((size_t)h->T.K + 1), h->stream);
+    if (op == kOpInsert && B > kWholeB)
+        cudaMemsetAsync(h->bins.p, 0, sizeof(int32_t) * ((size_t)h->T.K + 1), h->stream);
     GraphCtx g = make_ctx(h, op, dedges, B);
     g.hset = reinterpret_cast<unsigned long long *>(base + kStOffHset);
     g.hcap = hc;
@@ -1565,7 +1585,8 @@ extern "C" int plds_batch_static(plds_t *h, const int32_t *edges, int64_t B, int
     }
     float ms = 0.f;
     if (cudaEventElapsedTime(&ms, h->ev0, h->ev1) == cudaSuccess) h->last.kernel_ns = (int64_t)(ms * 1e6);
-    if (cudaEventElapsedTime(&ms, h->ev0, h->evm) == cudaSuccess) h->last.pre_ns = (int64_t)(ms * 1e6);
+    if (!g.pre_done) h->last.pre_ns = whole_pre_ns(h->host_ctl);
+    else if (cudaEventElapsedTime(&ms, h->ev0, h->evm) == cudaSuccess) h->last.pre_ns = (int64_t)(ms * 1e6);
     cudaGetLastError();
     const Ctl &c = h->host_ctl;
     h->last.err_bits = c.err;

@@ -3681,6 +3681,11 @@ __device__ __forceinline__ void run_batch(Team &T, const GraphCtx &g, const Batc
         g.ctl->trace_n = 1;
         tmark[nmark++] = global_ns();
     }
+    if constexpr (!kRoundsOnly && kWhat != kAnyRounds) {  // a whole batch in one launch
+        if (T.leader()) g.ctl->t_begin = global_ns();
+        if (kWhat != kDeleteRounds)
+            for (int k = T.tid(); k <= g.K; k += T.nthreads()) g.bins[k] = 0;
+    }
     if constexpr (kRoundsOnly) {  // a step kernel that failed stops the rounds too
         if (ld_volatile(&g.ctl->err)) return;
     } else if (in.B > 0) {
@@ -3711,6 +3716,7 @@ __device__ __forceinline__ void run_batch(Team &T, const GraphCtx &g, const Batc
             step_apply_insert(T, g);
             if (!T.sync()) return;
             if (tr) tmark[nmark++] = global_ns();
+            if (kWhat != kAnyRounds && T.leader()) g.ctl->t_rounds = global_ns();
         }
         if constexpr (kMayJump) {
             if (kWhat == kJumpRounds || g.jump) {
@@ -3747,6 +3753,7 @@ __device__ __forceinline__ void run_batch(Team &T, const GraphCtx &g, const Batc
             pre_shrink_c(T, g);
             if (!T.sync()) return;
             if (tr) tmark[nmark++] = global_ns();
+            if (kWhat != kAnyRounds && T.leader()) g.ctl->t_rounds = global_ns();
         }
         RoundStage st = stage_setup(sh_stage, stage_shift);
         DelState ds;

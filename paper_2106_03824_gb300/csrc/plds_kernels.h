@@ -9,6 +9,11 @@
 
 namespace pl {
 
+// A small batch in one launch (insertion, insertion by the jump variant, deletion).
+__global__ void k_whole_insert(const __grid_constant__ GraphCtx g);
+__global__ void k_whole_jump(const __grid_constant__ GraphCtx g);
+__global__ void k_whole_delete(const __grid_constant__ GraphCtx g);
+
 // Batched form: one graph's work of a round.
 struct SetItem {
     GraphCtx half[2];  // 0: insertion half, 1: deletion half

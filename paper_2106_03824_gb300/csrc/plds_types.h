@@ -103,6 +103,8 @@ struct Ctl {
     // finished its share of an insertion phase
     unsigned long long tw_max[2];
     unsigned long long tw_min_c[2];  // complement of the earliest time (zero means none)
+    // a whole batch in one launch: device time at its start and at the first round
+    unsigned long long t_begin, t_rounds;
     unsigned long long st[kStCount];
 };
 
