@@ -45,7 +45,7 @@ template <int kWhat>
 __global__ void __launch_bounds__(512) k_batch_grid(const __grid_constant__ GraphCtx g) {
     extern __shared__ int32_t sh[];
     GridTeam T{g.ctl, g.wait_limit_ns, g.barrier_sleep_ns};
-    run_batch<GridTeam, true, kWhat>(T, g, BatchIn{g.edges, g.B, g.op, g.stamp_base}, sh, 0);
+    run_batch<GridTeam, true, kWhat>(T, g, BatchIn{g.edges, g.B, g.op, g.stamp_base, g.hcap}, sh, 0);
 }
 
 // The steps before the level rounds (preprocessing, table growth and shrinking,
@@ -61,7 +61,7 @@ constexpr int kPreThreads = 256;
 
 __global__ void __launch_bounds__(kPreThreads) k_pre_canon_filter(const __grid_constant__ GraphCtx g) {
     PRE_SCRATCH;
-    pre_canon_filter(T, g, BatchIn{g.edges, g.B, g.op, g.stamp_base}, sh_res);
+    pre_canon_filter(T, g, BatchIn{g.edges, g.B, g.op, g.stamp_base, g.hcap}, sh_res);
 }
 
 // After an insertion batch was rejected for an id outside [0, n): the incoming
@@ -380,6 +380,11 @@ static bool ensure_batch_scratch(plds *h, int64_t B) {
     return true;
 }
 
+// Key-set entries that a batch of B edges uses.
+static int64_t key_set_size(const plds *h, int64_t B) {
+    return std::min<int64_t>(h->hcap, pow2_at_least(2 * std::max<int64_t>(B, 1024)));
+}
+
 static int block_threads(const plds *h) { return h->tune.block_threads > 0 ? h->tune.block_threads : 512; }
 
 // Dynamic shared memory of a batch kernel block: group tables, scan scratch,
@@ -677,7 +682,7 @@ static int run_op(plds *h, const int32_t *edges, int64_t B, int32_t op) {
         }
         cudaMemsetAsync(h->ctl.p, 0, sizeof(Ctl), h->stream);
         // the key set in the size this batch needs (the buffer's is that of the largest so far)
-        const int64_t hc = std::min<int64_t>(h->hcap, pow2_at_least(2 * std::max<int64_t>(B, 1024)));
+        const int64_t hc = key_set_size(h, B);
         cudaMemsetAsync(h->hset.p, 0xff, 8 * (size_t)hc, h->stream);
         if (op == kOpInsert && B > kWholeB)
             cudaMemsetAsync(h->bins.p, 0, sizeof(int32_t) * ((size_t)h->T.K + 1), h->stream);
@@ -1853,6 +1858,7 @@ extern "C" int plds_set_update(plds_set_t *s, const int32_t *edges, const int64_
                 }
                 GraphCtx g = make_ctx(h, half == 0 ? kOpInsert : kOpDelete, dedges + 2 * offsets[2 * gi + half], b);
                 g.ctl = dctl + 2 * j + half;
+                g.hcap = key_set_size(h, b);
                 g.trace = nullptr;
                 g.trace_cap = 0;
                 s->h_items[j].half[half] = g;
@@ -2198,7 +2204,12 @@ struct plds_server {
     bool running = false;
     int64_t next_seq = 0;  // sequence number of the next submitted request
     int64_t done_seq = 0;  // all sequence numbers below have been collected
-    int64_t idle_ns = 20ll * 1000 * 1000;
+    // An idle loop holds every SM (a server on another graph, or a kernel that needs
+    // the shared memory, waits for it) and a relaunch takes the host ~20 us: 2 ms.
+    int64_t idle_ns = 2ll * 1000 * 1000;
+    ServeExit *exit = nullptr;  // pinned, mapped
+    ServeExit *exit_dev = nullptr;
+    int occ_threads = 0, occ = 0;  // resident blocks per SM of the loop at occ_threads
     int64_t merge_cap = 0;        // edges per merged batch (0: unchanged boundaries)
     int64_t pool_limit = 0;       // bytes the adjacency pool may take (0: free HBM only)
     int64_t pool_used = 0;        // adjacency slots handed out, as last reported
@@ -2227,9 +2238,11 @@ static int server_launch(plds_server *sv) {
     const size_t smem = smem_bytes(threads);
     static std::atomic<bool> attr_serve[kAttrDevices];
     raise_smem_limit(k_serve, attr_serve, h->device);
-    int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_serve, threads, smem);
-    const int per_sm = h->tune.blocks_per_sm > 0 ? std::min(h->tune.blocks_per_sm, occ) : 1;
+    if (sv->occ_threads != threads) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&sv->occ, k_serve, threads, smem);
+        sv->occ_threads = threads;
+    }
+    const int per_sm = h->tune.blocks_per_sm > 0 ? std::min(h->tune.blocks_per_sm, sv->occ) : 1;
     if (per_sm < 1) return PLDS_EDEVICE;
     GraphCtx g = make_ctx(h, kOpInsert, nullptr, 0);
     g.trace = nullptr;
@@ -2238,7 +2251,9 @@ static int server_launch(plds_server *sv) {
     // (blocks leave a barrier early once the error word is set): start clean.
     cudaMemsetAsync(h->ctl.p, 0, sizeof(Ctl), sv->run);
     cudaMemsetAsync(&P<ServeCtl>(sv->sc)->exit_reason, 0, sizeof(int32_t) * 2, sv->run);
-    ServeArgs a{sv->ring_dev, sv->slots, sv->idle_ns, P<ServeCtl>(sv->sc), P<double>(h->powtab), P<int2>(sv->ebuf)};
+    ServeArgs a{sv->ring_dev, sv->slots, sv->idle_ns, P<ServeCtl>(sv->sc), P<double>(h->powtab), P<int2>(sv->ebuf),
+                sv->exit_dev};
+    *(volatile int32_t *)&sv->exit->reason = kExitNone;
     void *args[] = {(void *)&g, (void *)&a};
     if (cudaLaunchCooperativeKernel((const void *)k_serve, dim3(h->num_sms * per_sm), dim3(threads), args, smem,
                                     sv->run) != cudaSuccess) {
@@ -2259,22 +2274,28 @@ static int server_service(plds_server *sv) {
     cudaGetLastError();
     sv->running = false;
     plds *h = sv->h;
-    ServeCtl c{};
-    if (cudaMemcpy(&c, sv->sc.p, sizeof(ServeCtl), cudaMemcpyDeviceToHost) != cudaSuccess) {
-        cudaGetLastError();
-        h->poisoned = true;
-        return PLDS_EDEVICE;
+    ServeExit c = *sv->exit;
+    if (c.reason == kExitNone) {  // stopped by an error: read the control blocks
+        ServeCtl sc{};
+        Ctl hc{};
+        if (cudaMemcpy(&sc, sv->sc.p, sizeof(ServeCtl), cudaMemcpyDeviceToHost) != cudaSuccess ||
+            cudaMemcpy(&hc, h->ctl.p, sizeof(Ctl), cudaMemcpyDeviceToHost) != cudaSuccess) {
+            cudaGetLastError();
+            h->poisoned = true;
+            return PLDS_EDEVICE;
+        }
+        h->stamp_base = sc.stamp_next;
+        if (hc.err & kErrTimeout) {
+            h->poisoned = true;
+            return PLDS_ETIMEOUT;
+        }
+        c.reason = sc.exit_reason;
+        c.stamp_next = sc.stamp_next;
+        c.head = sc.head;
+        c.grow_total = sc.grow_total;
     }
     h->stamp_base = c.stamp_next;
-    Ctl hc{};
-    cudaMemcpy(&hc, h->ctl.p, sizeof(Ctl), cudaMemcpyDeviceToHost);
-    if (hc.err & kErrTimeout) {
-        h->poisoned = true;
-        return PLDS_ETIMEOUT;
-    }
-    int32_t reset = kExitNone;
-    cudaMemcpy(&reinterpret_cast<ServeCtl *>(sv->sc.p)->exit_reason, &reset, 4, cudaMemcpyHostToDevice);
-    if (c.exit_reason == kExitNeedPool) {
+    if (c.reason == kExitNeedPool) {
         const int64_t saved = h->pool_limit;
         h->pool_limit = sv->pool_limit;
         int rc = grow_pool(h, (int64_t)c.grow_total);
@@ -2328,6 +2349,7 @@ static void server_free(plds_server *sv) {
     for (int32_t *p : sv->stage)
         if (p) cudaFreeHost(p);
     if (sv->qbuf) cudaFreeHost(sv->qbuf);
+    if (sv->exit) cudaFreeHost(sv->exit);
     if (sv->h) {
         dev_free(sv->h, sv->sc);
         dev_free(sv->h, sv->ebuf);
@@ -2360,6 +2382,8 @@ extern "C" plds_server_t *plds_server_create(plds_t *h, int32_t slots, int64_t m
               cudaEventCreateWithFlags(&sv->done, cudaEventDisableTiming) == cudaSuccess &&
               cudaHostAlloc((void **)&sv->ring, sizeof(ReqSlot) * slots, cudaHostAllocMapped) == cudaSuccess &&
               cudaHostGetDevicePointer((void **)&sv->ring_dev, sv->ring, 0) == cudaSuccess &&
+              cudaHostAlloc((void **)&sv->exit, sizeof(ServeExit), cudaHostAllocMapped) == cudaSuccess &&
+              cudaHostGetDevicePointer((void **)&sv->exit_dev, sv->exit, 0) == cudaSuccess &&
               cudaHostAlloc((void **)&sv->qbuf, sizeof(double) * (size_t)h->n, cudaHostAllocMapped) == cudaSuccess &&
               cudaHostGetDevicePointer((void **)&sv->qbuf_dev, sv->qbuf, 0) == cudaSuccess;
     if (ok) {

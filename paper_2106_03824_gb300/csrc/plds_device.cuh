@@ -531,7 +531,7 @@ template <class Team>
 __device__ __forceinline__ void pre_canon(Team &T, const GraphCtx &g, const BatchIn &in, unsigned long long *sh) {
     const int2 *e = reinterpret_cast<const int2 *>(in.edges);
     unsigned long long loops = 0;
-    const int64_t mask = g.hcap - 1, stride = (int64_t)T.nblocks() * blockDim.x;
+    const int64_t mask = in.hcap - 1, stride = (int64_t)T.nblocks() * blockDim.x;
     for (int64_t b0 = (int64_t)T.bid() * blockDim.x; b0 < in.B; b0 += stride) {
         const int64_t i = b0 + threadIdx.x;
         bool fresh = false;
@@ -609,7 +609,7 @@ __device__ __forceinline__ void pre_canon_filter(Team &T, const GraphCtx &g, con
     const int2 *e = reinterpret_cast<const int2 *>(in.edges);
     const int32_t stouch = in.stamp_base;
     unsigned long long loops = 0, filtered = 0;
-    const int64_t mask = g.hcap - 1, stride = (int64_t)T.nblocks() * blockDim.x;
+    const int64_t mask = in.hcap - 1, stride = (int64_t)T.nblocks() * blockDim.x;
     for (int64_t b0 = (int64_t)T.bid() * blockDim.x; b0 < in.B; b0 += stride) {
         const int64_t i = b0 + threadIdx.x;
         bool fresh = false;

@@ -72,6 +72,15 @@ struct ServeCtl {  // device memory
     int32_t seg_bad[kMaxSeg];
 };
 
+// Why and where the loop stopped, written into pinned host memory as it leaves
+// (reason kExitNone: not written, an error stopped it).
+struct ServeExit {
+    int32_t reason;
+    int32_t stamp_next;
+    int64_t head;
+    unsigned long long grow_total;
+};
+
 struct ServeArgs {
     ReqSlot *ring;  // device pointer of the pinned ring
     int32_t slots;
@@ -79,6 +88,7 @@ struct ServeArgs {
     ServeCtl *sc;
     const double *powtab;
     int2 *ebuf;  // gathered edges of a merged batch [max_batch]
+    ServeExit *exit;
 };
 
 __global__ void k_serve(const __grid_constant__ GraphCtx base, const ServeArgs a);

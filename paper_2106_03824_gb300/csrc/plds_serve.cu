@@ -62,6 +62,25 @@ __device__ void serve_gather(GridTeam &T, const ServeCtl *sc, int ns, const int6
     }
 }
 
+// Key-set entries the current batch needs: a power of two of at least twice its edges
+// (the buffer is sized for max_batch).
+__device__ __forceinline__ int64_t serve_hcap(const GraphCtx &base, const ServeCtl *sc) {
+    const int64_t B = max((long long)1024, (long long)(*(volatile const int32_t *)&sc->nseg > 0
+                                                           ? *(volatile const int64_t *)&sc->seg_total
+                                                           : *(volatile const int64_t *)&sc->cur.B));
+    return min((long long)base.hcap, 2ll << (64 - __clzll(B - 1)));
+}
+
+// Leader: the loop is about to leave.
+__device__ __forceinline__ void serve_leave(const ServeArgs &a, const ServeCtl *sc, int32_t reason) {
+    volatile ServeExit *x = a.exit;
+    x->stamp_next = sc->stamp_next;
+    x->head = sc->head;
+    x->grow_total = sc->grow_total;
+    __threadfence_system();
+    x->reason = reason;
+}
+
 __global__ void __launch_bounds__(512) k_serve(const __grid_constant__ GraphCtx base, const ServeArgs a) {
     extern __shared__ int32_t sh[];
     __shared__ int64_t s_off[kMaxSeg + 1];
@@ -83,17 +102,19 @@ __global__ void __launch_bounds__(512) k_serve(const __grid_constant__ GraphCtx 
             } else {
                 sc->cmd = 0;
                 sc->exit_reason = kExitIdle;
+                serve_leave(a, sc, kExitIdle);
             }
             __threadfence();
         }
         if (!T.sync()) return;
         if (ld_volatile(&sc->cmd) == 0) return;
+        const int64_t hcap = serve_hcap(base, sc);  // (before rejected requests are dropped)
         // a fresh control block and key set for this request (the barrier words stay)
         {
             int32_t *cw = reinterpret_cast<int32_t *>(base.ctl);
             const int first = (int)(offsetof(Ctl, err) / 4);
             for (int k = T.tid() + first; k < (int)(sizeof(Ctl) / 4); k += T.nthreads()) cw[k] = 0;
-            for (int64_t k = T.tid(); k < base.hcap; k += T.nthreads()) base.hset[k] = kEmptyKey;
+            for (int64_t k = T.tid(); k < hcap; k += T.nthreads()) base.hset[k] = kEmptyKey;
             for (int k = T.tid(); k <= base.K; k += T.nthreads()) base.bins[k] = 0;
             if (sc->stamp_next + 2 * base.K + 8 >= 0x7fffffff) {  // stamps wrap: clear them
                 for (int k = T.tid(); k < base.n; k += T.nthreads()) base.stamp[k] = 0;
@@ -139,7 +160,7 @@ __global__ void __launch_bounds__(512) k_serve(const __grid_constant__ GraphCtx 
         } else {
             const BatchIn in{ns > 0 ? reinterpret_cast<const int32_t *>(a.ebuf) : req.edges,
                              ns > 0 ? *(volatile const int64_t *)&sc->seg_total : req.B,
-                             req.op == kReqInsert ? kOpInsert : kOpDelete, sbase};
+                             req.op == kReqInsert ? kOpInsert : kOpDelete, sbase, hcap};
             run_batch(T, base, in, sh, 0);
         }
         const bool ok = T.sync();
@@ -149,6 +170,7 @@ __global__ void __launch_bounds__(512) k_serve(const __grid_constant__ GraphCtx 
                 sc->exit_reason = kExitNeedPool;
                 sc->grow_total = base.ctl->grow_total;
                 sc->stamp_next = sbase + base.K + 2;
+                serve_leave(a, sc, kExitNeedPool);
             } else {
                 const int nr = ns > 0 ? ns : 1;
                 const uint64_t t_end = global_ns();

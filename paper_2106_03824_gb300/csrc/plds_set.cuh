@@ -24,7 +24,7 @@ __device__ __forceinline__ void set_graph(Team &T, GraphCtx &gsh, const SetItem 
             for (int k = T.tid(); k <= gsh.K; k += T.nthreads()) gsh.bins[k] = 0;
         barrier();
         T.ctl = gsh.ctl;
-        run_batch(T, gsh, BatchIn{gsh.edges, gsh.B, gsh.op, gsh.stamp_base}, sh, kSetStageShift);
+        run_batch(T, gsh, BatchIn{gsh.edges, gsh.B, gsh.op, gsh.stamp_base, gsh.hcap}, sh, kSetStageShift);
         barrier();
         const int32_t err = ld_volatile(&gsh.ctl->err);
         barrier();

@@ -174,6 +174,7 @@ struct BatchIn {
     int64_t B;
     int32_t op;            // kOpInsert / kOpDelete
     int32_t stamp_base;    // stamps of this batch are stamp_base + 1 .. stamp_base + K + 1
+    int64_t hcap;          // entries of the key set in use (power of two)
 };
 
 }  // namespace pl
