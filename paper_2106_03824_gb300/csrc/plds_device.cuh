@@ -1013,6 +1013,7 @@ constexpr int kStageF = 2048, kStageTL = 1024, kStageCL = 2048, kStagePK = 1024;
 struct RoundStage {
     Stage<int32_t> f, q;      // q shares tl's buffer (f's while tl fills)
     Stage<int4> tl, cl, pk;
+    int32_t tcap;     // insertion: tables up to this many slots are scanned by one thread next
     int32_t *movers;  // shared mover count of the block
     int32_t *bmin;    // shared minimum pending level of the block's near entries
     int32_t *qmin;    // and of its far vertices
@@ -1190,7 +1191,7 @@ __device__ __forceinline__ void enqueue_ins(const GraphCtx &g, const RoundStage 
     if (mm == 0) return;
     if (lane == __ffs(mm) - 1) atomicAdd(st.movers, __popc(mm));
     const bool list = is_mover && ilen >= 0;
-    const bool small = is_mover && !list && c <= g.thread_max_cap;
+    const bool small = is_mover && !list && c <= st.tcap;
     const int lg = (is_mover && !list) ? __ffs(c) - 1 : 31;
     const int32_t goff = list ? ioff4 : (int32_t)(off >> 2);
     stage_push(st.tl, small, make_int4(v, lg, goff, 0));
@@ -1505,6 +1506,17 @@ __device__ __forceinline__ void ins_test_initial(Team &T, const GraphCtx &g, con
         }
         enqueue_marked(g, st, mk, v, k1, wsm);
     }
+}
+
+// Tables that the next phase scans by a thread each, unless the caller set the cutoff:
+// the more movers a phase has for each warp, the more a warp's step per table costs.
+// (Mean phase times on R-MAT 20, 10^6-edge batches, cutoff 8 / 16 / 32: at 4,096-8,192
+// movers 15.9 / 16.0 / 16.7 us, 8,192-16,384 19.5 / 18.5 / 18.5, 16,384-32,768 23.2 /
+// 21.1 / 20.3, 32,768-65,536 34.9 / 24.8 / 19.9; R-MAT 18 at 257-1,024 11.3 / 11.4 /
+// 12.1; a 1.4 M-vertex road grid, all of it moving, 116.6 / 96.0 / 95.8.)
+__device__ __forceinline__ int32_t ins_thread_cap(const GraphCtx &g, int32_t m, int nwarps) {
+    if (!g.tcap_auto) return g.thread_max_cap;
+    return 2 * m <= nwarps ? 8 : m <= 7 * nwarps ? 16 : 32;
 }
 
 // Where the insertion rounds stand (the same in every thread of the team).
@@ -1905,6 +1917,7 @@ __device__ __forceinline__ bool ins_phases_local(const GraphCtx &g, const int32_
         st.cl.gcnt = h + 5;
         st.cl.glist = g.CL[nxt];
         st.cl.gcap = g.clcap;
+        st.tcap = ins_thread_cap(g, s.m, T.nwarps());
         st.movers = h + 6;
         st.ff = h + 7;
         st.ff64 = reinterpret_cast<unsigned long long *>(h + 10);
@@ -1997,6 +2010,7 @@ __device__ __forceinline__ bool ins_grid_phase(Team &T, const GraphCtx &g, const
     st.cl.gcnt = &g.ctl->icl[nxt];
     st.cl.glist = g.CL[nxt];
     st.cl.gcap = g.clcap;
+    st.tcap = ins_thread_cap(g, s.m, T.nwarps());
     const bool has_init = s.scan && s.ninit == s.l + 1;
     ins_phase_work(T, g, st, sh_upmax, wsm, s, s_lo, s_hi, g.TL[cur], g.CL[cur], a);
     const uint64_t t_work = (g.trace && T.leader()) ? global_ns() : 0;

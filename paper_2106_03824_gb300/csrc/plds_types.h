@@ -121,7 +121,7 @@ struct GraphCtx {
     int32_t list_cap;      // insertion: chunk-scanned tables from this size on get an up-list
     int32_t jump;          // insertion violators move straight to their targets (jump variant)
     int32_t pre_done;      // the steps before the rounds ran as separate kernels (plain form)
-    int32_t pad3;
+    int32_t tcap_auto;     // insertion: thread_max_cap is a default, each phase picks its own
     int64_t wait_limit_ns;
     const int32_t *upmax;  // [G]
     const int32_t *dnmin;  // [G]
