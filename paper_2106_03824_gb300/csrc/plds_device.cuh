@@ -89,9 +89,11 @@ struct GridTeam {
     // phase starts with, written to shared memory -- while lane 0 reads the error
     // word into *ok_slot: one round of loads for the block instead of a read of
     // the error word by every thread followed by the phase's own first loads.
-    template <class F>
-    __device__ __forceinline__ bool sync_fetch(F fetch, int32_t *ok_slot) {
+    // idle() runs on thread 32 meanwhile.
+    template <class F, class I>
+    __device__ __forceinline__ bool sync_fetch(F fetch, int32_t *ok_slot, I idle) {
         __syncthreads();
+        if (threadIdx.x == 32) idle();
         if (threadIdx.x < 32) {
             if (threadIdx.x == 0) arrive_wait();
             __syncwarp();  // orders warp 0's loads after the acquire
@@ -155,9 +157,10 @@ struct ClusterTeam {
         if (leader()) write();
         return sync();
     }
-    template <class F>
-    __device__ __forceinline__ bool sync_fetch(F fetch, int32_t *ok_slot) {
+    template <class F, class I>
+    __device__ __forceinline__ bool sync_fetch(F fetch, int32_t *ok_slot, I idle) {
         barrier();
+        if (threadIdx.x == 32) idle();
         if (threadIdx.x < 32) {
             if (threadIdx.x == 0) *ok_slot = ld_volatile(&ctl->err);
             fetch((int)threadIdx.x);
@@ -1727,6 +1730,34 @@ __device__ __forceinline__ void ins_scan_chunks(Team &T, const GraphCtx &g, cons
     }
 }
 
+// Up to G 16-byte groups of the lanes' thread-mode movers, from group j0 of the ng at
+// int4 offset goff: effects, marks, neighbours left on l (cnt_l) and live slots (ideg).
+template <int G>
+__device__ __forceinline__ void ins_scan_slots(const GraphCtx &g, const RoundStage &st, int32_t *wsm, int32_t *mbuf,
+                                               int &mc, const InsState &s, int32_t cut_next, int32_t goff, int ng,
+                                               int j0, int &cnt_l, int &ideg, int32_t &low, ScanCount &a) {
+    const int4 *pool4 = reinterpret_cast<const int4 *>(g.slots);
+    int32_t ws[4 * G], lv[4 * G];
+#pragma unroll
+    for (int j = 0; j < G; ++j) {
+        const int4 s4 = j0 + j < ng ? pool4[goff + j0 + j] : empty4();
+        ws[4 * j] = s4.x; ws[4 * j + 1] = s4.y; ws[4 * j + 2] = s4.z; ws[4 * j + 3] = s4.w;
+    }
+#pragma unroll
+    for (int q = 0; q < 4 * G; ++q) lv[q] = valid_id(g, ws[q]) ? g.level[ws[q]] : 0;
+    unsigned push = 0, keep = 0;
+    int c[G];
+#pragma unroll
+    for (int j = 0; j < G; ++j) c[j] = 0;
+#pragma unroll
+    for (int q = 0; q < 4 * G; ++q) ideg += ws[q] >= 0;
+    ins_effects(g, ws, lv, s.l, s.lmo, phase_flag(s.k), phase_flag(s.k + 1), cut_next, c, low, push, keep, a.aff);
+#pragma unroll
+    for (int j = 0; j < G; ++j) cnt_l += c[j];
+    a.scanned += 4 * max(0, min(G, ng - j0));
+    marks_add(g, st, push, ws, mbuf, mc, s.k + 1, wsm);
+}
+
 // The work of phase k: the initial candidates S[s_lo, s_hi) (on l in a test phase,
 // on l + 1 in a scan phase), and in a scan phase the effects of the movers of l,
 // items tl[0..s.tlc) and cl[0..s.clc).
@@ -1740,7 +1771,6 @@ __device__ __forceinline__ void ins_phase_work(Team &T, const GraphCtx &g, const
         ins_test_initial(T, g, st, s_lo, s_hi, l, sh_upmax[l / g.Lg], wsm, 0, k + 1);
         return;
     }
-    const int4 *pool4 = reinterpret_cast<const int4 *>(g.slots);
     int32_t *mbuf = wsm + 160;
     int mc = 0;
     int32_t low = kInf;  // lowest level above l of a neighbour of a mover that is no mover
@@ -1748,7 +1778,7 @@ __device__ __forceinline__ void ins_phase_work(Team &T, const GraphCtx &g, const
     const int32_t cut_next = sh_upmax[(l + 1) / g.Lg];
     if (s_lo < s_hi)  // initial candidates on l + 1
         ins_test_initial(T, g, st, s_lo, s_hi, l + 1, cut_next, wsm, T.nwarps() / 2, k + 1);
-    // thread-mode movers: up to 4 groups (16 slots) per pass, loads issued together
+    // thread-mode movers
     for (int i0 = T.srank() * 32; i0 < tlc; i0 += T.nwarps() * 32) {
         const int i = i0 + lane;
         const int4 it = i < tlc ? tl[i] : make_int4(0, 0, 0, 0);
@@ -1757,23 +1787,11 @@ __device__ __forceinline__ void ins_phase_work(Team &T, const GraphCtx &g, const
         const int32_t up_v = have ? g.up[it.x] : 0;  // issued with the slot loads
         const int maxg = (int)__reduce_max_sync(kFull, (unsigned)ng);
         int cnt_l = 0, ideg = 0;
-        for (int j0 = 0; j0 < maxg; j0 += 4) {
-            int32_t ws[16], lv[16];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int4 s4 = j0 + j < ng ? pool4[it.z + j0 + j] : empty4();
-                ws[4 * j] = s4.x; ws[4 * j + 1] = s4.y; ws[4 * j + 2] = s4.z; ws[4 * j + 3] = s4.w;
-            }
-#pragma unroll
-            for (int q = 0; q < 16; ++q) lv[q] = valid_id(g, ws[q]) ? g.level[ws[q]] : 0;
-            unsigned push = 0, keep = 0;
-            int c4[4] = {0, 0, 0, 0};
-#pragma unroll
-            for (int q = 0; q < 16; ++q) ideg += ws[q] >= 0;
-            ins_effects(g, ws, lv, l, s.lmo, fcur, fnext, cut_next, c4, low, push, keep, a.aff);
-            cnt_l += c4[0] + c4[1] + c4[2] + c4[3];
-            a.scanned += 4 * max(0, min(4, ng - j0));
-            marks_add(g, st, push, ws, mbuf, mc, k + 1, wsm);
+        if (maxg <= 2) {
+            ins_scan_slots<2>(g, st, wsm, mbuf, mc, s, cut_next, it.z, ng, 0, cnt_l, ideg, low, a);
+        } else {
+            for (int j0 = 0; j0 < maxg; j0 += 4)
+                ins_scan_slots<4>(g, st, wsm, mbuf, mc, s, cut_next, it.z, ng, j0, cnt_l, ideg, low, a);
         }
         a.visits += ideg;
         a.upv += up_v;
@@ -1781,7 +1799,10 @@ __device__ __forceinline__ void ins_phase_work(Team &T, const GraphCtx &g, const
         ff_note(st, again, up_v - cnt_l, ideg);
         enqueue_ins(g, st, again, it.x, have ? 1 << it.y : 0, (int64_t)it.z * 4, -1, 0, 0, k + 1, wsm);
     }
-    if (!Team::kGrid && s.clc <= T.nwarps()) ins_scan_chunks<1>(T, g, st, wsm, mbuf, mc, s, cut_next, cl, low, a);
+    // as many items per warp step as the list gives each warp: the step's instructions, not
+    // its loads, set the time of a phase in which a warp has one item
+    if (s.clc <= T.nwarps()) ins_scan_chunks<1>(T, g, st, wsm, mbuf, mc, s, cut_next, cl, low, a);
+    else if (s.clc <= 2 * T.nwarps()) ins_scan_chunks<2>(T, g, st, wsm, mbuf, mc, s, cut_next, cl, low, a);
     else ins_scan_chunks<4>(T, g, st, wsm, mbuf, mc, s, cut_next, cl, low, a);
     marks_flush(g, st, mbuf, mc, k + 1, wsm);
     low = (int32_t)__reduce_min_sync(kFull, (unsigned)low);
@@ -2022,59 +2043,66 @@ __device__ __forceinline__ bool ins_grid_phase(Team &T, const GraphCtx &g, const
             atomicMax(&g.ctl->tw_min_c[k & 1], ~tb);
         }
     }
-    stage_flush_round(g, st, 6u);
-    if (threadIdx.x == 0) {
-        if (*st.movers) {
-            atomicAdd(&g.ctl->imcnt[nxt], *st.movers);
-            *st.movers = 0;
-        }
-        if (st.ff[0]) {  // the block's climbing movers (complements: zero means none)
-            atomicAdd(&g.ctl->icont[nxt], st.ff[0]);
-            atomicMax(&g.ctl->iminup_c[nxt], kInf - st.ff[1]);
-            atomicAdd(&g.ctl->isdeg[nxt], st.ff64[0]);
-            atomicAdd(&g.ctl->isup[nxt], st.ff64[1]);
-            st.ff[0] = 0;
-            st.ff[1] = kInf;
-            st.ff64[0] = 0;
-            st.ff64[1] = 0;
-        }
-        if (st.ff[2] < kInf) {
-            atomicMax(&g.ctl->ilow_c[nxt], kInf - st.ff[2]);
-            st.ff[2] = kInf;
-        }
+    // publish: the lists' global ranges (a warp each) and the block's totals (a lane each)
+    // are taken together, then the block copies its staged items out
+    __syncthreads();
+    const int nt = min(st.tl.hdr[0], st.tl.hdr[1]), nc = min(st.cl.hdr[0], st.cl.hdr[1]);
+    if (threadIdx.x == 32) stage_reserve_global(g, st.tl, st.tmp + 1);
+    if (threadIdx.x == 64) stage_reserve_global(g, st.cl, st.tmp + 2);
+    if (threadIdx.x >= 96 && threadIdx.x < 102) {  // (complements where zero means none)
+        const int j = threadIdx.x - 96;
+        if (j == 0 && *st.movers) atomicAdd(&g.ctl->imcnt[nxt], *st.movers);
+        if (j == 1 && st.ff[0]) atomicAdd(&g.ctl->icont[nxt], st.ff[0]);
+        if (j == 2 && st.ff[1] < kInf) atomicMax(&g.ctl->iminup_c[nxt], kInf - st.ff[1]);
+        if (j == 3 && st.ff[2] < kInf) atomicMax(&g.ctl->ilow_c[nxt], kInf - st.ff[2]);
+        if (j == 4 && st.ff64[0]) atomicAdd(&g.ctl->isdeg[nxt], st.ff64[0]);
+        if (j == 5 && st.ff64[1]) atomicAdd(&g.ctl->isup[nxt], st.ff64[1]);
     }
+    __syncthreads();
+    const int bt = st.tmp[1], bc = st.tmp[2];
+    for (int i = threadIdx.x; i < nt; i += blockDim.x)
+        if (bt + i < st.tl.gcap) st.tl.glist[bt + i] = st.tl.buf[i];
+    for (int i = threadIdx.x; i < nc; i += blockDim.x)
+        if (bc + i < st.cl.gcap) st.cl.glist[bc + i] = st.cl.buf[i];
     // the level the next phase scans if it has movers, and its initial-candidate
     // entry; warp 0 fetches them with the next phase's counts and each warp's
-    // first chunk item while it passes the barrier
+    // first chunk item while it passes the barrier: one load per lane (a branch per
+    // word would take a round trip each), word j from lane 16 + j
     const int spos2 = has_init ? s.spos + 1 : s.spos;
     const int32_t l2 = s.scan ? s.l + 1 : s.l;
     const int4 *cl_next = g.CL[nxt];
     const bool passed = T.sync_fetch(
         [&](int ln) {
-            if (ln < (int)(blockDim.x >> 5)) {  // warp ln of the block: its first chunk item
-                const int cr = T.nwarps() - 1 - (ln * T.nblocks() + T.bid());  // warp ln's srank
-                st.ph4[ln] = cr < g.clcap ? cl_next[cr] : make_int4(0, 0, 0, 0);
-            } else if (ln == 16) {
-                st.phs[1] = g.ctl->imcnt[nxt];
-            } else if (ln == 17) {
-                st.phs[2] = g.ctl->itl[nxt];
-            } else if (ln == 18) {
-                st.phs[3] = g.ctl->icl[nxt];
-            } else if (ln == 19) {
-                st.phs[4] = spos2 < nlev ? g.levlist[spos2] : kInf;
-            } else if (ln == 20) {
-                st.phs[5] = l2 < g.K ? g.bins[l2] : 0;
-            } else if (ln == 21) {
-                st.phs[6] = l2 < g.K ? g.bins[l2 + 1] : 0;
-            } else if (ln == 22) {
-                st.phs[7] = g.ctl->icont[nxt];
-            } else if (ln == 23) {
-                st.phs[8] = g.ctl->ilow_c[nxt];
-            } else if (ln == 24) {
-                st.phs[9] = g.ctl->iminup_c[nxt];
-            }
+            const Ctl *c = g.ctl;
+            const int j = ln - 16;
+            const int32_t *p = j == 0   ? &c->imcnt[nxt]
+                               : j == 1 ? &c->itl[nxt]
+                               : j == 2 ? &c->icl[nxt]
+                               : j == 3 ? g.levlist + min(spos2, nlev - 1)
+                               : j == 4 ? g.bins + min(l2, g.K)
+                               : j == 5 ? g.bins + min(l2 + 1, g.K)
+                               : j == 6 ? &c->icont[nxt]
+                               : j == 7 ? &c->ilow_c[nxt]
+                                        : &c->iminup_c[nxt];
+            const int cr = T.nwarps() - 1 - (ln * T.nblocks() + T.bid());  // warp ln's srank
+            const bool item = ln < (int)(blockDim.x >> 5) && cr < g.clcap, word = j >= 0 && j < 9;
+            int4 it = make_int4(0, 0, 0, 0);
+            int32_t v = 0;
+            if (item) it = cl_next[cr];
+            if (word) v = ld_volatile(p);
+            if (ln < 16) st.ph4[ln] = it;
+            if (word) st.phs[1 + j] = j == 3 && spos2 >= nlev ? kInf : v;
         },
-        st.phs);
+        st.phs, [&] {  // the lists and totals start empty in the next phase
+            st.tl.hdr[0] = 0;
+            st.tl.hdr[1] = st.tl.cap;
+            st.cl.hdr[0] = 0;
+            st.cl.hdr[1] = st.cl.cap;
+            *st.movers = 0;
+            st.ff[0] = 0;
+            st.ff[1] = st.ff[2] = kInf;
+            st.ff64[0] = st.ff64[1] = 0;
+        });
     if (!passed) return false;
     const InsState before = s;
     ins_advance(g, sh_upmax, s, has_init, st.phs[4], nlev, st.phs[1], st.phs[7], kInf - st.phs[9],
@@ -2774,36 +2802,52 @@ __device__ __forceinline__ void del_apply_chunks(Team &T, const GraphCtx &g, con
     }
 }
 
+// Up to G 16-byte groups of the lanes' thread-mode movers (item it, ng groups), from group
+// j0; x and y gather the mover's own up- and up*-degree.
+template <int G>
+__device__ __forceinline__ void del_scan_slots(const GraphCtx &g, const RoundStage &st, const int4 &it, int ng, int j0,
+                                               int32_t l, int32_t sid, int &x, int &y, ScanCount &a) {
+    const int4 *pool4 = reinterpret_cast<const int4 *>(g.slots);
+    int32_t ws[4 * G], pv[G];
+    int cu[G], cs[G];
+#pragma unroll
+    for (int j = 0; j < G; ++j) {
+        const int4 s4 = j0 + j < ng ? pool4[it.z + j0 + j] : empty4();
+        ws[4 * j] = s4.x; ws[4 * j + 1] = s4.y; ws[4 * j + 2] = s4.z; ws[4 * j + 3] = s4.w;
+        pv[j] = it.w;
+        cu[j] = cs[j] = 0;
+    }
+    a.scanned += 4 * max(0, min(G, ng - j0));
+    del_effects(g, st, ws, l, pv, sid, cu, cs, a);
+#pragma unroll
+    for (int j = 0; j < G; ++j) {
+        x += cu[j];
+        y += cs[j];
+    }
+}
+
 // Effects of the round's movers (scan items tl and cl) on their neighbours.
 template <class Team>
 __device__ __forceinline__ void del_apply(Team &T, const GraphCtx &g, const RoundStage &st, const DelState &s,
                                           const int4 *tl, const int4 *cl, int32_t sid, ScanCount &a) {
     const int lane = lane_id();
-    const int4 *pool4 = reinterpret_cast<const int4 *>(g.slots);
     for (int i0 = T.srank() * 32; i0 < s.tlc; i0 += T.nwarps() * 32) {
         const int i = i0 + lane;
         const int4 it = i < s.tlc ? tl[i] : make_int4(0, 0, 0, 0);
         const int ng = (i < s.tlc && item_ok(g, it, it.y)) ? (1 << it.y) >> 2 : 0;
         const int maxg = (int)__reduce_max_sync(kFull, (unsigned)ng);
-        const int32_t pv[4] = {it.w, it.w, it.w, it.w};
-        int cu[4] = {0, 0, 0, 0}, cs[4] = {0, 0, 0, 0};
-        for (int j0 = 0; j0 < maxg; j0 += 4) {
-            int32_t ws[16];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int4 s4 = j0 + j < ng ? pool4[it.z + j0 + j] : empty4();
-                ws[4 * j] = s4.x; ws[4 * j + 1] = s4.y; ws[4 * j + 2] = s4.z; ws[4 * j + 3] = s4.w;
-            }
-            a.scanned += 4 * max(0, min(4, ng - j0));
-            del_effects(g, st, ws, s.l, pv, sid, cu, cs, a);
+        int x = 0, y = 0;
+        if (maxg <= 2) {
+            del_scan_slots<2>(g, st, it, ng, 0, s.l, sid, x, y, a);
+        } else {
+            for (int j0 = 0; j0 < maxg; j0 += 4) del_scan_slots<4>(g, st, it, ng, j0, s.l, sid, x, y, a);
         }
         if (i < s.tlc) {
-            const int x = cu[0] + cu[1] + cu[2] + cu[3], y = cs[0] + cs[1] + cs[2] + cs[3];
             if (x) atomicAdd(&g.up[it.x], x);
             if (y) atomicAdd(&g.upstar[it.x], y);
         }
     }
-    if (!Team::kGrid && s.clc <= T.nwarps()) del_apply_chunks<1>(T, g, st, cl, s.clc, s.l, sid, a);
+    if (s.clc <= T.nwarps()) del_apply_chunks<1>(T, g, st, cl, s.clc, s.l, sid, a);
     else del_apply_chunks<4>(T, g, st, cl, s.clc, s.l, sid, a);
 }
 
