@@ -64,8 +64,8 @@ __global__ void __launch_bounds__(kPreThreads) k_pre_canon_filter(const __grid_c
     pre_canon_filter(T, g, BatchIn{g.edges, g.B, g.op, g.stamp_base, g.hcap}, sh_res);
 }
 
-// After an insertion batch was rejected for an id outside [0, n): the incoming
-// counts of the touched vertices back to zero (they are per batch).
+// After a batch was rejected for an id outside [0, n): the counts of the touched
+// vertices' edges back to zero (they are per batch).
 __global__ void k_undo_inc(const int32_t *__restrict__ touched, int64_t count, int32_t *inc) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
         inc[touched[i]] = 0;
@@ -603,10 +603,10 @@ static void launch_pre(plds *h, GraphCtx &g) {
     g.pre_done = 1;
 }
 
-// An insertion batch rejected for an id outside [0, n) by the one-pass step
-// kernel: its valid keys' incoming counts are cleared, leaving the graph as before.
+// A batch rejected for an id outside [0, n) by the one-pass step kernel: its valid
+// keys' counts are cleared, leaving the graph as before.
 static void undo_incoming(plds *h, const Ctl &c, const GraphCtx &g) {
-    if (g.op != kOpInsert || c.ttotal == 0) return;
+    if (c.ttotal == 0) return;
     const int64_t cnt = (int64_t)c.ttotal;
     const int blocks = (int)std::min<int64_t>((cnt + 255) / 256, (int64_t)h->num_sms * 8);
     k_undo_inc<<<blocks, 256, 0, h->stream>>>(g.touched, cnt, g.inc);

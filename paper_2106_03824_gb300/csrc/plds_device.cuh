@@ -403,8 +403,9 @@ inline __device__ int block_exclusive(int x, int *sh32, int *total) {
     return r;
 }
 
-// Steps A2+A3 (insert): put both directions into the tables and update deg, up
-// (other endpoint on a level >= own) and up* (other endpoint on a level >= own-1).
+// Steps A2+A3 (insert): put both directions into the tables and update up (other
+// endpoint on a level >= own) and up* (other endpoint on a level >= own-1).  The degrees
+// take a touched vertex's whole number of new edges (inc) when the rounds start.
 template <class Team>
 __device__ __forceinline__ void step_apply_insert(Team &T, const GraphCtx &g) {
     const int64_t V = (int64_t)g.ctl->vcount;
@@ -417,8 +418,6 @@ __device__ __forceinline__ void step_apply_insert(Team &T, const GraphCtx &g) {
         if (ru < 0 || rv < 0) report(g, kErrInternal, 1, ru < 0 ? u : v, g.cap[ru < 0 ? u : v], g.deg[ru < 0 ? u : v]);
         if (ru == 1) atomicSub(&g.tomb[u], 1);
         if (rv == 1) atomicSub(&g.tomb[v], 1);
-        atomicAdd(&g.deg[u], 1);
-        atomicAdd(&g.deg[v], 1);
         if (lv >= lu) atomicAdd(&g.up[u], 1);
         if (lv >= lu - 1) atomicAdd(&g.upstar[u], 1);
         if (lu >= lv) atomicAdd(&g.up[v], 1);
@@ -431,7 +430,11 @@ __device__ __forceinline__ void del_reset(Ctl *c) {
     c->nextmin[0] = c->nextmin[1] = c->qmin[0] = c->qmin[1] = kInf;
 }
 
-// Steps A2+A3 (delete): tombstone both directions, decrement the counters.
+// Steps A2+A3 (delete): tombstone both directions, decrement up and up*; the shrink plan
+// takes a touched vertex's number of deleted edges (inc) from its degree and adds it to
+// its tombstones.  (One counter atomic per endpoint and edge in the filter instead of
+// three here and in the filter: the atomics of 4 million edges at random vertices of a
+// 4.8 M-vertex graph were most of this step's 1.04 ms.)
 template <class Team>
 __device__ __forceinline__ void step_apply_delete(Team &T, const GraphCtx &g) {
     const int64_t V = (int64_t)g.ctl->vcount;
@@ -442,10 +445,6 @@ __device__ __forceinline__ void step_apply_delete(Team &T, const GraphCtx &g) {
         bool eu = table_erase(g.slots, g.off[u], g.cap[u], v);
         bool ev = table_erase(g.slots, g.off[v], g.cap[v], u);
         if (!eu || !ev) report(g, kErrInternal, 2);
-        atomicAdd(&g.tomb[u], 1);
-        atomicAdd(&g.tomb[v], 1);
-        atomicSub(&g.deg[u], 1);
-        atomicSub(&g.deg[v], 1);
         if (lv >= lu) atomicSub(&g.up[u], 1);
         if (lv >= lu - 1) atomicSub(&g.upstar[u], 1);
         if (lu >= lv) atomicSub(&g.up[v], 1);
@@ -565,12 +564,11 @@ __device__ __forceinline__ void pre_canon(Team &T, const GraphCtx &g, const Batc
 }
 
 // Step A1, second half: keep insertions of absent / deletions of present edges;
-// collect the touched endpoints (deduplicated by stamp) and, for insertions, the
-// number of incoming edges per endpoint.
+// collect the touched endpoints and each one's number of valid edges (inc; the first
+// edge of an endpoint lists it).
 template <class Team>
 __device__ __forceinline__ void pre_filter(Team &T, const GraphCtx &g, const BatchIn &in, unsigned long long *sh) {
     const int64_t U = (int64_t)g.ctl->ucount, stride = (int64_t)T.nblocks() * blockDim.x;
-    const int32_t stouch = in.stamp_base;
     unsigned long long filtered = 0;
     for (int64_t b0 = (int64_t)T.bid() * blockDim.x; b0 < U; b0 += stride) {
         const int64_t i = b0 + threadIdx.x;
@@ -585,12 +583,8 @@ __device__ __forceinline__ void pre_filter(Team &T, const GraphCtx &g, const Bat
             keep = (in.op == kOpInsert) ? !present : present;
             if (!keep) filtered++;
         }
-        const bool tu = keep && atomicExch(&g.stamp[u], stouch) != stouch;
-        const bool tv = keep && atomicExch(&g.stamp[v], stouch) != stouch;
-        if (keep && in.op == kOpInsert) {
-            atomicAdd(&g.inc[u], 1);
-            atomicAdd(&g.inc[v], 1);
-        }
+        const bool tu = keep && atomicAdd(&g.inc[u], 1) == 0;
+        const bool tv = keep && atomicAdd(&g.inc[v], 1) == 0;
         const unsigned long long pos = block_reserve<unsigned long long>(&g.ctl->vcount, keep ? 1ull : 0ull, sh);
         if (keep) g.vkeys[pos] = key;
         const unsigned long long pt =
@@ -610,7 +604,6 @@ __device__ __forceinline__ void pre_filter(Team &T, const GraphCtx &g, const Bat
 template <class Team>
 __device__ __forceinline__ void pre_canon_filter(Team &T, const GraphCtx &g, const BatchIn &in, unsigned long long *sh) {
     const int2 *e = reinterpret_cast<const int2 *>(in.edges);
-    const int32_t stouch = in.stamp_base;
     unsigned long long loops = 0, filtered = 0;
     const int64_t mask = in.hcap - 1, stride = (int64_t)T.nblocks() * blockDim.x;
     for (int64_t b0 = (int64_t)T.bid() * blockDim.x; b0 < in.B; b0 += stride) {
@@ -644,12 +637,8 @@ __device__ __forceinline__ void pre_canon_filter(Team &T, const GraphCtx &g, con
             if (!keep) filtered++;
         }
         block_reserve<unsigned long long>(&g.ctl->ucount, fresh ? 1ull : 0ull, sh);
-        const bool tu = keep && atomicExch(&g.stamp[u], stouch) != stouch;
-        const bool tv = keep && atomicExch(&g.stamp[v], stouch) != stouch;
-        if (keep && in.op == kOpInsert) {
-            atomicAdd(&g.inc[u], 1);
-            atomicAdd(&g.inc[v], 1);
-        }
+        const bool tu = keep && atomicAdd(&g.inc[u], 1) == 0;
+        const bool tv = keep && atomicAdd(&g.inc[v], 1) == 0;
         const unsigned long long pos = block_reserve<unsigned long long>(&g.ctl->vcount, keep ? 1ull : 0ull, sh);
         if (keep) g.vkeys[pos] = key;
         const unsigned long long pt =
@@ -795,9 +784,13 @@ __device__ __forceinline__ void pre_shrink_plan(Team &T, const GraphCtx &g, unsi
         bool want = false;
         if (i < tc) {
             x = g.touched[i];
-            d = g.deg[x];
+            const int32_t gone = g.inc[x];
+            d = g.deg[x] - gone;
             c = g.cap[x];
-            const int32_t tb = g.tomb[x];
+            const int32_t tb = g.tomb[x] + gone;
+            g.deg[x] = d;
+            g.tomb[x] = tb;
+            g.inc[x] = 0;
             if (c > 4 && ((int64_t)d * 8 < c || (int64_t)tb * 4 > c)) {
                 nc = min(next_pow2(2 * (int64_t)d), c);  // in place: never larger than the region
                 want = nc < c || tb > 0;
@@ -1252,8 +1245,8 @@ __device__ __forceinline__ void enqueue_ins(const GraphCtx &g, const RoundStage 
 // ---------------------------------------------------------------------------
 
 // Sort the touched vertices that violate Invariant 1 by level (counting sort) into
-// S; levlist gets their distinct levels in increasing order.  Also resets the
-// per-batch inc counters.  Only violators are initial candidates: while a vertex
+// S; levlist gets their distinct levels in increasing order.  Also moves the
+// per-batch inc counters into the degrees.  Only violators are initial candidates: while a vertex
 // stays on its level its up-degree only grows, so one that violates now is tested
 // when its level is reached, and one that does not is marked by the arrival that
 // takes it past the cutoff.  (Listing every touched vertex made nearly every level
@@ -1269,6 +1262,7 @@ __device__ __forceinline__ bool ins_sort_candidates(Team &T, const GraphCtx &g, 
         int32_t x = 0, lx = -1;
         if (i < tc) {
             x = g.touched[i];
+            g.deg[x] += g.inc[x];
             g.inc[x] = 0;
             const int32_t lv = g.level[x];
             viol = g.up[x] > sh_upmax[lv / g.Lg];
@@ -3494,6 +3488,7 @@ __device__ __forceinline__ bool ins_rounds_jump(Team &T, const GraphCtx &g, cons
         int32_t x = 0, lx = 0;
         if (i < tc) {
             x = g.touched[i];
+            g.deg[x] += g.inc[x];
             g.inc[x] = 0;
             lx = g.level[x];
             v_ = g.up[x] > sh_upmax[lx / g.Lg];

@@ -73,3 +73,24 @@ def test_set_of_uneven_graphs(P, ns):  # noqa: F811
             assert o.insert(ins) == 0 and o.delete(dele) == 0
             assert_same(g, o, f"round {r}, n={g.n}")
     S.close()
+
+
+@pytest.mark.parametrize("op", ["insert", "delete"])
+@pytest.mark.parametrize("size", [100, 20_000])
+def test_rejected_batch_leaves_no_trace(P, op, size):  # noqa: F811
+    """A batch with an id out of range (run in one launch or as step kernels) is rejected
+    whole: the per-vertex counts of its valid edges do not reach the next batch."""
+    n, e = GRAPHS["power"]()
+    g, o = P.PLDS(n), O.OraclePLDS(n)
+    first = e[:25_000]
+    g.insert(first)
+    assert o.insert(first) == 0
+    bad = np.concatenate([(e[25_000:] if op == "insert" else first)[:size], [[0, n]]]).astype(np.int32)
+    assert getattr(g, op)(bad, check=False) == -1
+    assert_same(g, o, "after the rejected batch")
+    for what, part in ((op, bad[:-1]), ("insert", e[:30_000]), ("delete", e[10_000:12_000])):
+        getattr(g, what)(part)
+        assert getattr(o, what)(part) == 0
+        assert_same(g, o, what)
+        assert_stats(g, o, what)
+    g.close()
