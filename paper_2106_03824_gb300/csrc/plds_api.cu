@@ -1161,8 +1161,8 @@ namespace {
 struct StaticCtl {
     unsigned long long bar_arrivals;  // grid barrier (same layout as Ctl's first word)
     int32_t err;
-    int32_t acnt[2];    // alive lists
-    int32_t icnt;       // peeled in this iteration
+    unsigned long long lists[3];  // per iteration mod 3: survivors << 32 | peeled
+    int32_t nbig[3], nhuge[3];  // peeled with large tables
     int32_t minb[3];    // lowest bucket among survivors (per iteration mod 3)
     unsigned long long outer, inner, visits;
 };
@@ -1190,82 +1190,114 @@ __device__ __forceinline__ int32_t sk_bucket(const double *thr, int32_t nb, int3
     return lo;
 }
 
+// A peeled vertex's table is scanned by a warp, above kStaticBig slots by a block and above
+// kStaticHuge by the whole grid (a warp would take a hub's 131,072 slots in 1,024 steps one
+// after another; the grid takes its tables one after another, so only a few may be its own).
+constexpr int32_t kStaticBig = 1024, kStaticHuge = 65536;
+
 __global__ void __launch_bounds__(512) k_static_core(const StaticArgs a) {
     GridTeam T{reinterpret_cast<Ctl *>(a.sc), a.wait_limit_ns, 32};
     StaticCtl *sc = a.sc;
     const int lane = threadIdx.x & 31;
     unsigned long long visits = 0;
-    // init: C = deg, bucket of C, alive list; isolated vertices get 0
-    for (int64_t v = T.tid(); v < a.n; v += T.nthreads()) {
-        const int32_t d = a.deg[v];
-        a.C[v] = d;
-        a.r[v] = 0;
-        a.est[v] = 0.0;
-        int32_t b = -1;
-        if (d > 0) {
-            b = sk_bucket(a.thr, a.nb, d);
-            a.A0[atomicAdd(&sc->acnt[0], 1)] = (int32_t)v;
-            atomicMin(&sc->minb[0], b);
+    __shared__ unsigned long long sh_res[17];
+    const int64_t stride = (int64_t)T.nblocks() * blockDim.x;
+    // init: C = deg, bucket of C, alive list; isolated vertices get 0.  List room is taken
+    // once per block and minima once per warp (an atomic per vertex on one address took a
+    // fifth of the whole call).
+    int32_t mb = 0x7fffffff;
+    for (int64_t b0 = (int64_t)T.bid() * blockDim.x; b0 < a.n; b0 += stride) {
+        const int64_t v = b0 + threadIdx.x;
+        int32_t d = 0;
+        if (v < a.n) {
+            d = a.deg[v];
+            const int32_t b = d > 0 ? sk_bucket(a.thr, a.nb, d) : -1;
+            a.C[v] = d;
+            a.r[v] = 0;
+            a.est[v] = 0.0;
+            a.bk[v] = b;
+            if (d > 0) mb = min(mb, b);
         }
-        a.bk[v] = b;
+        const unsigned long long at = block_reserve<unsigned long long>(&sc->lists[0], d > 0 ? 1ull << 32 : 0ull, sh_res);
+        if (d > 0) a.A0[at >> 32] = (int32_t)v;
     }
+    mb = (int32_t)__reduce_min_sync(kFull, (unsigned)mb);
+    if (lane == 0 && mb != 0x7fffffff) atomicMin(&sc->minb[0], mb);
     if (!T.sync()) return;
     int32_t t = ld_volatile(&sc->minb[0]), bkt = t, j = 0;
-    for (int it = 1;; ++it) {
-        if (ld_volatile(&sc->acnt[(it - 1) & 1]) == 0) break;
+    int32_t ac = (int32_t)(*(volatile unsigned long long *)&sc->lists[0] >> 32);
+    for (int it = 1; ac > 0; ++it) {
         const int cur = (it - 1) & 1, nxt = it & 1, w = it % 3;
-        const int32_t ac = ld_volatile(&sc->acnt[cur]);
         const int32_t *A = cur ? a.A1 : a.A0;
         int32_t *An = nxt ? a.A1 : a.A0;
         if (T.leader()) {
             sc->minb[(it + 1) % 3] = 0x7fffffff;  // written in iteration it + 1, last read two barriers ago
+            sc->lists[(it + 1) % 3] = 0;          // likewise
+            sc->nbig[(it + 1) % 3] = sc->nhuge[(it + 1) % 3] = 0;
             sc->inner += 1;
             if (j == 0) sc->outer += 1;
         }
         // select: peel bucket bkt, keep the rest
-        for (int64_t i0 = (int64_t)T.wid() * 32; i0 < ac; i0 += (int64_t)T.nwarps() * 32) {
-            const int64_t i = i0 + lane;
+        for (int64_t b0 = (int64_t)T.bid() * blockDim.x; b0 < ac; b0 += stride) {
+            const int64_t i = b0 + threadIdx.x;
             int32_t v = 0, b = -1;
             if (i < ac) {
                 v = A[i];
                 b = a.bk[v];
             }
             const bool peel = i < ac && b == bkt, keep = i < ac && b != bkt;
+            bool small = peel;
             if (peel) {
                 a.bk[v] = -1;
                 a.est[v] = a.thr[bkt];
+                const int32_t c = a.cap[v];
+                if (c > kStaticBig) {  // large tables: listed from the back, of I or of the survivors' list
+                    small = false;
+                    if (c > kStaticHuge) An[a.n - 1 - atomicAdd(&sc->nhuge[w], 1)] = v;
+                    else a.I[a.n - 1 - atomicAdd(&sc->nbig[w], 1)] = v;
+                }
             }
-            const int pi = warp_append(&sc->icnt, peel);
-            if (peel) a.I[pi] = v;
-            const int pk = warp_append(&sc->acnt[nxt], keep);
-            if (keep) An[pk] = v;
+            const unsigned long long at =
+                block_reserve<unsigned long long>(&sc->lists[w], (keep ? 1ull << 32 : 0ull) | (small ? 1ull : 0ull), sh_res);
+            if (small) a.I[at & 0xffffffffull] = v;
+            if (keep) An[at >> 32] = v;
         }
         if (!T.sync()) return;
         // count: surviving neighbours of the peeled vertices
-        const int32_t ic = ld_volatile(&sc->icnt);
-        if (T.leader()) sc->acnt[cur] = 0;  // read by every thread before the barrier
-        for (int64_t i = T.wid(); i < ic; i += T.nwarps()) {
+        const unsigned long long both = *(volatile unsigned long long *)&sc->lists[w];
+        const int32_t ic = (int32_t)(both & 0xffffffffull), sn = (int32_t)(both >> 32);
+        auto count4 = [&](const int4 &q) {
+            const int32_t w4[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int32_t x = w4[k];
+                if (x >= 0 && x < a.n) {
+                    ++visits;
+                    if (a.bk[x] >= 0) atomicAdd(&a.r[x], 1);
+                }
+            }
+        };
+        for (int64_t i = T.srank(); i < ic; i += T.nwarps()) {
             const int32_t u = a.I[i];
             const int4 *tb = reinterpret_cast<const int4 *>(a.slots + a.off[u]);
             const int32_t ng = a.cap[u] >> 2;
-            for (int32_t g0 = 0; g0 < ng; g0 += 32) {
-                const int32_t gi = g0 + lane;
-                const int4 q = gi < ng ? tb[gi] : make_int4(-1, -1, -1, -1);
-                const int32_t w4[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int32_t x = w4[k];
-                    if (x >= 0 && x < a.n) {
-                        ++visits;
-                        if (a.bk[x] >= 0) atomicAdd(&a.r[x], 1);
-                    }
-                }
-            }
+            for (int32_t gi = lane; gi < ng; gi += 32) count4(tb[gi]);
+        }
+        const int32_t nbig = ld_volatile(&sc->nbig[w]), nhuge = ld_volatile(&sc->nhuge[w]);
+        for (int32_t i = T.bid(); i < nbig; i += T.nblocks()) {
+            const int32_t u = a.I[a.n - 1 - i];
+            const int4 *tb = reinterpret_cast<const int4 *>(a.slots + a.off[u]);
+            const int32_t ng = a.cap[u] >> 2;
+            for (int32_t gi = threadIdx.x; gi < ng; gi += blockDim.x) count4(tb[gi]);
+        }
+        for (int32_t i = 0; i < nhuge; ++i) {
+            const int32_t u = An[a.n - 1 - i];
+            const int4 *tb = reinterpret_cast<const int4 *>(a.slots + a.off[u]);
+            const int32_t ng = a.cap[u] >> 2;
+            for (int32_t gi = T.tid(); gi < ng; gi += T.nthreads()) count4(tb[gi]);
         }
         if (!T.sync()) return;
         // update: the survivors that lost neighbours; the lowest bucket of all survivors
-        const int32_t sn = ld_volatile(&sc->acnt[nxt]);
-        if (T.leader()) sc->icnt = 0;
         int32_t mu = 0x7fffffff;
         for (int64_t i = T.tid(); i < sn; i += T.nthreads()) {
             const int32_t x = An[i];
@@ -1284,7 +1316,8 @@ __global__ void __launch_bounds__(512) k_static_core(const StaticArgs a) {
         if (lane == 0 && mu != 0x7fffffff) atomicMin(&sc->minb[w], mu);
         if (!T.sync()) return;
         // next: another bucket at the same threshold t while it is within (2+eps) thr[t]
-        if (ld_volatile(&sc->acnt[nxt]) == 0) break;
+        if (sn == 0) break;
+        ac = sn;
         const int32_t next = ld_volatile(&sc->minb[w]);
         if (next < 0 || next >= a.nb) {
             if (T.leader()) {

@@ -94,3 +94,24 @@ def test_rejected_batch_leaves_no_trace(P, op, size):  # noqa: F811
         assert_same(g, o, what)
         assert_stats(g, o, what)
     g.close()
+
+
+@pytest.mark.parametrize("degrees", [(500, 513, 1_100), (3_000, 33_000), (40_000, 40_000, 700)])
+def test_static_core_of_hubs(P, degrees):  # noqa: F811
+    """Static k-core with peeled tables scanned by a warp, a block (above 1,024 slots) and
+    the whole grid (above 65,536): estimates and iteration counts equal the oracle's."""
+    n = 45_000
+    rng = np.random.default_rng(3)
+    parts = [W.erdos_renyi(2_000, 9_000, seed=1)]
+    for h, d in enumerate(degrees):
+        leaves = rng.permutation(np.arange(len(degrees), n))[:d]
+        parts.append(np.stack([np.full(d, h), leaves], 1))
+    e = np.unique(np.sort(np.concatenate(parts).astype(np.int32), axis=1), axis=0)
+    g, o = P.PLDS(n), O.OraclePLDS(n)
+    g.insert(e)
+    assert o.insert(e) == 0
+    for eps in (0.5, 1.0):
+        ge, gs = g.static_coreness(eps)
+        oe, os_ = o.static_coreness(eps)
+        assert np.array_equal(ge, oe) and gs == os_
+    g.close()
