@@ -44,8 +44,9 @@ static int set_status(int s) {
 template <int kWhat>
 __global__ void __launch_bounds__(512) k_batch_grid(const __grid_constant__ GraphCtx g) {
     extern __shared__ int32_t sh[];
-    GridTeam T{g.ctl, g.wait_limit_ns, g.barrier_sleep_ns};
-    run_batch<GridTeam, true, kWhat>(T, g, BatchIn{g.edges, g.B, g.op, g.stamp_base, g.hcap}, sh, 0);
+    using Team = GridTeamOf<kWhat == kJumpRounds>;
+    Team T{g.ctl, g.wait_limit_ns, g.barrier_sleep_ns};
+    run_batch<Team, true, kWhat>(T, g, BatchIn{g.edges, g.B, g.op, g.stamp_base, g.hcap}, sh, 0);
 }
 
 // The steps before the level rounds (preprocessing, table growth and shrinking,
@@ -391,7 +392,7 @@ static int block_threads(const plds *h) { return h->tune.block_threads > 0 ? h->
 // block-wide desire-level histogram, one histogram per warp, staging area.
 static size_t smem_bytes(int threads, int stage_shift = 0) {
     return sizeof(int32_t) *
-           (size_t)(2 * kMaxGroups + 64 + kWarpHist + 32 + (threads / 32) * kWarpHist + stage_ints(stage_shift));
+           (size_t)(2 * kMaxGroups + 64 + kWarpHist + 32 + (threads / 32) * kWarpScratch + stage_ints(stage_shift));
 }
 
 // Device memory that pool growth and serving admission leave free for everything else.
@@ -603,8 +604,9 @@ static void launch_pre(plds *h, GraphCtx &g) {
     g.pre_done = 1;
 }
 
-// A batch rejected for an id outside [0, n) by the one-pass step kernel: its valid
-// keys' counts are cleared, leaving the graph as before.
+// A batch rejected for an id outside [0, n) by the one-pass step kernel, or stopped by a
+// full pool (a block that sees the error word early leaves without its share of the
+// device's own undo): its valid keys' counts are cleared, leaving the graph as before.
 static void undo_incoming(plds *h, const Ctl &c, const GraphCtx &g) {
     if (c.ttotal == 0) return;
     const int64_t cnt = (int64_t)c.ttotal;
@@ -714,6 +716,7 @@ static int run_op(plds *h, const int32_t *edges, int64_t B, int32_t op) {
             undo_incoming(h, c, g);
             return PLDS_EINVAL;
         }
+        if (c.err == kErrNeedPool) undo_incoming(h, c, g);
         if (c.err == kErrNeedPool && attempt < 3) {
             rc = grow_pool(h, (int64_t)c.grow_total);
             if (rc) return rc;
@@ -1196,7 +1199,7 @@ __device__ __forceinline__ int32_t sk_bucket(const double *thr, int32_t nb, int3
 constexpr int32_t kStaticBig = 1024, kStaticHuge = 65536;
 
 __global__ void __launch_bounds__(512) k_static_core(const StaticArgs a) {
-    GridTeam T{reinterpret_cast<Ctl *>(a.sc), a.wait_limit_ns, 32};
+    GridTeamOf<true> T{reinterpret_cast<Ctl *>(a.sc), a.wait_limit_ns, 32};
     StaticCtl *sc = a.sc;
     const int lane = threadIdx.x & 31;
     unsigned long long visits = 0;
@@ -1638,7 +1641,10 @@ extern "C" int plds_batch_static(plds_t *h, const int32_t *edges, int64_t B, int
     }
     // the adjacency pool is full: growing it would allocate, so report and leave
     // the graph unchanged (a regular plds_batch_insert call can grow it)
-    if (c.err == kErrNeedPool) return set_status(PLDS_ENOMEM);
+    if (c.err == kErrNeedPool) {
+        undo_incoming(h, c, g);
+        return set_status(PLDS_ENOMEM);
+    }
     if (c.err) {
         h->poisoned = true;
         return set_status(PLDS_EINTERNAL);
@@ -2325,6 +2331,13 @@ static int server_service(plds_server *sv) {
     }
     h->stamp_base = c.stamp_next;
     if (c.reason == kExitNeedPool) {
+        Ctl hc{};
+        if (cudaMemcpy(&hc, h->ctl.p, sizeof(Ctl), cudaMemcpyDeviceToHost) != cudaSuccess) {
+            cudaGetLastError();
+            h->poisoned = true;
+            return PLDS_EDEVICE;
+        }
+        undo_incoming(h, hc, make_ctx(h, kOpInsert, nullptr, 0));
         const int64_t saved = h->pool_limit;
         h->pool_limit = sv->pool_limit;
         int rc = grow_pool(h, (int64_t)c.grow_total);

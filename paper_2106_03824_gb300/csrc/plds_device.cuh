@@ -33,9 +33,8 @@ __device__ __forceinline__ int ld_volatile(const int32_t *p) { return *(volatile
 // Teams
 // ---------------------------------------------------------------------------
 // Wait until the grid barrier has seen target arrivals (compared modulo 2^32), the
-// error word is set or limit_ns is over (then kErrTimeout is recorded).  A call of its
-// own: inlined it cost the rounds kernels registers around their scan loops.
-static __device__ __noinline__ void arrivals_wait(Ctl *ctl, uint32_t target, int64_t limit_ns, int32_t sleep_ns) {
+// error word is set or limit_ns is over (then kErrTimeout is recorded).
+__device__ __forceinline__ void arrivals_spin(Ctl *ctl, uint32_t target, int64_t limit_ns, int32_t sleep_ns) {
     volatile int32_t *errp = &ctl->err;
     uint64_t t0 = 0;
     unsigned spins = 0;
@@ -56,7 +55,16 @@ static __device__ __noinline__ void arrivals_wait(Ctl *ctl, uint32_t target, int
     }
 }
 
-struct GridTeam {
+// The same as a call of its own: inlined it cost the rounds kernels registers around
+// their scan loops.
+static __device__ __noinline__ void arrivals_wait(Ctl *ctl, uint32_t target, int64_t limit_ns, int32_t sleep_ns) {
+    arrivals_spin(ctl, target, limit_ns, sleep_ns);
+}
+
+// kSpinInline: for kernels with registers to spare (the jump variant's rounds, 3 barriers
+// each, were 4 % slower with the call).
+template <bool kSpinInline>
+struct GridTeamOf {
     static constexpr bool kGrid = true;  // barriers cost a round trip to L2: fetch at the barrier
     static constexpr bool kJump = true;  // may run the jump variant
     Ctl *ctl;
@@ -123,8 +131,12 @@ struct GridTeam {
         asm volatile("atom.add.release.gpu.global.u64 %0, [%1], 1;" : "=l"(before) : "l"(&ctl->bar_arrivals) : "memory");
         if (before != ~0ull) wait_for(goal);  // (polling only once the counter's old value is back)
     }
-    __device__ __forceinline__ void wait_for(uint32_t target) { arrivals_wait(ctl, target, limit_ns, sleep_ns); }
+    __device__ __forceinline__ void wait_for(uint32_t target) {
+        if constexpr (kSpinInline) arrivals_spin(ctl, target, limit_ns, sleep_ns);
+        else arrivals_wait(ctl, target, limit_ns, sleep_ns);
+    }
 };
+using GridTeam = GridTeamOf<false>;
 
 // A thread-block cluster (hardware barrier; its blocks are always resident together).
 // The error word is read between two barriers, so that every block of the cluster
@@ -1447,7 +1459,7 @@ __device__ __forceinline__ void enqueue_marked(const GraphCtx &g, const RoundSta
 // scratch, after the 160 ints enqueue_mover uses) and are queued 32 at a time, so
 // their table lookups are issued together.
 constexpr int kMarkCap = 256;
-constexpr int kTotalsAt = 160 + kMarkCap;  // a warp's totals: 6 x 64 bit of its kWarpHist ints
+constexpr int kTotalsAt = kWarpHist;  // a warp's totals, behind its histogram
 
 __device__ __forceinline__ void marks_flush(const GraphCtx &g, const RoundStage &st, int32_t *mbuf, int &mc,
                                             int k1, int32_t *wsm) {
@@ -1528,8 +1540,7 @@ struct InsState {
 };
 
 // The statistics a thread gathers; when one comes near 32 bits, and at the end of the
-// batch, the warp's sums go to the warp's own totals in shared memory (after its
-// scratch and its buffer of marks).
+// batch, the warp's sums go to the warp's own totals in shared memory.
 struct ScanCount {
     unsigned visits = 0, scanned = 0, upv = 0;
     unsigned aff = 0;  // neighbours whose counters a move changed
@@ -3716,7 +3727,7 @@ __device__ __forceinline__ void run_batch(Team &T, const GraphCtx &g, const Batc
     int32_t *sh_block = sh + 2 * kMaxGroups + 64;  // kWarpHist + 32 ints, block-wide desire-levels
     // (the staging area before the warps' histograms: its addresses are constants then)
     int32_t *sh_stage = sh_block + kWarpHist + 32;
-    int32_t *whist = sh_stage + stage_ints(stage_shift) + (threadIdx.x >> 5) * kWarpHist;
+    int32_t *whist = sh_stage + stage_ints(stage_shift) + (threadIdx.x >> 5) * kWarpScratch;
     for (int i = threadIdx.x; i < g.G; i += blockDim.x) {
         sh_upmax[i] = g.upmax[i];
         sh_dnmin[i] = g.dnmin[i];

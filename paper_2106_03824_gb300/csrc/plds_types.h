@@ -16,6 +16,7 @@ constexpr int32_t kInf = 0x7fffffff;
 constexpr int kMaxGroups = 512;        // groups (t+1) supported by the device tables
 constexpr int kWindow = 256;           // desire-level histogram window (levels)
 constexpr int kWarpHist = 512;         // per-warp shared histogram ints (>= kMaxGroups, kWindow)
+constexpr int kWarpScratch = kWarpHist + 16;  // with the warp's six 64-bit totals behind them
 
 // device error bits
 enum : int32_t {

@@ -115,3 +115,22 @@ def test_static_core_of_hubs(P, degrees):  # noqa: F811
         oe, os_ = o.static_coreness(eps)
         assert np.array_equal(ge, oe) and gs == os_
     g.close()
+
+
+@pytest.mark.parametrize("batch", [9_000, 40_000])
+def test_pool_growth_between_batches(P, batch):  # noqa: F811
+    """Batches (one launch, or step kernels) that find the adjacency pool full are stopped,
+    their per-vertex counts undone, and run again in a larger pool: equal to the oracle's."""
+    n = 12_000
+    e = W.shuffled(W.chung_lu(n, 280_000, 2.6, seed=4), 5)
+    o = O.OraclePLDS(n, levels_per_group=1)
+    gs = [P.PLDS(n, levels_per_group=1) for _ in range(6)]
+    for k, part in enumerate(W.batches(e, batch)):
+        assert o.insert(part) == 0
+        for g in gs:
+            g.insert(part)
+            assert np.array_equal(g.levels(), o.levels()), f"batch {k}"
+    assert all(g.stats()["pool_grows"] > 0 for g in gs)
+    for g in gs:
+        assert_same(g, o, "loaded")
+        g.close()
