@@ -564,7 +564,9 @@ static std::atomic<bool> g_attr_batch[8][kAttrDevices];
 
 // Batches of at most this many edges run as one cooperative launch (k_whole_*): their
 // steps are short, and seven launches with their gaps cost more than the grid barriers
-// between steps at one block per SM.
+// between steps at one block per SM.  (Step kernels / one launch: windows of 10 edges 212 /
+// 181 us, of 9,973 edges 289 / 272 us; cycles of 10^5-edge batches 77.4 / 78.4 ms, windows of
+// 5 10^5 edges 841 / 1,103 us.)
 constexpr int64_t kWholeB = 16384;
 
 // The step kernels of one batch attempt, in stream order, then pre_done set so

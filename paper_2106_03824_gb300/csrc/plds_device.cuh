@@ -1895,7 +1895,10 @@ __device__ __forceinline__ void ins_trace(const GraphCtx &g, const InsState &bef
 // The headers of a phase (three sets, phase index mod 3: a set is reset a phase
 // after its last readers passed the barrier) hold the list headers, the counts of the
 // lists' overflow to global memory, the movers, their totals and the error word.
-constexpr int kSoloCl = 96, kSoloTl = 512;  // largest lists of a phase that one block runs alone
+// Largest lists of a phase that one block runs alone.  (Chunk items 32 / 64 / 96 / 160: R-MAT
+// 18 cycle 68.4 / 69.1 / 68.8 / 70.1 ms, R-MAT 20 windows 812 / 816 / 808 / 827 us; none alone:
+// 10k windows 268 against 247 us, R-MAT 20 windows 1,008 against 842 us.)
+constexpr int kSoloCl = 96, kSoloTl = 512;
 
 template <bool kLimit>
 __device__ __forceinline__ bool ins_phases_local(const GraphCtx &g, const int32_t *sh_upmax, int32_t *wsm, RoundStage st,
