@@ -1708,6 +1708,40 @@ struct plds_set {
     bool has_alloc = false;
 };
 
+// How many of a round's graphs (batch sizes x, decreasing) go to the clusters.  A graph is a
+// candidate when one block would still be busy with it after all blocks together could have
+// finished the round.  Many small graphs of one size are all candidates, but a cluster takes
+// eight blocks' room and is not eight times faster, so the candidates go to the clusters only
+// if the round is then estimated to be shorter than by blocks alone.  Times in 0.1 us, from
+// rounds of 1-600 equal graphs, x edges each (insertions + deletions), clusters only / blocks
+// only, us of a round: 100 graphs of x = 40: 245 / 99, of 2,000: 405 / 306, of 8,000: 632 /
+// 1,087; 300 graphs of 40: 648 / 147, of 2,000: 1,070 / 392; one graph of 400: 92 / 86, of
+// 2,000: 121 / 240, of 20,000: 355 / 1,667.  Rounds of 16 / 128 / 512 graphs of 1e3-1e5
+// vertices: candidates 3.3 / 7.1 / 25.6 ms, blocks only 10.7 / 23.6 / 42.8 ms.
+static int32_t set_large_count(const std::vector<int64_t> &x, int blocks, int clusters) {
+    const int32_t m = (int32_t)x.size();
+    int64_t sum = 0;
+    for (int64_t b : x) sum += b;
+    int32_t large = 0;
+    while (large < m && x[large] * blocks > sum) ++large;
+    if (large == 0) return 0;
+    auto by_block = [](int64_t b) { return 0.85 * (double)b + 300.0; };
+    auto by_cluster = [](int64_t b) { return 0.19 * (double)b + 700.0; };
+    double work_b = 0.0, work_c = 0.0, rest = 0.0;
+    for (int32_t i = 0; i < m && x[i] > 0; ++i) {
+        work_b += by_block(x[i]);
+        if (i < large) work_c += by_cluster(x[i]);
+        else rest += by_block(x[i]);
+    }
+    // blocks alone: the largest graph, slower the more of the room is in use, or all the work
+    const double t_b = std::max(by_block(x[0]) * (1.0 + 1.4 * std::min(1.0, (double)m / blocks)), work_b / blocks);
+    // clusters: the largest graph, the number of graphs one cluster takes, or all the work
+    const int32_t waves = (large + clusters - 1) / clusters;
+    const double t_c = std::max({by_cluster(x[0]), waves * by_cluster(x[large - 1]), work_c / clusters,
+                                 (kSetCluster * work_c + rest) / blocks});
+    return t_c < t_b ? large : 0;
+}
+
 // Runs one round for n_items graphs on the private stream (the caller's stream
 // has been synchronised, so everything it enqueued before is visible).
 static int set_launch(plds_set *s, int32_t n_items, bool use_graph) {
@@ -1871,14 +1905,10 @@ extern "C" int plds_set_update(plds_set_t *s, const int32_t *edges, const int64_
     Ctl *dctl = P<Ctl>(s->ctls);
     for (int attempt = 0; attempt < 4 && !todo.empty(); ++attempt) {
         const int32_t m = (int32_t)todo.size();
-        // a graph is large when one block would still be busy with it after all blocks
-        // together could have finished the round
-        int64_t sum = 0;
-        for (int32_t gi : todo) sum += batch_of(gi);
-        int32_t large = 0;
-        while (large < m && batch_of(todo[large]) * s->grid > sum) ++large;
+        std::vector<int64_t> sizes(m);
+        for (int32_t j = 0; j < m; ++j) sizes[j] = batch_of(todo[j]);
         s->h_queue->next[0] = s->h_queue->next[1] = 0;
-        s->h_queue->large = large;
+        s->h_queue->large = set_large_count(sizes, s->grid, s->clusters);
         s->h_queue->count = m;
         for (int32_t j = 0; j < m; ++j) {
             const int32_t gi = todo[j];

@@ -5,6 +5,8 @@ by a block or a cluster of blocks; a batch passes from one to another as its lis
 grow and shrink.  Every quantity is an integer decided by exact arithmetic, so levels,
 counters and work counts must equal the oracle's after every batch.
 """
+import time
+
 import numpy as np
 import pytest
 
@@ -73,6 +75,33 @@ def test_set_of_uneven_graphs(P, ns):  # noqa: F811
             assert o.insert(ins) == 0 and o.delete(dele) == 0
             assert_same(g, o, f"round {r}, n={g.n}")
     S.close()
+
+
+def _round_seconds(P, count):  # noqa: F811
+    """Best wall time of a round of 20 insertions and 20 deletions in each of `count` graphs alike."""
+    n, b = 300, 20
+    es = [W.shuffled(W.chung_lu(n, 6 * n, 2.4, seed=7 + i % 8), i) for i in range(count)]
+    S = P.PLDSSet([n] * count)
+    S.update(*S.pack([(e[b:], e[:0]) for e in es]))
+    turns = [S.pack([(e[:b], e[b:2 * b]) for e in es]), S.pack([(e[b:2 * b], e[:b]) for e in es])]
+    best = float("inf")
+    for _ in range(8):
+        t0 = time.perf_counter()
+        for t in turns:
+            S.update(*t)
+        best = min(best, time.perf_counter() - t0)
+    o = O.OraclePLDS(n)
+    for ins, dele in [(es[-1][b:], es[-1][:0])] + 8 * [(es[-1][:b], es[-1][b:2 * b]), (es[-1][b:2 * b], es[-1][:b])]:
+        assert o.insert(ins) == 0 and o.delete(dele) == 0
+    assert_same(S.graphs[-1], o, f"{count} graphs")
+    S.close()
+    return best
+
+
+def test_small_graphs_alike_are_not_queued_for_clusters(P):  # noqa: F811
+    """300 small graphs of one size fit one block each: a round of them takes no longer than
+    one of 600 (eight queues' waves of clusters took 2.4 times as long; now 0.6 times)."""
+    assert _round_seconds(P, 300) < 1.4 * _round_seconds(P, 600)
 
 
 @pytest.mark.parametrize("op", ["insert", "delete"])
