@@ -8,16 +8,16 @@ namespace pl {
 template <int kWhat>
 __device__ __forceinline__ void whole_batch(const GraphCtx &g) {
     extern __shared__ int32_t sh[];
-    using Team = GridTeamOf<kWhat == kJumpRounds>;
-    Team T{g.ctl, g.wait_limit_ns, g.barrier_sleep_ns};
-    run_batch<Team, false, kWhat>(T, g, BatchIn{g.edges, g.B, g.op, g.stamp_base, g.hcap}, sh, 0);
+    GridTeam T{g.ctl, g.wait_limit_ns, g.barrier_sleep_ns};
+    run_batch<GridTeam, false, kWhat>(T, g, BatchIn{g.edges, g.B, g.op, g.stamp_base, g.hcap}, sh, 0);
 }
 
 __global__ void __launch_bounds__(512) k_whole_insert(const __grid_constant__ GraphCtx g) {
     whole_batch<kInsertRounds>(g);
 }
 
-__global__ void __launch_bounds__(512) k_whole_jump(const __grid_constant__ GraphCtx g) {
+// (The second launch bound as for the rounds kernel.)
+__global__ void __launch_bounds__(512, 1) k_whole_jump(const __grid_constant__ GraphCtx g) {
     whole_batch<kJumpRounds>(g);
 }
 
