@@ -384,9 +384,12 @@ static bool ensure_batch_scratch(plds *h, int64_t B) {
     return true;
 }
 
-// Key-set entries that a batch of B edges uses.
+// Key-set entries that a batch of B edges uses: four to eight per edge, as far as the buffer
+// (two per edge of the largest batch so far) has them.  (Deletions of 250,000 edges after a
+// larger batch: 103 us of steps with two per edge, 91 with four, 89 with eight or the whole
+// buffer, whose clearing takes longer than that saves.)
 static int64_t key_set_size(const plds *h, int64_t B) {
-    return std::min<int64_t>(h->hcap, pow2_at_least(2 * std::max<int64_t>(B, 1024)));
+    return std::min<int64_t>(h->hcap, pow2_at_least(4 * std::max<int64_t>(B, 1024)));
 }
 
 static int block_threads(const plds *h) { return h->tune.block_threads > 0 ? h->tune.block_threads : 512; }

@@ -62,13 +62,13 @@ __device__ void serve_gather(GridTeam &T, const ServeCtl *sc, int ns, const int6
     }
 }
 
-// Key-set entries the current batch needs: a power of two of at least twice its edges
-// (the buffer is sized for max_batch).
+// Key-set entries the current batch uses: a power of two of at least four times its edges,
+// as far as the buffer has them (it is sized for max_batch).
 __device__ __forceinline__ int64_t serve_hcap(const GraphCtx &base, const ServeCtl *sc) {
     const int64_t B = max((long long)1024, (long long)(*(volatile const int32_t *)&sc->nseg > 0
                                                            ? *(volatile const int64_t *)&sc->seg_total
                                                            : *(volatile const int64_t *)&sc->cur.B));
-    return min((long long)base.hcap, 2ll << (64 - __clzll(B - 1)));
+    return min((long long)base.hcap, 4ll << (64 - __clzll(B - 1)));
 }
 
 // Leader: the loop is about to leave.
