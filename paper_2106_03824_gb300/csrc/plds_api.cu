@@ -1203,10 +1203,15 @@ __device__ __forceinline__ int32_t sk_bucket(const double *thr, int32_t nb, int3
 
 // A peeled vertex's table is scanned by a warp, above kStaticBig slots by a block and above
 // kStaticHuge by the whole grid (a warp would take a hub's 131,072 slots in 1,024 steps one
-// after another; the grid takes its tables one after another, so only a few may be its own).
-constexpr int32_t kStaticBig = 1024, kStaticHuge = 65536;
+// after another).  The grid takes its tables one after another: when an iteration peels more
+// than kStaticFew of them, they are scanned by a block each as well.  (R-MAT 19, 8.4 M samples:
+// blocks above 512 / 1,024 / 4,096 slots 1.69 / 1.70 / 1.74 ms; the grid above 512 / 2,048 /
+// 16,384 / 65,536 slots 11.99 / 4.08 / 1.92 / 1.70 ms.  Hubs of 131,072 slots, by the grid / by
+// blocks: 1 hub 0.12 / 0.20 ms, 20: 0.40 / 0.45, 300: 3.79 / 3.42, 1,500: 8.08 / 5.77.)
+constexpr int32_t kStaticBig = 1024, kStaticHuge = 65536, kStaticFew = 32;
 
-__global__ void __launch_bounds__(512) k_static_core(const StaticArgs a) {
+// (The second launch bound as for k_batch_grid: the R-MAT call 1,660 us with it, 1,713 without.)
+__global__ void __launch_bounds__(512, 1) k_static_core(const StaticArgs a) {
     GridTeamOf<true> T{reinterpret_cast<Ctl *>(a.sc), a.wait_limit_ns, 32};
     StaticCtl *sc = a.sc;
     const int lane = threadIdx.x & 31;
@@ -1295,13 +1300,14 @@ __global__ void __launch_bounds__(512) k_static_core(const StaticArgs a) {
             for (int32_t gi = lane; gi < ng; gi += 32) count4(tb[gi]);
         }
         const int32_t nbig = ld_volatile(&sc->nbig[w]), nhuge = ld_volatile(&sc->nhuge[w]);
-        for (int32_t i = T.bid(); i < nbig; i += T.nblocks()) {
-            const int32_t u = a.I[a.n - 1 - i];
+        const int32_t nwide = nhuge > kStaticFew ? 0 : nhuge, nblk = nbig + nhuge - nwide;
+        for (int32_t i = T.bid(); i < nblk; i += T.nblocks()) {
+            const int32_t u = i < nbig ? a.I[a.n - 1 - i] : An[a.n - 1 - (i - nbig)];
             const int4 *tb = reinterpret_cast<const int4 *>(a.slots + a.off[u]);
             const int32_t ng = a.cap[u] >> 2;
             for (int32_t gi = threadIdx.x; gi < ng; gi += blockDim.x) count4(tb[gi]);
         }
-        for (int32_t i = 0; i < nhuge; ++i) {
+        for (int32_t i = 0; i < nwide; ++i) {
             const int32_t u = An[a.n - 1 - i];
             const int4 *tb = reinterpret_cast<const int4 *>(a.slots + a.off[u]);
             const int32_t ng = a.cap[u] >> 2;

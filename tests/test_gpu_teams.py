@@ -146,6 +146,24 @@ def test_static_core_of_hubs(P, degrees):  # noqa: F811
     g.close()
 
 
+@pytest.mark.parametrize("hubs", [8, 32, 33, 170])
+def test_static_core_of_many_huge_tables(P, hubs):  # noqa: F811
+    """Tables above 65,536 slots (a load factor of 1/16: degrees above 4,096): up to 32 peeled
+    at once are scanned by the whole grid, more by a block each."""
+    n = 9_000
+    leaves = np.arange(4_200)
+    e = np.concatenate([np.stack([np.full(leaves.size, h), hubs + (leaves + 37 * h) % (n - hubs)], 1)
+                        for h in range(hubs)]).astype(np.int32)
+    g, o = P.PLDS(n), O.OraclePLDS(n)
+    g.set_tuning(load_num=1, load_den=16)
+    g.insert(e)
+    assert o.insert(e) == 0
+    ge, gs = g.static_coreness(1.0)
+    oe, os_ = o.static_coreness(1.0)
+    assert np.array_equal(ge, oe) and gs == os_
+    g.close()
+
+
 @pytest.mark.parametrize("batch", [9_000, 40_000])
 def test_pool_growth_between_batches(P, batch):  # noqa: F811
     """Batches (one launch, or step kernels) that find the adjacency pool full are stopped,
