@@ -2394,6 +2394,22 @@ static int server_service(plds_server *sv) {
     return PLDS_OK;
 }
 
+// After a slot was marked ready: a loop that is leaving may not have seen it.  Wait until it
+// has taken the request after all or has stopped (microseconds), then start it again, so that
+// the request is served without another call.
+static int server_wake(plds_server *sv) {
+    std::atomic_thread_fence(std::memory_order_seq_cst);
+    volatile int32_t *reason = &sv->exit->reason;
+    const auto t0 = std::chrono::steady_clock::now();
+    while (sv->running && *reason == kExitLeaving)
+        if (std::chrono::steady_clock::now() - t0 > std::chrono::nanoseconds(sv->h->wait_limit_ns))
+            return PLDS_ETIMEOUT;
+    if (sv->running && *reason != kExitNone) cudaEventSynchronize(sv->done);
+    const int rc = server_service(sv);
+    if (rc) return rc;
+    return sv->running ? PLDS_OK : server_launch(sv);
+}
+
 // Move finished requests out of the ring; frees their slots.
 static void server_collect(plds_server *sv) {
     while (sv->done_seq < sv->next_seq) {
@@ -2602,13 +2618,7 @@ extern "C" int plds_server_submit(plds_server_t *sv, int32_t op, const int32_t *
     *(volatile int32_t *)&r->state = kSlotReady;
     if (ticket) *ticket = sv->next_seq;
     sv->next_seq++;
-    int rc = server_service(sv);
-    if (rc) return set_status(rc);
-    if (!sv->running) {
-        rc = server_launch(sv);
-        if (rc) return set_status(rc);
-    }
-    return set_status(PLDS_OK);
+    return set_status(server_wake(sv));
 }
 
 extern "C" int plds_server_configure(plds_server_t *sv, int64_t merge_max_edges, int64_t pool_limit_bytes) {

@@ -39,7 +39,7 @@ __global__ void k_batch_set_cluster(const SetItem *items, SetQueue *q);
 // Serving form.
 enum : int32_t { kSlotFree = 0, kSlotReady = 1, kSlotDone = 2 };
 enum : int32_t { kReqInsert = 0, kReqDelete = 1, kReqCoreness = 2 };
-enum : int32_t { kExitNone = 0, kExitIdle = 1, kExitNeedPool = 2, kExitError = 3 };
+enum : int32_t { kExitNone = 0, kExitIdle = 1, kExitNeedPool = 2, kExitError = 3, kExitLeaving = 4 };
 constexpr int kMaxSeg = 64;  // requests merged into one batch at most
 
 struct alignas(64) ReqSlot {
@@ -75,7 +75,10 @@ struct ServeCtl {  // device memory
 };
 
 // Why and where the loop stopped, written into pinned host memory as it leaves
-// (reason kExitNone: not written, an error stopped it).
+// (reason kExitNone: not written, an error stopped it).  An idle loop first writes
+// kExitLeaving and looks at its slot once more: either it sees a request marked ready
+// meanwhile, takes the mark back and serves it, or the host, which reads the reason after
+// marking its slot, sees that the loop is leaving.
 struct ServeExit {
     int32_t reason;
     int32_t stamp_next;

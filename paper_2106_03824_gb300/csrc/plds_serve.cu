@@ -94,6 +94,12 @@ __global__ void __launch_bounds__(512) k_serve(const __grid_constant__ GraphCtx 
             int32_t st;
             while ((st = *(volatile int32_t *)&r->state) != kSlotReady && global_ns() - t0 < (uint64_t)a.idle_ns)
                 __nanosleep(256);
+            if (st != kSlotReady) {
+                *(volatile int32_t *)&a.exit->reason = kExitLeaving;
+                __threadfence_system();
+                st = *(volatile int32_t *)&r->state;
+                if (st == kSlotReady) *(volatile int32_t *)&a.exit->reason = kExitNone;
+            }
             if (st == kSlotReady) {
                 __threadfence_system();
                 copy_slot(&sc->cur, r);

@@ -15,6 +15,7 @@ counts and query values; a request with a bad id is rejected alone; and every
 query's estimates, in the mix and with the same requests applied alone, are within
 the paper's bound (2 + 3/lambda)(1 + delta) of the exact coreness both ways.
 """
+import time
 from fractions import Fraction
 
 import numpy as np
@@ -222,3 +223,32 @@ def test_admission_is_gated_by_memory(P):
     o.delete(e[:10])
     assert np.array_equal(g.levels(), o.levels())
     g.close()
+
+
+def test_request_at_the_idle_limit_is_served_without_another_call(P):
+    """An idle loop leaves after 2 ms.  Queries submitted around that moment, with no poll,
+    drain or further submit after them, fill their output buffers all the same."""
+    n = 2_000
+    g = P.PLDS(n)
+    g.insert(W.chung_lu(n, 10_000, 2.3, seed=1))
+    want = g.coreness()
+    sv = P.Server(g, slots=8, max_batch=1_000)
+    out = torch.empty(n, dtype=torch.float64).pin_memory()
+    view, lost, rounds = out.numpy(), [], 600
+    for k in range(rounds):
+        view[:] = -1.0
+        sv.submit(sv.CORENESS, out=out)
+        t0 = time.perf_counter()
+        while (view < 0).any():
+            if time.perf_counter() - t0 > 0.2:
+                lost.append(k)
+                sv.drain()
+                break
+        t0 = time.perf_counter()
+        while time.perf_counter() - t0 < 1e-3 * (1.95 + 0.1 * k / rounds):
+            pass
+    assert np.array_equal(view, want)
+    sv.drain()
+    sv.close()
+    g.close()
+    assert not lost, f"{len(lost)} of {rounds} requests waited for another call"
