@@ -347,6 +347,8 @@ void plds_set_destroy(plds_set_t *s);
  *     cost(t, ctx) returns a cost (seconds) or a negative value to stop the search
  *     with PLDS_EINTERNAL.  *best gets the chosen knobs (the other fields of start
  *     are kept); returns the number of evaluations or a negative code.
+ *     start->thread_max_cap = -1: the cutoff starts unset -- 0, which a handle takes as
+ *     its own choice by phase -- and 0 is a candidate as well.
  *   plds_set_tune: the same knobs for every graph of a set.
  *   plds_set_autotune: the search for a set, on a sample of its workload: each
  *     evaluation builds a scratch set of the same graph sizes, applies rounds
@@ -368,7 +370,9 @@ int plds_tune_search(const plds_tuning *start, plds_tune_cost cost, void *ctx, i
  *     kinds[b] == 0, a deletion if 1 -- and costs the wall time of the batches from
  *     timed_from on (the earlier ones build the sample's state untimed).  h's graph
  *     is not touched; its knobs become the best ones (also written to *best when
- *     non-null).  PLDS_EINVAL on bad arguments; a failing sample batch's code
+ *     non-null).  The first evaluation is the handle as it is; one whose thread cutoff
+ *     was unset keeps its choice by phase unless a fixed cutoff costs at least 2 % less
+ *     (*best then says 8, the cutoff of its deletion rounds).  PLDS_EINVAL on bad arguments; a failing sample batch's code
  *     otherwise.
  */
 int plds_autotune(plds_t *h, const int32_t *edges, const int64_t *offsets, const int32_t *kinds, int32_t nbatches,

@@ -485,6 +485,9 @@ static int grow_pool(plds *h, int64_t extra) {
 // R-MAT 20); insertion phases pick their own (ins_thread_cap).
 constexpr int32_t kThreadCap = 8;
 
+// Default block cutoff (tuning field 0).
+constexpr int32_t kBlockCap = 1024;
+
 static GraphCtx make_ctx(plds *h, int32_t op, const int32_t *edges, int64_t B) {
     GraphCtx g{};
     g.n = h->n;
@@ -497,7 +500,7 @@ static GraphCtx make_ctx(plds *h, int32_t op, const int32_t *edges, int64_t B) {
     g.tcap_auto = h->tune.thread_max_cap <= 0;
     g.load_num = h->tune.load_num > 0 ? h->tune.load_num : 3;
     g.load_den = h->tune.load_den > 0 ? h->tune.load_den : 4;
-    g.block_cap = h->tune.block_cap > 0 ? h->tune.block_cap : 1024;
+    g.block_cap = h->tune.block_cap > 0 ? h->tune.block_cap : kBlockCap;
     g.list_cap = h->tune.list_cap > 0 ? h->tune.list_cap : 256;
     g.jump = h->jump ? 1 : 0;
     g.wait_limit_ns = h->wait_limit_ns;
@@ -2067,7 +2070,9 @@ extern "C" int plds_tune_search(const plds_tuning *start, plds_tune_cost cost, v
                                 plds_tuning *best) {
     if (!start || !cost || !best || max_trials < 1) return set_status(PLDS_EINVAL);
     plds_tuning cur = *start;
-    if (cur.thread_max_cap <= 0) cur.thread_max_cap = 16;
+    const bool by_phase = cur.thread_max_cap < 0;  // a cutoff left unset (0) takes part
+    if (by_phase) cur.thread_max_cap = 0;
+    else if (cur.thread_max_cap == 0) cur.thread_max_cap = 16;
     if (cur.block_cap <= 0) cur.block_cap = 4096;
     if (cur.load_num <= 0 || cur.load_den <= 0) {
         cur.load_num = 3;
@@ -2097,11 +2102,11 @@ extern "C" int plds_tune_search(const plds_tuning *start, plds_tune_cost cost, v
     while (improved && !spent) {
         improved = false;
         for (int knob = 0; knob < 4 && !spent; ++knob) {
-            const int nv = knob >= 2 ? 4 : 5;
+            const int nv = knob >= 2 ? 4 : knob == 0 && by_phase ? 6 : 5;
             for (int v = 0; v < nv; ++v) {
                 plds_tuning t = cur;
                 if (knob == 0) {
-                    t.thread_max_cap = kTuneThread[v];
+                    t.thread_max_cap = v < 5 ? kTuneThread[v] : 0;
                 } else if (knob == 1) {
                     t.block_cap = kTuneBlock[v];
                 } else if (knob == 2) {
@@ -2204,15 +2209,21 @@ extern "C" int plds_autotune(plds_t *h, const int32_t *edges, const int64_t *off
         if (offsets[b] < 0 || offsets[b + 1] < offsets[b] || (kinds[b] != 0 && kinds[b] != 1))
             return set_status(PLDS_EINVAL);
     HandleTuneCtx c{h, edges, offsets, kinds, nbatches, timed_from, PLDS_OK};
-    plds_tuning out{};
-    const int trials = plds_tune_search(&h->tune, handle_trial_cost, &c, max_trials, &out);
+    // the first trial is the handle as it is: unset knobs at its own defaults
+    plds_tuning start = h->tune, out{};
+    if (start.thread_max_cap == 0) start.thread_max_cap = -1;
+    if (start.block_cap == 0) start.block_cap = kBlockCap;
+    const int trials = plds_tune_search(&start, handle_trial_cost, &c, max_trials, &out);
     if (trials < 0) return set_status(c.status != PLDS_OK ? c.status : trials);
     h->tune.thread_max_cap = out.thread_max_cap;
     h->tune.block_cap = out.block_cap;
     h->tune.load_num = out.load_num;
     h->tune.load_den = out.load_den;
     h->tune.list_cap = out.list_cap;
-    if (best) *best = h->tune;
+    if (best) {
+        *best = h->tune;
+        if (best->thread_max_cap == 0) best->thread_max_cap = kThreadCap;
+    }
     return set_status(PLDS_OK);
 }
 

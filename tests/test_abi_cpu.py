@@ -103,6 +103,23 @@ def test_tune_search_budget_and_failure(lib):
     assert best["thread_max_cap"] == 16
 
 
+@pytest.mark.parametrize("fixed_cost, picked", [(1.2, 0), (0.99, 0), (0.9, 8)])
+def test_tune_search_times_an_unset_cutoff(lib, fixed_cost, picked):
+    """From a start with the cutoff left to the handle (-1), that setting (0) is evaluated
+    first and stays unless a fixed cutoff costs at least 2 % less."""
+    seen = []
+
+    def cost(k):
+        seen.append(k["thread_max_cap"])
+        c = {0: 1.0, 8: fixed_cost}.get(k["thread_max_cap"], 1.5)
+        return c * (0.9 if k["block_cap"] == 2048 else 1.0)
+
+    best, n = P.tune_search(cost, start={"thread_max_cap": -1, "block_cap": 1024})
+    assert seen[0] == 0 and n == len(seen)
+    assert set(seen) == {0, 4, 8, 16, 32, 64}
+    assert best == {"thread_max_cap": picked, "block_cap": 2048, "load_num": 3, "load_den": 4, "list_cap": 256}
+
+
 def test_opt_levels_per_group_matches_oracle(lib):
     """The library's exact PLDSOpt group size agrees with the oracle's own bignum."""
     from oracle import oracle as O
