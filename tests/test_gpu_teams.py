@@ -57,6 +57,40 @@ def test_batches_of_uneven_size(P, name, sizes):  # noqa: F811
     g.close()
 
 
+def test_deletions_with_a_narrowed_window(P):  # noqa: F811
+    """Deletion batches of a road-like graph that leave more than 4,096 vertices pending over
+    many levels: the near window is narrowed, the rest is sent to the far list and comes back
+    refill by refill.  By the grid, and by a cluster (a set of one graph)."""
+    side = 600
+    n = side * side
+    e = W.shuffled(W.grid2d(side, 0.1, seed=3), 4)
+    dele = W.shuffled(e, 9)
+    g, S, o = P.PLDS(n), P.PLDSSet([n]), O.OraclePLDS(n)
+    g.set_tuning(trace_rounds=1)
+    g.insert(e)
+    S.update(*S.pack([(e, e[:0])]))
+    assert o.insert(e) == 0
+    assert_same(g, o, "loaded")
+    m = e.shape[0]
+    narrowed = refilled = 0
+    for a, b in ((0, 0.3), (0.3, 0.6), (0.6, 0.8)):
+        part = np.ascontiguousarray(dele[int(a * m): int(b * m)])
+        g.delete(part)
+        S.update(*S.pack([(part[:0], part)]))
+        assert o.delete(part) == 0
+        assert_same(g, o, f"deleted to {b}")
+        assert_stats(g, o, f"deleted to {b}")
+        assert_same(S.graphs[0], o, f"set, deleted to {b}")
+        t = g.trace()[1:]
+        near, movers = t[:, 1].astype(int), t[:, 2].astype(int)
+        left = near[:-1] - movers[:-1]  # near entries that did not move in a round
+        narrowed += int(((near[:-1] > 4096) & (left - near[1:] > near[:-1] // 2)).sum())
+        refilled += int((near[1:] - left > 64).sum())
+    assert narrowed >= 2 and refilled >= 4, (narrowed, refilled)
+    g.close()
+    S.close()
+
+
 @pytest.mark.parametrize("ns", [(9_000,), (1, 2, 9_000, 40, 700), (4_000,) * 3 + (100,) * 60])
 def test_set_of_uneven_graphs(P, ns):  # noqa: F811
     """A round's largest graphs go to clusters, the others to blocks: each equals the oracle."""
