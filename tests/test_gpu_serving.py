@@ -225,6 +225,31 @@ def test_admission_is_gated_by_memory(P):
     g.close()
 
 
+def test_pool_growth_between_served_batches(P):
+    """Served batches that find the adjacency pool full stop the loop: the host clears their
+    per-vertex counts, grows the pool and starts the loop again.  Equal to the oracle's."""
+    n = 12_000
+    parts = list(W.batches(W.shuffled(W.chung_lu(n, 280_000, 2.6, seed=4), 5), 9_000))
+    o = O.OraclePLDS(n, levels_per_group=1)
+    want = []
+    for part in parts:
+        assert o.insert(part) == 0
+        want.append(o.stats())
+    for _ in range(6):
+        g = P.PLDS(n, levels_per_group=1)
+        sv = P.Server(g, slots=4, max_batch=9_000, merge_max_edges=0)
+        for part in parts:
+            sv.submit(sv.INSERT, part)
+        sv.drain()
+        done = sorted(sv.poll(64), key=lambda r: r["ticket"])
+        sv.close()
+        for r, w in zip(done, want, strict=True):
+            assert r["status"] == 0 and all(r[k] == w[k] for k in ("valid", "rounds", "moves")), (r, w)
+        assert g.stats()["pool_grows"] > 0
+        assert np.array_equal(g.levels(), o.levels())
+        g.close()
+
+
 def test_request_at_the_idle_limit_is_served_without_another_call(P):
     """An idle loop leaves after 2 ms.  Queries submitted around that moment, with no poll,
     drain or further submit after them, fill their output buffers all the same."""
