@@ -2982,7 +2982,7 @@ __device__ __forceinline__ bool del_rounds_local(const GraphCtx &g, int32_t stam
                 return true;
             }
             if (kLimit && (s.qc > kSoloFar || leave)) return true;
-            if (++refills > g.K + 4) {  // every window takes at least one level
+            if (++refills > g.K + 4) {  // each window ends above the last one's end, also an empty one
                 if (threadIdx.x == 0) report(g, kErrInternal, 26, s.qc, s.qmin, s.limit);
                 return false;
             }
@@ -3188,6 +3188,9 @@ __device__ __forceinline__ bool del_rounds(Team &T, const GraphCtx &g, const int
             uint64_t t0 = tr ? global_ns() : 0, t1 = t0, t2 = t0;
             if (s.stage == 0 && s.nmin == kInf) {  // the near list is used up: the window moves on
                 if (s.qc == 0) break;
+                // Rounds take a level each.  Windows end above one another until the window is
+                // narrowed; all but the last before that lie within the levels the rounds since
+                // the narrowing have passed: no more windows than levels in all.
                 if (s.r > 2 * g.K + 4) {
                     if (T.leader()) report(g, kErrInternal, 26, s.qc, s.qmin, s.limit);
                     return false;
@@ -3322,8 +3325,6 @@ __device__ __forceinline__ bool del_rounds(Team &T, const GraphCtx &g, const int
 //      violates there.  The flag stays on until the next round's phase A, so every
 //      reader of B tells movers from the rest.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int32_t round_flag(int r) { return (r & 1) ? kFlagOdd : kFlagEven; }
-
 // Smallest x in [lo, hi] (hi - lo < 256) with above + sum_{y=x..hi} h[y-lo] <= upmax
 // of x's group, or -1.  The count falls and the bound rises with x, so the test
 // fails below the answer and passes from it on.  One warp.
@@ -3564,7 +3565,7 @@ __device__ __forceinline__ bool ins_rounds_jump(Team &T, const GraphCtx &g, cons
             if (T.leader()) report(g, kErrInternal, 21, l, r, 0);
             return false;
         }
-        const int32_t flr = round_flag(r), flp = round_flag(r + 1);
+        const int32_t flr = phase_flag(r), flp = phase_flag(r + 1);
         const int mi = r % 3, mprev = (r + 2) % 3;
         const uint64_t t_round = (g.trace && T.leader()) ? global_ns() : 0;
         // the list is rewritten (live entries only) once most of it has been taken
