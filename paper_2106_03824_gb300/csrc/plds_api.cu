@@ -485,7 +485,9 @@ static int grow_pool(plds *h, int64_t extra) {
 // R-MAT 20); insertion phases pick their own (ins_thread_cap).
 constexpr int32_t kThreadCap = 8;
 
-// Default block cutoff (tuning field 0).
+// Default block cutoff (tuning field 0): a block instead of a warp evaluates the desire-level
+// of a vertex with a table above it.
+// (256 / 1,024 / 4,096 slots: R-MAT 20 cycle 59.1 / 57.8 / 59.3 ms, R-MAT 18 68.0 / 67.9 / 68.6.)
 constexpr int32_t kBlockCap = 1024;
 
 static GraphCtx make_ctx(plds *h, int32_t op, const int32_t *edges, int64_t B) {
@@ -1732,7 +1734,7 @@ struct plds_set {
 // only, us of a round: 100 graphs of x = 40: 245 / 99, of 2,000: 405 / 306, of 8,000: 632 /
 // 1,087; 300 graphs of 40: 648 / 147, of 2,000: 1,070 / 392; one graph of 400: 92 / 86, of
 // 2,000: 121 / 240, of 20,000: 355 / 1,667.  Rounds of 16 / 128 / 512 graphs of 1e3-1e5
-// vertices: candidates 3.3 / 7.1 / 25.6 ms, blocks only 10.7 / 23.6 / 42.8 ms.
+// vertices: candidates 3.3 / 7.0 / 25.6 ms, blocks only 10.7 / 23.6 / 42.8 ms.
 static int32_t set_large_count(const std::vector<int64_t> &x, int blocks, int clusters) {
     const int32_t m = (int32_t)x.size();
     int64_t sum = 0;
@@ -2295,7 +2297,9 @@ struct plds_server {
     int64_t next_seq = 0;  // sequence number of the next submitted request
     int64_t done_seq = 0;  // all sequence numbers below have been collected
     // An idle loop holds every SM (a server on another graph, or a kernel that needs
-    // the shared memory, waits for it) and a relaunch takes the host ~20 us: 2 ms.
+    // the shared memory, waits for it) and a relaunch takes the host ~20 us: 2 ms.  (48 requests,
+    // two servers in turn, 35.1 ms with 20 ms and 16.5 ms with 2 ms; a lone server with a request
+    // every 2.5-6 ms pays the relaunch each time, 0.173 ms a deletion instead of 0.151.)
     int64_t idle_ns = 2ll * 1000 * 1000;
     ServeExit *exit = nullptr;  // pinned, mapped
     ServeExit *exit_dev = nullptr;

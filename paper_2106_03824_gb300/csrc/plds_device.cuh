@@ -140,7 +140,9 @@ struct GridTeamOf {
 };
 using GridTeam = GridTeamOf<false>;
 
-// A thread-block cluster (hardware barrier; its blocks are always resident together).
+// A thread-block cluster (hardware barrier; its blocks are always resident together).  The
+// barrier has no time limit: what bounds a wait is that every loop between two barriers has an
+// iteration limit and that a stretch run by one block ends at a quarter of the wait limit.
 // The error word is read between two barriers, so that every block of the cluster
 // decides alike and no block is left waiting.
 struct ClusterTeam {
@@ -1899,7 +1901,8 @@ __device__ __forceinline__ void ins_trace(const GraphCtx &g, const InsState &bef
 // lists' overflow to global memory, the movers, their totals and the error word.
 // Largest lists of a phase that one block runs alone.  (Chunk items 32 / 64 / 96 / 160: R-MAT
 // 18 cycle 68.4 / 69.1 / 68.8 / 70.1 ms, R-MAT 20 windows 812 / 816 / 808 / 827 us; none alone:
-// 10k windows 268 against 247 us, R-MAT 20 windows 1,008 against 842 us.)
+// 10k windows 268 against 247 us, R-MAT 20 windows 1,008 against 842 us.  Thread items 128 / 512
+// / 2,048: cycles of 1,000-edge batches 40.3 / 37.9 / 37.9 ms, R-MAT 18 cycle 68.0 / 67.9 / 78.0.)
 constexpr int kSoloCl = 96, kSoloTl = 512;
 
 template <bool kLimit>
@@ -2739,6 +2742,8 @@ __device__ __forceinline__ void del_window(const GraphCtx &g, DelState &s) {
     s.limit = (int32_t)min((int64_t)s.qmin + s.delta - 1, (int64_t)g.K);
 }
 
+// (Bounds of 128 and 512 entries: road grid 35.7 ms, R-MAT 18 68.2; 512 and 2,048: 37.0, 67.9;
+// 2,048 and 8,192: 40.5, 67.5; steps of two instead of four: 37.9, 68.1.)
 __device__ __forceinline__ void del_window_done(DelState &s) {
     if (s.pc < 512) s.delta = min(4 * s.delta, 1 << 20);
     else if (s.pc > 2048) s.delta = max(1, s.delta >> 2);
@@ -2917,6 +2922,9 @@ __device__ __forceinline__ bool del_initial(Team &T, const GraphCtx &g, RoundSta
 // published before each; a block's three block barriers).  With kLimit the rounds stop, at
 // the stage that s names, when the next stage is above the kSolo bounds or the stretch
 // has taken a quarter of the wait limit; a stage's input lists are then in global memory.
+// (Road grid of 1.4 M vertices / R-MAT 18 cycles, ms: kSoloNear 1,024 37.6 / 66.8, 4,096 37.0 /
+// 67.9, 16,384 41.1 / 68.8; kSoloFar 1,024 36.9 / 68.2, 4,096 37.0 / 67.9, 16,384 37.4 / 68.5;
+// kSoloEval 64 36.9 / 68.3, 256 37.0 / 67.9, 1,024 37.1 / 68.0.)
 constexpr int kSoloNear = 4096, kSoloFar = 4096, kSoloEval = 256;
 
 template <bool kLimit>
@@ -3287,7 +3295,7 @@ __device__ __forceinline__ bool del_rounds(Team &T, const GraphCtx &g, const int
             // one, whose far list is empty: in another a vertex that came back near may still
             // be listed (and its count, which faster blocks' takes change, decides nothing).
             if (s.calm >= 2 && s.pc > kSoloNear && s.limit >= g.K) {
-                s.delta = 16;
+                s.delta = 16;  // (4 / 16 / 64 levels: road grid 37.9 / 37.0 / 37.9 ms)
                 s.limit = s.nmin + s.delta - 1;
             }
             if (tr) del_trace(g, s, pc, nb, t0, t1, t2);

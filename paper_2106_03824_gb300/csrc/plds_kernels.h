@@ -20,8 +20,9 @@ struct SetItem {
 };
 constexpr int kSetThreads = 256;
 constexpr int kSetStageShift = 1;
-// Blocks per large graph.  Rounds of 128 / 512 / 16 graphs with 4: 9.9 / 16.0 / 5.2 ms, with 8:
-// 7.4 / 18.4 / 3.8 ms, with 16: 11.1 / 28.3 / 3.1 ms (one block per graph: 28 / 33 / 13.5 ms).
+// Blocks per large graph.  Rounds of 16 / 64 / 128 / 512 graphs of 1e3-1e5 vertices, level reads
+// included, with 4: 4.4 / 7.7 / 9.2 / 23.6 ms, with 8: 3.3 / 5.4 / 7.0 / 25.6, with 16: 2.7 / 6.3 /
+// 11.2 / 32.7 (one block per graph: 10.7 / 19.7 / 23.6 / 42.8).
 constexpr int kSetCluster = 8;
 
 // A round's work: graphs items[0..large) for the clusters, items[large..count) for
