@@ -134,7 +134,7 @@ def _round_seconds(P, count):  # noqa: F811
 
 def test_small_graphs_alike_are_not_queued_for_clusters(P):  # noqa: F811
     """300 small graphs of one size fit one block each: a round of them takes no longer than
-    one of 600 (eight queues' waves of clusters took 2.4 times as long; now 0.6 times)."""
+    one of 600 (queued for clusters, eight of them one after another, it took 2.4 times as long; now 0.6 times)."""
     assert _round_seconds(P, 300) < 1.4 * _round_seconds(P, 600)
 
 
