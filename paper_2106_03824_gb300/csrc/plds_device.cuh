@@ -1806,7 +1806,8 @@ __device__ __forceinline__ void ins_phase_work(Team &T, const GraphCtx &g, const
         a.upv += up_v;
         const bool again = have && ins_finish_mover(g, it.x, up_v, cnt_l, l, fcur, fnext, cut_next);
         ff_note(st, again, up_v - cnt_l, ideg);
-        enqueue_ins(g, st, again, it.x, have ? 1 << it.y : 0, (int64_t)it.z * 4, -1, 0, 0, k + 1, wsm);
+        // (the next phase's thread cutoff may be lower: room for an up-list as from a chunk scan)
+        enqueue_ins(g, st, again, it.x, have ? 1 << it.y : 0, (int64_t)it.z * 4, -1, 0, up_v - cnt_l, k + 1, wsm);
     }
     // as many items per warp step as the list gives each warp: the step's instructions, not
     // its loads, set the time of a phase in which a warp has one item

@@ -57,6 +57,36 @@ def test_batches_of_uneven_size(P, name, sizes):  # noqa: F811
     g.close()
 
 
+@pytest.mark.parametrize("list_cap", [4, 8, 16, 32, 33])
+@pytest.mark.parametrize("graph", ["rmat", "power"])
+def test_short_up_lists_with_the_cutoff_by_phase(P, graph, list_cap):  # noqa: F811
+    """A climbing vertex scanned by a thread in one phase and, the next phase's cutoff being
+    lower, by a warp in the next gets an up-list when its table has list_cap slots: the list
+    needs room for its up-degree (it had none, and lists overwrote one another)."""
+    if graph == "rmat":
+        n, e = 1_024, W.shuffled(W.rmat(10, 12, seed=488236076), 2)
+    else:
+        n, e = GRAPHS["power"]()
+    g, o = P.PLDS(n, delta=0.2), O.OraclePLDS(n, delta=0.2)
+    g.set_tuning(list_cap=list_cap)
+    sizes = [2_887, 39, 362, 14, 3_074]
+    at = 0
+    for k, b in enumerate(sizes + [e.shape[0] - sum(sizes)]):
+        part = np.ascontiguousarray(e[at: at + b])
+        at += b
+        g.insert(part)
+        assert o.insert(part) == 0
+        assert_same(g, o, f"batch {k}")
+        assert_stats(g, o, f"batch {k}")
+        if k == 1:
+            back = np.ascontiguousarray(e[: at: 50])
+            for x in (g, o):
+                x.delete(back)
+                x.insert(back)
+            assert_same(g, o, "put back")
+    g.close()
+
+
 def test_deletions_with_a_narrowed_window(P):  # noqa: F811
     """Deletion batches of a road-like graph that leave more than 4,096 vertices pending over
     many levels: the near window is narrowed, the rest is sent to the far list and comes back
