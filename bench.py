@@ -54,7 +54,7 @@ UNIT = "updates/s"
 # DRAM bytes per algorithmic byte, from an ncu counter capture of the timed steps'
 # kernels (profiles/traffic_rmat20_B1e6.md); valid only for the kernel sources it was
 # taken on (kernel_sha), otherwise `traffic` is reported as null.
-NCU_TRAFFIC = {"kernel_sha": "d9ea8a5fdbc86212", "rounds_dram_per_algo_byte": 0.713,
+NCU_TRAFFIC = {"kernel_sha": "c2eedaca519d5fbe", "rounds_dram_per_algo_byte": 0.713,
                "batch_dram_per_algo_byte": 2.173,
                "capture": "ncu DRAM counters of every kernel of the timed steps of the R-MAT 20 stream, "
                           "Ins 14-15 and Del 0-1 (profiles/traffic_rmat20_B1e6.md)"}
